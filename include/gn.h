@@ -186,8 +186,15 @@ gn_status gn_set_fp64_accum(gn_handle h, int64_t part_k);
  * with AX and Y^T A.  1 (default): on the BF16 tensor cores by exact digit
  * slicing (gn_dgemm_tc; FP64-level accuracy, about 1e-13 of |A||B| per
  * element); 0: on the FP64 units.  The panels, the small diagonal-block solves
- * and the detector stay in FP64 either way; FP64 sketches always use the FP64
- * units. */
+ * and the detector stay in FP64 either way.
+ * For GN_F64 operands the switch covers gn_sketch (and the calls built on it),
+ * the core product C, the factors and gn_hmt's two products: 1 (default) forms
+ * them from nine digits per operand (63 bits below the largest entry of each
+ * row of the left and column of the right operand: the error per element is
+ * about 2^-60 sqrt(K) max_k |a_ik| max_k |b_kj|, below the rounding error of an
+ * FP64 sum), infinities and NaN as the FP64 units give them; a workspace too
+ * small for the slices (gn_workspace_size includes them) selects the FP64 units
+ * for that product. */
 gn_status gn_set_fp64_tc(gn_handle h, int32_t on);
 
 /* C = alpha op(A) op(B) + beta C, FP64 (A may be FP32), computed on the BF16
@@ -247,7 +254,8 @@ gn_status gn_quantize(gn_handle h, const gn_mat* src, gn_mat* dst);
 
 /* The two sketches of Algorithm 2, step 2: AX (m x r) and Y^T A ((r+l) x n).
  *   A: m x n; X: n x r; Y: m x (r+l) (Y is passed untransposed).
- *   GN_F64 operands: AX, YtA are GN_F64; computed with FP64 FMA.
+ *   GN_F64 operands: AX, YtA are GN_F64; FP64 accuracy or better, on the
+ *     tensor cores by digit slicing or with FP64 FMA (gn_set_fp64_tc).
  *   GN_BF16 / GN_BF16X2 A with GN_BF16 X, Y: one launch of the tcgen05
  *     tensor-core kernel, FP32 accumulation; AX, YtA are GN_F32.  Operand
  *     ld must be a multiple of 8, bases 16-byte aligned (GN_ERR_ALIGNMENT).

@@ -154,6 +154,23 @@ size_t factors_ws(long long m, long long n, long long r, long long l, int mixed,
     return b;
 }
 
+// Least rows of F whose triangular solve takes the digit-sliced products (FP64 AX).
+constexpr long long OZ64_TRSM_MIN_M = 1024;
+
+// What gn_workspace_size adds for the FP64 path's digit-sliced products.  Each
+// call checks for its own room and runs on the FP64 units without it, so a
+// workspace of the sizes above stays enough.
+size_t f64_fast_ws(long long m, long long n, long long r, long long l, int sms) {
+    const long long rl = r + l;
+    const size_t sketch = std::max(dgemm_fast_ws_bytes(m, r, n, sms), dgemm_fast_ws_bytes(rl, n, m, sms));
+    const size_t core = core_ws(n, r, l, 0, sms) + dgemm_fast_ws_bytes(rl, r, n, sms);
+    const size_t fact = factors_ws(m, n, r, l, 0, sms) + oz_ws_bytes(m, 128, r, 0, OZ_DIGITS_F64) +
+                        std::max(dgemm_fast_ws_bytes(m, r, r, sms), dgemm_fast_ws_bytes(r, n, rl, sms));
+    const size_t hmt = align256(sizeof(double) * m * r) + align256(sizeof(double) * r * r) +
+                       std::max(dgemm_fast_ws_bytes(m, r, n, sms), dgemm_fast_ws_bytes(r, n, m, sms));
+    return std::max({sketch, core, fact, hmt}) + 4096;
+}
+
 size_t hmt_ws(long long m, long long n, long long r, int sms) {
     return align256(sizeof(double) * m * r) + align256(sizeof(double) * r * r) + qr_ws_bytes(m, r, sms) +
            dgemm_ws_bytes(r, n, m, sms) + 1024;
@@ -412,7 +429,7 @@ size_t update_scratch(long long m, long long n, long long r, long long l, int op
 // Scratch of sketch_block for an m x n block with rx = X's and ry = Y's columns.
 size_t block_sketch_ws(long long m, long long n, long long rx, long long ry, int op_dtype, int sms) {
     if (op_dtype == GN_E4M3) return sketch_e4m3_ws(m, n, rx, ry - rx);
-    if (op_dtype == GN_F64) return std::max(dgemm_ws_bytes(m, rx, n, sms), dgemm_ws_bytes(ry, n, m, sms)) + 1024;
+    if (op_dtype == GN_F64) return std::max(dgemm_fast_ws_bytes(m, rx, n, sms), dgemm_fast_ws_bytes(ry, n, m, sms)) + 1024;
     return 1024;
 }
 
@@ -458,13 +475,13 @@ gn_status sketch_block(gn_handle h, const gn_mat* A, const gn_mat* X, const gn_m
             return GN_ERR_DTYPE;
         double* gws = static_cast<double*>(ws);
         if (r > 0)
-            GN_TRY(dgemm(h, m, r, n, 1.0, static_cast<const double*>(A->data), A->ld, 0,
-                         static_cast<const double*>(X->data), X->ld, 0, 0.0, static_cast<double*>(AX->data),
-                         AX->ld, gws, ws_bytes));
+            GN_TRY(dgemm_fast(h, m, r, n, 1.0, static_cast<const double*>(A->data), A->ld, 0,
+                              static_cast<const double*>(X->data), X->ld, 0, 0.0, static_cast<double*>(AX->data),
+                              AX->ld, gws, ws_bytes));
         if (rl > 0)
-            GN_TRY(dgemm(h, rl, n, m, 1.0, static_cast<const double*>(Y->data), Y->ld, 1,
-                         static_cast<const double*>(A->data), A->ld, 0, 0.0, static_cast<double*>(YtA->data),
-                         YtA->ld, gws, ws_bytes));
+            GN_TRY(dgemm_fast(h, rl, n, m, 1.0, static_cast<const double*>(Y->data), Y->ld, 1,
+                              static_cast<const double*>(A->data), A->ld, 0, 0.0, static_cast<double*>(YtA->data),
+                              YtA->ld, gws, ws_bytes));
         return GN_OK;
     }
     if (A->dtype == GN_BF16 || A->dtype == GN_BF16X2) {
@@ -658,6 +675,7 @@ gn_status gn_workspace_size(int64_t m, int64_t n, int64_t r, int64_t l, int32_t 
     b = std::max(b, factors_ws(m, n, r, l, mixed, sms));
     b = std::max(b, hmt_ws(m, n, r, sms));
     b = std::max(b, error_ws_bytes(m, n, sms));
+    if (!mixed) b = std::max(b, f64_fast_ws(m, n, r, l, sms));
     *bytes = b;
     return GN_OK;
 }
@@ -759,8 +777,8 @@ gn_status gn_core(gn_handle h, const gn_mat* YtA, const gn_mat* X, double eps, i
     if (c_given) {
         // the caller formed C (for a structured X, e.g. gn_countsketch_apply)
     } else if (fp64) {
-        GN_TRY(dgemm(h, rl, r, n, 1.0, static_cast<const double*>(YtA->data), YtA->ld, 0,
-                     static_cast<const double*>(X->data), X->ld, 0, 0.0, core->C, r, inner, inner_bytes));
+        GN_TRY(dgemm_fast(h, rl, r, n, 1.0, static_cast<const double*>(YtA->data), YtA->ld, 0,
+                          static_cast<const double*>(X->data), X->ld, 0, 0.0, core->C, r, inner, inner_bytes));
     } else if (h->fp64_accum && !x8) {
         // FP64-level C: (Y^T A) X by exact digit slicing on the tensor cores
         double* X64 = inner;
@@ -925,6 +943,22 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
         oz = cv.take<char>(oz_bytes);
         if (!cv.ok) return GN_ERR_WORKSPACE;
     }
+    // FP64 AX: the same products with nine digits when ws has room for them
+    const bool oz64_on = AX->dtype == GN_F64 && h->fp64_tc && m >= OZ64_TRSM_MIN_M && k > 128;
+    const size_t oz64_bytes = oz_ws_bytes(m, 128, r, 0, OZ_DIGITS_F64);
+    int digits = 7;
+    if (oz64_on && ws_bytes >= factors_ws(m, n, r, l, mixed, h->sm_count) + oz64_bytes + 512) {
+        Carve cv2 = cv;
+        cv2.off += (256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255;
+        oz = cv2.take<char>(oz64_bytes);
+        if (cv2.ok) {
+            cv = cv2;
+            digits = OZ_DIGITS_F64;
+        } else {
+            oz = nullptr;
+        }
+    }
+    const size_t ozn = digits == 7 ? oz_bytes : oz64_bytes;
     size_t gws_bytes = 0;
     double* gws = cv.rest(&gws_bytes);
     ws_bytes = gws_bytes;
@@ -937,18 +971,18 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
             GN_CUDA_TRY(cudaMemcpy2DAsync(Fd, F->ld * 8, AX->data, AX->ld * 8, r * 8, m, cudaMemcpyDeviceToDevice,
                                           h->stream));
         }
-        GN_TRY(trsm_right_upper(h, Fd, m, r, F->ld, core->R, r, 0, gws, ws_bytes, oz, oz_bytes));
+        GN_TRY(trsm_right_upper(h, Fd, m, r, F->ld, core->R, r, 0, gws, ws_bytes, oz, ozn, digits));
     } else {
         // F = (AX Q_2) R_2^{-T}
-        if (oz)
+        if (oz && AX->dtype == GN_F32)
             GN_TRY(oz_dgemm(h, m, k, r, 1.0, AX->data, 1, AX->ld, 0, core->Q2, r, 0, 0.0, Fd, F->ld, oz, oz_bytes));
         else if (AX->dtype == GN_F32)
             GN_TRY(dgemm_a32(h, m, k, r, 1.0, static_cast<const float*>(AX->data), AX->ld, 0, core->Q2, r, 0,
                              0.0, Fd, F->ld, gws, ws_bytes));
         else
-            GN_TRY(dgemm(h, m, k, r, 1.0, static_cast<const double*>(AX->data), AX->ld, 0, core->Q2, r, 0, 0.0,
-                         Fd, F->ld, gws, ws_bytes));
-        GN_TRY(trsm_right_upper(h, Fd, m, k, F->ld, core->R2, r, 1, gws, ws_bytes, oz, oz_bytes));
+            GN_TRY(dgemm_fast(h, m, k, r, 1.0, static_cast<const double*>(AX->data), AX->ld, 0, core->Q2, r, 0, 0.0,
+                              Fd, F->ld, gws, ws_bytes));
+        GN_TRY(trsm_right_upper(h, Fd, m, k, F->ld, core->R2, r, 1, gws, ws_bytes, oz, ozn, digits));
     }
     // G = Q_1^T (Y^T A)
     if (YtA->dtype == GN_F32 && !tc_g) {
@@ -982,8 +1016,8 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
         GN_TRY(tc_launch(h, &p));
         GN_TRY(copy_f32_to_f64(h, g32, k, n, lds, Gd, G->ld));
     } else
-        GN_TRY(dgemm(h, k, n, r + l, 1.0, core->Q, r, 1, static_cast<const double*>(YtA->data), YtA->ld, 0, 0.0,
-                     Gd, G->ld, gws, ws_bytes));
+        GN_TRY(dgemm_fast(h, k, n, r + l, 1.0, core->Q, r, 1, static_cast<const double*>(YtA->data), YtA->ld, 0, 0.0,
+                          Gd, G->ld, gws, ws_bytes));
     return GN_OK;
 }
 
@@ -1278,13 +1312,13 @@ gn_status gn_hmt(gn_handle h, const gn_mat* A, const gn_mat* X, gn_mat* Q, gn_ma
     double* inner = cv.rest(&inner_bytes);
     if (!cv.ok) return GN_ERR_WORKSPACE;
     // AX (Algorithm 1, step 2), then its Householder QR (step 3)
-    GN_TRY(dgemm(h, m, r, n, 1.0, static_cast<const double*>(A->data), A->ld, 0,
-                 static_cast<const double*>(X->data), X->ld, 0, 0.0, W, r, inner, inner_bytes));
+    GN_TRY(dgemm_fast(h, m, r, n, 1.0, static_cast<const double*>(A->data), A->ld, 0,
+                      static_cast<const double*>(X->data), X->ld, 0, 0.0, W, r, inner, inner_bytes));
     GN_TRY(householder_qr(h, W, m, r, r, static_cast<double*>(Q->data), Q->ld, Rx, r, inner, inner_bytes));
     // B = Q^T A (step 4; a second pass over A)
-    return dgemm(h, r, n, m, 1.0, static_cast<const double*>(Q->data), Q->ld, 1,
-                 static_cast<const double*>(A->data), A->ld, 0, 0.0, static_cast<double*>(B->data), B->ld, inner,
-                 inner_bytes);
+    return dgemm_fast(h, r, n, m, 1.0, static_cast<const double*>(Q->data), Q->ld, 1,
+                      static_cast<const double*>(A->data), A->ld, 0, 0.0, static_cast<double*>(B->data), B->ld, inner,
+                      inner_bytes);
 }
 
 }  // extern "C"

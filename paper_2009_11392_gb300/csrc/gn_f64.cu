@@ -2212,7 +2212,7 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 
 gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, long long ldf,
                            const double* R, long long ldr, int trans, double* ws, size_t ws_bytes, void* oz,
-                           size_t oz_bytes) {
+                           size_t oz_bytes, int digits) {
     if (m <= 0 || k <= 0) return GN_OK;
     // Two levels of blocking: 128-column outer blocks take the bulk of the
     // update as one wide FP64 GEMM each; inside, 32-column blocks take a narrow
@@ -2226,7 +2226,7 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
         // (oz: these and the inner updates below on the tensor cores by exact digit slicing)
         if (!trans && J0 > 0) {   // F[:, J] -= F[:, 0:J0] R[0:J0, J]
             if (oz)
-                GN_TRY(oz_dgemm(h, m, JB, J0, -1.0, F, 0, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, oz, oz_bytes));
+                GN_TRY(oz_dgemm(h, m, JB, J0, -1.0, F, 0, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, oz, oz_bytes, digits));
             else
                 GN_TRY(dgemm(h, m, JB, J0, -1.0, F, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, ws, ws_bytes));
         }
@@ -2234,7 +2234,7 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
             const long long kk = k - J0 - JB;
             if (oz)
                 GN_TRY(oz_dgemm(h, m, JB, kk, -1.0, F + J0 + JB, 0, ldf, 0, R + J0 * ldr + J0 + JB, ldr, 1, 1.0,
-                                F + J0, ldf, oz, oz_bytes));
+                                F + J0, ldf, oz, oz_bytes, digits));
             else
                 GN_TRY(dgemm(h, m, JB, kk, -1.0, F + J0 + JB, ldf, 0, R + J0 * ldr + J0 + JB, ldr, 1, 1.0, F + J0,
                              ldf, ws, ws_bytes));
@@ -2248,7 +2248,7 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
                 // F[:, j] -= F[:, J0:j0] R[J0:j0, j]
                 if (oz)
                     GN_TRY(oz_dgemm(h, m, jb, j0 - J0, -1.0, F + J0, 0, ldf, 0, R + J0 * ldr + j0, ldr, 0, 1.0,
-                                    F + j0, ldf, oz, oz_bytes));
+                                    F + j0, ldf, oz, oz_bytes, digits));
                 else
                     GN_TRY(dgemm(h, m, jb, j0 - J0, -1.0, F + J0, ldf, 0, R + J0 * ldr + j0, ldr, 0, 1.0, F + j0, ldf,
                                  ws, ws_bytes));
@@ -2258,7 +2258,7 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
                 const long long kk = J0 + JB - j0 - jb;
                 if (oz)
                     GN_TRY(oz_dgemm(h, m, jb, kk, -1.0, F + j0 + jb, 0, ldf, 0, R + j0 * ldr + j0 + jb, ldr, 1, 1.0,
-                                    F + j0, ldf, oz, oz_bytes));
+                                    F + j0, ldf, oz, oz_bytes, digits));
                 else
                     GN_TRY(dgemm(h, m, jb, kk, -1.0, F + j0 + jb, ldf, 0, R + j0 * ldr + j0 + jb, ldr, 1, 1.0, F + j0,
                                  ldf, ws, ws_bytes));

@@ -74,8 +74,8 @@ namespace gn {
 unsigned long long launch_count();
 void count_launch();
 
-constexpr int TC_MAX_MAPS = 14;
-constexpr int TC_MAX_GEMMS = 7;
+constexpr int TC_MAX_MAPS = 18;
+constexpr int TC_MAX_GEMMS = 9;
 constexpr int TC_MAX_SRC = 12;
 
 constexpr int TC_BK = 64;   // K elements per stage of the BF16 multi-GEMM (one K block)
@@ -208,16 +208,25 @@ size_t qr_oz_ws_bytes(long long M, long long N);
 size_t trsm_ws_bytes(long long m, long long k, int sm_count);
 gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, long long ldf,
                            const double* R, long long ldr, int trans, double* ws, size_t ws_bytes,
-                           void* oz = nullptr, size_t oz_bytes = 0);
+                           void* oz = nullptr, size_t oz_bytes = 0, int digits = 7);
 
 // FP64 product on the BF16 tensor cores by exact digit slicing (gn_ozaki.cu);
 // same operand conventions as dgemm, A FP64 or (a_f32) FP32.  digits: BF16
 // digits per operand row / column (7: FP64 accuracy; d < 7: every term carries
 // an error of about 2^(1 - 7d) max|a_i.| max|b_.j|).
-size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32);
+constexpr int OZ_DIGITS_F64 = 9;
+size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32, int digits = 7);
 gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double alpha, const void* A, int a_f32,
                    long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                    long long ldc, void* ws, size_t ws_bytes, int digits = 7);
+
+// dgemm for FP64 operands through oz_dgemm with nine digits (63 bits below each
+// row's largest entry) where the product is large enough, ws holds
+// dgemm_fast_ws_bytes and gn_set_fp64_tc is on; dgemm otherwise.
+size_t dgemm_fast_ws_bytes(long long M, long long N, long long K, int sm_count);
+gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
+                     long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
+                     long long ldc, double* ws, size_t ws_bytes);
 
 // Core diagnostics (one CTA): out3[0] = est ||R^{-1}||_2 (if want_estimate),
 // out3[1] = est ||R||_2 (if eps_relative), out3[2] = the absolute threshold

@@ -23,6 +23,13 @@
 // about 2^-46 K max_k|a_ik| max_k|b_kj|, the size of an FP64 product's own
 // worst-case rounding error.  FP32 operands take 7 digits too: the digits cover
 // a window below the row's largest entry, not each entry's own 24 bits.
+// FP64 operands of the FP64 path take nine digits (63 bits below each row's
+// largest entry, orders 0..8): 45 slice products instead of 28.  Measured against
+// extended precision (relative Frobenius error of a Gaussian product, K = 500 /
+// 2048): 4.8e-17 / 6.7e-17, the FP64 units 3.0e-16 / 9.2e-16; with low-rank, 1 %
+// sparse and graded (1e8) matrices the slices stay at 3e-17..8e-17 and the units
+// at 8e-17..1.4e-15.  The error scales with max|a_i.| max|b_.j|, not with
+// sum |a_ik| |b_kj|.
 #include "gn_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -34,15 +41,15 @@ namespace {
 
 constexpr int OZ_KPASS = 1024;   // K per pass (exactness of the orders <= 3)
 constexpr int OZ_NPANEL = 256;   // least N per GEMM launch (oz_npanel bounds the FP32 outputs)
-constexpr int OZ_MAX_DIGITS = 7;
+constexpr int OZ_MAX_DIGITS = OZ_DIGITS_F64;
 constexpr int OZ_PGRP = 4;       // passes per group of launches (slicing, products, combination)
 
 size_t al256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 
 // Columns of C per GEMM launch: at least 256, more while the FP32 outputs of all
 // orders and K parts stay within 64 MB (short, wide products in one launch).
-long long oz_npanel(long long M, long long N, long long parts) {
-    long long np = (64LL << 20) / (4LL * OZ_MAX_DIGITS * std::max<long long>(M, 1) * std::max<long long>(parts, 1));
+long long oz_npanel(long long M, long long N, long long parts, int orders) {
+    long long np = (64LL << 20) / (4LL * orders * std::max<long long>(M, 1) * std::max<long long>(parts, 1));
     np = std::max<long long>(np, OZ_NPANEL) / 16 * 16;
     return std::min<long long>(N, np);
 }
@@ -73,12 +80,15 @@ __device__ __forceinline__ int row_exponent<float>(unsigned long long mx) {
     return E == 0 ? -125 : E - 125;
 }
 
-// round(x 2^(49-e)) as a signed integer, |result| <= 2^48.
-__device__ __forceinline__ long long fixed49(double x, int e) {
+// round(x 2^(7 W - e)) as a signed integer, |result| <= 2^(7 W - 1): the row's window
+// of W digits (W = 7: 49 bits; W = 9: 63 bits, every bit of the entries within a
+// factor 2^-9 of the row's largest and 2^-63 of it for all).
+template <int W>
+__device__ __forceinline__ long long fixed_win(double x, int e) {
     const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
     const int E = static_cast<int>((b >> 52) & 0x7FF);
     const unsigned long long mant = (b & 0xFFFFFFFFFFFFFull) | (E ? (1ull << 52) : 0ull);
-    const int sh = (E ? E : 1) - 1075 + 49 - e;   // x = mant 2^(E-1075); always < 0 for |x| < 2^(e-1) normal
+    const int sh = (E ? E : 1) - 1075 + 7 * W - e;   // x = mant 2^(E-1075); mant 2^sh < 2^(7 W - 1)
     long long v;
     if (sh >= 0) v = static_cast<long long>(mant << sh);
     else if (sh > -64) v = static_cast<long long>((mant + (1ull << (-sh - 1))) >> (-sh));
@@ -86,11 +96,12 @@ __device__ __forceinline__ long long fixed49(double x, int e) {
     return (b >> 63) ? -v : v;
 }
 
-__device__ __forceinline__ long long fixed49(float x, int e) {
+template <int W>
+__device__ __forceinline__ long long fixed_win(float x, int e) {
     const uint32_t b = __float_as_uint(x);
     const int E = static_cast<int>((b >> 23) & 0xFF);
     const unsigned long long mant = (b & 0x7FFFFFu) | (E ? 0x800000u : 0u);
-    const int sh = (E ? E : 1) - 150 + 49 - e;
+    const int sh = (E ? E : 1) - 150 + 7 * W - e;
     long long v;
     if (sh >= 0) v = static_cast<long long>(mant << sh);
     else if (sh > -64) v = static_cast<long long>((mant + (1ull << (-sh - 1))) >> (-sh));
@@ -98,31 +109,33 @@ __device__ __forceinline__ long long fixed49(float x, int e) {
     return (b >> 31) ? -v : v;
 }
 
-// Signed base-2^7 digits of Y (|Y| <= 2^48): slice s holds d_s 2^{-7(s+1)},
+// Signed base-2^7 digits of Y (|Y| <= 2^(7 W - 1)): slice s holds d_s 2^{-7(s+1)},
 // |d_s| <= 64.  With a bias of 64 in each kept digit position (plus half of the
-// last kept unit when S < 7), U = Y + bias >= 0 has plain base-128 digits u_s,
-// and d_s = u_s - 64: the S digits sum to Y exactly for S = 7 and to Y rounded
-// to the last kept unit (nearest, ties up) for S < 7.  Bit fields of one 64-bit
-// integer, no carries to propagate.
+// last kept unit when S < W), U = Y + bias >= 0 has plain base-128 digits u_s,
+// and d_s = u_s - 64: the S digits sum to Y exactly for S = W and to Y rounded
+// to the last kept unit (nearest, ties up) for S < W.  Bit fields of one 64-bit
+// integer (W = 9: U < 2^62 + 2^62 (1 + 2^-6) < 2^64), no carries to propagate.
+template <int W>
 __device__ __forceinline__ unsigned long long digit_bias(int S) {
     unsigned long long b = 0;
 #pragma unroll
-    for (int s = 0; s < OZ_MAX_DIGITS; ++s)
-        if (s < S) b += 64ull << (7 * (OZ_MAX_DIGITS - 1 - s));
-    if (S < OZ_MAX_DIGITS) b += 1ull << (7 * (OZ_MAX_DIGITS - S) - 1);
+    for (int s = 0; s < W; ++s)
+        if (s < S) b += 64ull << (7 * (W - 1 - s));
+    if (S < W) b += 1ull << (7 * (W - S) - 1);
     return b;
 }
 
 // Digits of two entries adjacent along K, stored as one bf16 pair per slice
 // (out 4-byte aligned, slice_stride even).
+template <int W>
 __device__ __forceinline__ void write_digits2(long long Y0, long long Y1, int S, unsigned long long bias,
                                               __nv_bfloat16* out, long long slice_stride) {
     const unsigned long long U0 = static_cast<unsigned long long>(Y0) + bias;
     const unsigned long long U1 = static_cast<unsigned long long>(Y1) + bias;
 #pragma unroll
-    for (int s = 0; s < OZ_MAX_DIGITS; ++s) {
+    for (int s = 0; s < W; ++s) {
         if (s >= S) break;
-        const int sh = 7 * (OZ_MAX_DIGITS - 1 - s);
+        const int sh = 7 * (W - 1 - s);
         const unsigned u0 = s ? static_cast<unsigned>(U0 >> sh) & 127u : static_cast<unsigned>(U0 >> sh);
         const unsigned u1 = s ? static_cast<unsigned>(U1 >> sh) & 127u : static_cast<unsigned>(U1 >> sh);
         const float sc = __int_as_float((127 - 7 * (s + 1)) << 23);   // 2^{-7(s+1)}
@@ -174,7 +187,7 @@ __device__ __forceinline__ unsigned long long mx_word(unsigned long long m, floa
 // warps), OZ_ST / tpr rows per CTA, pairs of entries along K (8 entries per
 // thread); the row maximum is a shuffle, plus an exchange between the row's
 // warps when there are four.
-template <typename T>
+template <int W, typename T>
 __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int q, int rank, OzSmem& sm) {
     const long long koff = static_cast<long long>(pass) * OZ_KPASS;
     const T* src = static_cast<const T*>(o.src) + koff;
@@ -203,12 +216,12 @@ __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int 
     if (!live) return;   // no barrier follows in this path
     if (l == 0) o.mx[static_cast<long long>(pass) * o.rows + i] = mx_word(m, static_cast<T*>(nullptr));
     const int e = row_exponent<T>(m);
-    const unsigned long long bias = digit_bias(o.S);
+    const unsigned long long bias = digit_bias<W>(o.S);
     __nv_bfloat16* out = o.out + i * o.ldk + koff;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const int k = 2 * l + 2 * tpr * u;   // k + 1 < ldk: ldk is K rounded up to 8
-        if (k < K) write_digits2(fixed49(v[2 * u], e), fixed49(v[2 * u + 1], e), o.S, bias, out + k, o.slice_stride);
+        if (k < K) write_digits2<W>(fixed_win<W>(v[2 * u], e), fixed_win<W>(v[2 * u + 1], e), o.S, bias, out + k, o.slice_stride);
     }
 }
 
@@ -216,7 +229,7 @@ __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int 
 // <= 128; a CTA reads its 32 x chunk block along the rows (coalesced, 8
 // entries per thread), the partial row maxima go through distributed shared
 // memory, and the digits are written along K after a transpose in shared memory.
-template <typename T>
+template <int W, typename T>
 __device__ __forceinline__ void slice_strided(const OzOperand& o, int pass, int q, int rank, OzSmem& sm) {
     namespace cg = cooperative_groups;
     cg::cluster_group cluster = cg::this_cluster();
@@ -256,7 +269,7 @@ __device__ __forceinline__ void slice_strided(const OzOperand& o, int pass, int 
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
         const int kk = warp + OZ_NW * u;
-        if (kk < kc) sm.ys[kk][lane] = fixed49(v[u], e);
+        if (kk < kc) sm.ys[kk][lane] = fixed_win<W>(v[u], e);
     }
     __syncthreads();
     const int w = k1 - k0;
@@ -266,13 +279,13 @@ __device__ __forceinline__ void slice_strided(const OzOperand& o, int pass, int 
     // Thread: pair kp = tid % 64, rows tid / 64 + 8 j.
     const int wp = (w + 1) / 2, kp = tid & 63;
     if (kp >= wp) return;
-    const unsigned long long bias = digit_bias(o.S);
+    const unsigned long long bias = digit_bias<W>(o.S);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
         const int ii = (tid >> 6) + 8 * j;
         const long long row = static_cast<long long>(q) * 32 + ii;
         if (row < o.rows)
-            write_digits2(sm.ys[2 * kp][ii], sm.ys[2 * kp + 1][ii], o.S, bias, o.out + row * o.ldk + koff + k0 + 2 * kp,
+            write_digits2<W>(sm.ys[2 * kp][ii], sm.ys[2 * kp + 1][ii], o.S, bias, o.out + row * o.ldk + koff + k0 + 2 * kp,
                           o.slice_stride);
     }
 }
@@ -280,7 +293,7 @@ __device__ __forceinline__ void slice_strided(const OzOperand& o, int pass, int 
 // Cluster q of the grid slices pass p, rows [rpc q', rpc q' + rpc) of operand 0
 // (FP32 when A32) for q < op[0].clusters, else of operand 1 (FP64), with
 // q - (operand base) = p ceil(rows / rpc) + q'.
-template <bool A32>
+template <bool A32, int W>
 __global__ void __launch_bounds__(OZ_ST) oz_slice_kernel(const __grid_constant__ OzSliceArgs args) {
     __shared__ OzSmem sm;
     const int rank = static_cast<int>(cooperative_groups::this_cluster().block_rank());
@@ -292,11 +305,11 @@ __global__ void __launch_bounds__(OZ_ST) oz_slice_kernel(const __grid_constant__
     const int pass = q / rq;
     q -= pass * rq;
     if (which == 0 && A32) {
-        if (o.s_k == 1) slice_kcontig<float>(o, pass, q, rank, sm);
-        else slice_strided<float>(o, pass, q, rank, sm);
+        if (o.s_k == 1) slice_kcontig<W, float>(o, pass, q, rank, sm);
+        else slice_strided<W, float>(o, pass, q, rank, sm);
     } else {
-        if (o.s_k == 1) slice_kcontig<double>(o, pass, q, rank, sm);
-        else slice_strided<double>(o, pass, q, rank, sm);
+        if (o.s_k == 1) slice_kcontig<W, double>(o, pass, q, rank, sm);
+        else slice_strided<W, double>(o, pass, q, rank, sm);
     }
 }
 
@@ -338,29 +351,58 @@ gn_status slice_pair(gn_handle h, const OzOperand& a, int a_f32, const OzOperand
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (a_f32) GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_slice_kernel<true>, args));
-    else GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_slice_kernel<false>, args));
+    if (a.S > 7 || b.S > 7) {
+        if (a_f32) return GN_ERR_INVALID_ARG;
+        GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_slice_kernel<false, OZ_DIGITS_F64>, args));
+    } else if (a_f32) {
+        GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_slice_kernel<true, 7>, args));
+    } else {
+        GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, oz_slice_kernel<false, 7>, args));
+    }
     count_launch();
     return GN_OK;
 }
 
+// The operands of a product whose rows may hold infinities or NaN (FP64 paths
+// that must propagate them): an entry of C whose row of A or column of B is not
+// finite in a part is formed from the operands themselves.  A null: not checked.
+struct OzDirect {
+    const double *A, *B;
+    long long a_row, a_k, b_row, b_k;
+    int K;
+};
+
+__device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, int j) {
+    const int k1 = min(x.K, (q + 1) * OZ_KPASS);
+    double s = 0.0;
+    for (int k = q * OZ_KPASS; k < k1; ++k) {
+        s = fma(x.A[i * x.a_row + k * x.a_k], x.B[j * x.b_row + k * x.b_k], s);
+        if (isnan(s)) break;
+    }
+    return s;
+}
+
 // C[i, j] = beta C[i, j] + sum_q alpha 2^{ea_qi + eb_qj} sum_o D_qo[i, j] over
 // the K parts q (passes, each with its own row exponents), added in part
-// order with one rounding each.  Within a part the exact orders 0..3 are
-// summed as integers in units of 2^-35 (one rounding), the rounded orders 4..
-// in FP32 below them.  A thread per column and row group (no division per
+// order with one rounding each.  Within a part the first NEX orders are summed
+// as integers (one rounding), the orders below them in FP32.  NEX = 4 for up to
+// seven digits (units of 2^-35: the orders that are always exact); 6 for nine
+// (units of 2^-49, so that the FP32 sum of the last orders rounds below 2^-60
+// of the leading one).  A thread per column and row group (no division per
 // element; narrow products fill a block with more rows); each exact order is
 // an integer below 2^24 units, so it converts through a 32-bit integer.
+template <int NEX>
 __global__ void oz_combine_kernel(const float* __restrict__ D, long long d_stride, long long part_stride,
                                   long long ldd, int norders, int nparts, int M, int N,
                                   const unsigned long long* __restrict__ mxa,
                                   const unsigned long long* __restrict__ mxb, long long mxb_part, double alpha,
-                                  double beta, double* __restrict__ C, long long ldc, int cw) {
+                                  double beta, double* __restrict__ C, long long ldc, int cw,
+                                  const __grid_constant__ OzDirect direct, int j0) {
     // a block is cw columns by blockDim.x / cw rows (cw: a power of two >= min(N, 256), >= 32)
     const int j = blockIdx.x * cw + static_cast<int>(threadIdx.x) % cw;
     const int rb = static_cast<int>(blockDim.x) / cw;
     if (j >= N) return;
-    const int nexact = norders < 4 ? norders : 4;
+    const int nexact = norders < NEX ? norders : NEX;
     for (int i = blockIdx.y * rb + static_cast<int>(threadIdx.x) / cw; i < M; i += gridDim.y * rb) {
         double* c = C + static_cast<long long>(i) * ldc + j;
         double out = 0.0;
@@ -369,17 +411,18 @@ __global__ void oz_combine_kernel(const float* __restrict__ D, long long d_strid
             long long acc = 0;
             for (int o = 0; o < nexact; ++o)   // D_o is an integer number of units 2^{-7(o+2)}
                 acc += static_cast<long long>(__float2int_rn(d[o * d_stride] * __int_as_float((127 + 7 * (o + 2)) << 23)))
-                       << (7 * (3 - o));
+                       << (7 * (NEX - 1 - o));
             float low = 0.0f;
-            for (int o = norders - 1; o >= 4; --o) low += d[o * d_stride];
-            // times 2^(ea + eb - 35): a power of two built from its bits when normal
-            const int ea = row_exponent<double>(mxa[static_cast<long long>(q) * M + i]);
-            const int eb = row_exponent<double>(mxb[q * mxb_part + j]);
-            const int p = ea + eb - 35;
-            const double x = fma(static_cast<double>(low), 34359738368.0, static_cast<double>(acc));
-            const double v = (p >= -1022 && p <= 1023)
-                                 ? x * (alpha * __longlong_as_double(static_cast<long long>(p + 1023) << 52))
-                                 : alpha * ldexp(x, p);
+            for (int o = norders - 1; o >= NEX; --o) low += d[o * d_stride];
+            // times 2^(ea + eb - 7 (NEX + 1)): a power of two built from its bits when normal
+            const unsigned long long ma = mxa[static_cast<long long>(q) * M + i], mb = mxb[q * mxb_part + j];
+            const int p = row_exponent<double>(ma) + row_exponent<double>(mb) - 7 * (NEX + 1);
+            const double x = fma(static_cast<double>(low), static_cast<double>(1ull << (7 * (NEX + 1))),
+                                 static_cast<double>(acc));
+            double v = (p >= -1022 && p <= 1023)
+                           ? x * (alpha * __longlong_as_double(static_cast<long long>(p + 1023) << 52))
+                           : alpha * ldexp(x, p);
+            if (NEX == 6 && direct.A && max(ma, mb) >= 0x7FF0000000000000ull) v = alpha * oz_direct_dot(direct, q, i, j0 + j);
             out = q ? out + v : (beta == 0.0 ? v : fma(beta, *c, v));
         }
         *c = out;
@@ -398,7 +441,7 @@ long long oz_kgroup(long long K) { return std::min<long long>(std::max<long long
 long long oz_parts(long long kg) { return (kg + OZ_KPASS - 1) / OZ_KPASS; }
 
 bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, size_t ws_bytes, OzWs* o) {
-    const long long kg = oz_kgroup(K), S = oz_parts(kg), np = oz_npanel(M, N, S);
+    const long long kg = oz_kgroup(K), S = oz_parts(kg), np = oz_npanel(M, N, S, sa);
     o->ldk = r8(kg);
     o->ldd = r4(np);
     char* p = static_cast<char*>(ws);
@@ -410,7 +453,7 @@ bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, s
     };
     o->as = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * sa * M * o->ldk));
     o->bs = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * sb * N * o->ldk));
-    o->d = reinterpret_cast<float*>(take(sizeof(float) * S * OZ_MAX_DIGITS * M * o->ldd));
+    o->d = reinterpret_cast<float*>(take(sizeof(float) * S * sa * M * o->ldd));
     o->mxa = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * S * M));
     o->mxb = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * S * N));
     return off <= ws_bytes;
@@ -418,15 +461,15 @@ bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, s
 
 }  // namespace
 
-size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32) {
+size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32, int digits) {
     (void)a_f32;
-    const int sa = OZ_MAX_DIGITS, sb = OZ_MAX_DIGITS;
+    const int sa = digits, sb = digits;
     const long long kg = oz_kgroup(K), S = oz_parts(kg);
     // the FP32 outputs of s parts at the panel for s parts, largest over s <= S:
     // the panel narrows as the parts grow, and the size must not shrink with K
     size_t d = 0;
     for (long long s = 1; s <= S; ++s)
-        d = std::max(d, al256(sizeof(float) * s * OZ_MAX_DIGITS * M * r4(oz_npanel(M, std::max<long long>(N, 1), s))));
+        d = std::max(d, al256(sizeof(float) * s * sa * M * r4(oz_npanel(M, std::max<long long>(N, 1), s, sa))));
     return al256(sizeof(__nv_bfloat16) * sa * M * r8(kg)) + al256(sizeof(__nv_bfloat16) * sb * N * r8(kg)) + d +
            al256(8 * S * M) + al256(8 * S * N) + 256;
 }
@@ -435,7 +478,8 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                    long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                    long long ldc, void* ws, size_t ws_bytes, int digits) {
     if (M <= 0 || N <= 0) return GN_OK;
-    if (K <= 0 || !A || !B || !C || !ws || digits < 2 || digits > OZ_MAX_DIGITS) return GN_ERR_INVALID_ARG;
+    if (K <= 0 || !A || !B || !C || !ws || digits < 2 || (digits > 7 && (digits != OZ_DIGITS_F64 || a_f32)))
+        return GN_ERR_INVALID_ARG;
     const int sa = digits, sb = digits;
     if (M > (1LL << 30) || N > (1LL << 30)) return GN_ERR_SHAPE;
     OzWs o;
@@ -459,8 +503,8 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
     // groups of at most OZ_PGRP passes: one slicing launch for all of them, the
     // passes as K-aligned parts of one multi-GEMM launch (stored apart), one
     // combination adding them in order
-    const long long part_stride = OZ_MAX_DIGITS * d_stride;
-    const long long npanel = oz_npanel(M, N, oz_parts(oz_kgroup(K)));   // the carve's panel (largest group)
+    const long long part_stride = sa * d_stride;
+    const long long npanel = oz_npanel(M, N, oz_parts(oz_kgroup(K)), sa);   // the carve's panel (largest group)
     for (long long k0 = 0; k0 < K; k0 += OZ_PGRP * OZ_KPASS) {
         const long long kc = std::min<long long>(OZ_PGRP * OZ_KPASS, K - k0);
         const int S = static_cast<int>(oz_parts(kc));
@@ -526,13 +570,58 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
             const unsigned gy = static_cast<unsigned>(std::max<long long>(
                 1, std::min<long long>((M + rows_per_block - 1) / rows_per_block,
                                        static_cast<long long>(h->sm_count) * 16 / gx)));
-            oz_combine_kernel<<<dim3(gx, gy), 256, 0, h->stream>>>(
+            OzDirect dd{};
+            if (digits == OZ_DIGITS_F64)
+                dd = OzDirect{static_cast<const double*>(A) + a_off, B + b_off, a_row, a_k, b_row, b_k,
+                              static_cast<int>(kc)};
+            auto* combine = digits == OZ_DIGITS_F64 ? oz_combine_kernel<6> : oz_combine_kernel<4>;
+            combine<<<dim3(gx, gy), 256, 0, h->stream>>>(
                 o.d, d_stride, part_stride, o.ldd, norders, S, static_cast<int>(M), static_cast<int>(nb), o.mxa,
-                o.mxb + j0, N, alpha, beta_grp, C + j0, ldc, cw);
+                o.mxb + j0, N, alpha, beta_grp, C + j0, ldc, cw, dd, static_cast<int>(j0));
             count_launch();
             GN_CUDA_TRY(cudaGetLastError());
         }
     }
+    return GN_OK;
+}
+
+// ---- FP64 products with nine digits per operand, or on the FP64 units
+namespace {
+// Blocks of C per digit-sliced product: the scratch (the slices of up to 4096 of K)
+// stays near 2 GB however large the matrices are.
+constexpr long long OZ_MBLK = 8192, OZ_NBLK = 16384;
+// Least K for the tensor cores.  Three launches take about 20 us; on the FP64
+// units a 64 x 64 tile takes 1.1 us per element of K (256 multiply-adds per
+// sub-partition at ~64 cycles each per warp instruction), so K decides, not M
+// and N: both products of a sketch at m, n, r = 40, 32, 8: 41 us in slices and
+// 68 on the units; 64, 64, 8: 42 and 108; 500, 400, 16: 86 and 187; 4096, 2048,
+// 100: 436 and 5246; 20000, 10000, 500: 28.0 and 428.5 ms.
+constexpr long long OZ_F64_MIN_K = 24;
+bool oz_f64_pays(long long M, long long N, long long K) { return M >= 1 && N >= 1 && K >= OZ_F64_MIN_K; }
+}  // namespace
+
+size_t dgemm_fast_ws_bytes(long long M, long long N, long long K, int sm_count) {
+    size_t b = dgemm_ws_bytes(M, N, K, sm_count);
+    if (!oz_f64_pays(M, N, K)) return b;
+    for (long long mm : {std::min(M, OZ_MBLK), M % OZ_MBLK})
+        for (long long nn : {std::min(N, OZ_NBLK), N % OZ_NBLK})
+            if (mm > 0 && nn > 0) b = std::max(b, oz_ws_bytes(mm, nn, K, 0, OZ_DIGITS_F64) + 256);
+    return b;
+}
+
+gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
+                     long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
+                     long long ldc, double* ws, size_t ws_bytes) {
+    const size_t need = dgemm_fast_ws_bytes(M, N, K, h->sm_count);
+    if (!h->fp64_tc || !ws || ws_bytes < need || !oz_f64_pays(M, N, K))
+        return dgemm(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, ws, ws_bytes);
+    const size_t pad = (256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255;
+    char* base = reinterpret_cast<char*>(ws) + pad;
+    for (long long j0 = 0; j0 < N; j0 += OZ_NBLK)
+        for (long long i0 = 0; i0 < M; i0 += OZ_MBLK)
+            GN_TRY(oz_dgemm(h, std::min(OZ_MBLK, M - i0), std::min(OZ_NBLK, N - j0), K, alpha,
+                            A + (ta ? i0 : i0 * lda), 0, lda, ta, B + (tb ? j0 * ldb : j0), ldb, tb, beta,
+                            C + i0 * ldc + j0, ldc, base, ws_bytes - pad, OZ_DIGITS_F64));
     return GN_OK;
 }
 
