@@ -181,8 +181,8 @@ gn_status gn_set_fp64_accum(gn_handle h, int64_t part_k);
  * factorization runs in 256-column blocks and each block's reflectors update
  * the columns to its right as two products after U = V T; below that, the columns beyond
  * the next two panels of the look-ahead) and the formation of the thin Q; in
- * gn_factors / gn_approx, the outer-block updates of the triangular solve
- * F R = AX (eq. 5.1) and, after a truncation, AX Q_2; in gn_apply, the products
+ * gn_factors / gn_approx, the products of the blocked triangular solve
+ * F R = AX (eq. 5.1; 8 digits per operand) and, after a truncation, AX Q_2; in gn_apply, the products
  * with AX and Y^T A.  1 (default): on the BF16 tensor cores by exact digit
  * slicing (gn_dgemm_tc; FP64-level accuracy, about 1e-13 of |A||B| per
  * element); 0: on the FP64 units.  The panels, the small diagonal-block solves

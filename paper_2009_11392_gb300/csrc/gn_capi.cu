@@ -154,9 +154,6 @@ size_t factors_ws(long long m, long long n, long long r, long long l, int mixed,
     return b;
 }
 
-// Least rows of F whose triangular solve takes the digit-sliced products (FP64 AX).
-constexpr long long OZ64_TRSM_MIN_M = 1024;
-
 // What gn_workspace_size adds for the FP64 path's digit-sliced products.  Each
 // call checks for its own room and runs on the FP64 units without it, so a
 // workspace of the sizes above stays enough.
@@ -164,7 +161,7 @@ size_t f64_fast_ws(long long m, long long n, long long r, long long l, int sms) 
     const long long rl = r + l;
     const size_t sketch = std::max(dgemm_fast_ws_bytes(m, r, n, sms), dgemm_fast_ws_bytes(rl, n, m, sms));
     const size_t core = core_ws(n, r, l, 0, sms) + dgemm_fast_ws_bytes(rl, r, n, sms);
-    const size_t fact = factors_ws(m, n, r, l, 0, sms) + oz_ws_bytes(m, 128, r, 0, OZ_DIGITS_F64) +
+    const size_t fact = factors_ws(m, n, r, l, 0, sms) + trsm_oz_ws_bytes(m, r, OZ_DIGITS_F64) +
                         std::max(dgemm_fast_ws_bytes(m, r, r, sms), dgemm_fast_ws_bytes(r, n, rl, sms));
     const size_t hmt = align256(sizeof(double) * m * r) + align256(sizeof(double) * r * r) +
                        std::max(dgemm_fast_ws_bytes(m, r, n, sms), dgemm_fast_ws_bytes(r, n, m, sms));
@@ -676,6 +673,8 @@ gn_status gn_workspace_size(int64_t m, int64_t n, int64_t r, int64_t l, int32_t 
     b = std::max(b, hmt_ws(m, n, r, sms));
     b = std::max(b, error_ws_bytes(m, n, sms));
     if (!mixed) b = std::max(b, f64_fast_ws(m, n, r, l, sms));
+    // (the factors' own check asks for less: the solve then takes fewer rows at a time)
+    if (mixed) b = std::max(b, factors_ws(m, n, r, l, 1, sms) + trsm_oz_ws_bytes(m, r, OZ_DIGITS_SOLVE));
     *bytes = b;
     return GN_OK;
 }
@@ -929,10 +928,14 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
     const long long rl = r + l, lds = round8(n), ldq = round8(k);
     __nv_bfloat16 *sl[3] = {nullptr, nullptr, nullptr}, *ql[3] = {nullptr, nullptr, nullptr};
     float* g32 = nullptr;
-    // FP32 AX: the solve's large products on the tensor cores (digit slicing)
-    const bool oz_on = AX->dtype == GN_F32 && h->fp64_tc && m >= 1024;
+    // FP32 AX: the solve's products on the tensor cores (digit slicing)
+    const bool oz_on = AX->dtype == GN_F32 && h->fp64_tc;
     void* oz = nullptr;
-    const size_t oz_bytes = oz_on ? factors_oz_ws(m, r) : 0;
+    // at least what the check above asks for, and what ws holds beyond it up to the whole solve
+    const size_t oz_spare = ws_bytes - factors_ws(m, n, r, l, mixed, h->sm_count);
+    const size_t oz_bytes = oz_on ? (std::max(factors_oz_ws(m, r), std::min(factors_oz_ws(m, r) + oz_spare,
+                                                                            trsm_oz_ws_bytes(m, r, OZ_DIGITS_SOLVE))) &
+                                     ~static_cast<size_t>(255)) : 0;
     if (tc_g) {
         for (int i = 0; i < 3; ++i) sl[i] = cv.take<__nv_bfloat16>(rl * lds);
         for (int i = 0; i < 3; ++i) ql[i] = cv.take<__nv_bfloat16>(rl * ldq);
@@ -943,35 +946,23 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
         oz = cv.take<char>(oz_bytes);
         if (!cv.ok) return GN_ERR_WORKSPACE;
     }
-    // FP64 AX: the same products with nine digits when ws has room for them
-    const bool oz64_on = AX->dtype == GN_F64 && h->fp64_tc && m >= OZ64_TRSM_MIN_M && k > 128;
-    const size_t oz64_bytes = oz_ws_bytes(m, 128, r, 0, OZ_DIGITS_F64);
-    int digits = 7;
-    if (oz64_on && ws_bytes >= factors_ws(m, n, r, l, mixed, h->sm_count) + oz64_bytes + 512) {
-        Carve cv2 = cv;
-        cv2.off += (256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255;
-        oz = cv2.take<char>(oz64_bytes);
-        if (cv2.ok) {
-            cv = cv2;
-            digits = OZ_DIGITS_F64;
-        } else {
-            oz = nullptr;
-        }
+    // FP64 AX: the same products with nine digits, in what ws holds beyond the FP64 units' scratch
+    int digits = OZ_DIGITS_SOLVE;
+    size_t ozn = oz_bytes;
+    if (AX->dtype == GN_F64 && h->fp64_tc && ws_bytes > factors_ws(m, n, r, l, mixed, h->sm_count)) {
+        ozn = std::min(ws_bytes - factors_ws(m, n, r, l, mixed, h->sm_count),
+                       trsm_oz_ws_bytes(m, r, OZ_DIGITS_F64)) & ~static_cast<size_t>(255);
+        oz = ozn ? cv.take<char>(ozn) : nullptr;
+        digits = OZ_DIGITS_F64;
     }
-    const size_t ozn = digits == 7 ? oz_bytes : oz64_bytes;
     size_t gws_bytes = 0;
     double* gws = cv.rest(&gws_bytes);
     ws_bytes = gws_bytes;
     const bool truncated = core->sgn && k < r;
     if (!truncated) {
         // F = AX R^{-1}
-        if (AX->dtype == GN_F32) {
-            GN_TRY(copy_f32_to_f64(h, static_cast<const float*>(AX->data), m, r, AX->ld, Fd, F->ld));
-        } else {
-            GN_CUDA_TRY(cudaMemcpy2DAsync(Fd, F->ld * 8, AX->data, AX->ld * 8, r * 8, m, cudaMemcpyDeviceToDevice,
-                                          h->stream));
-        }
-        GN_TRY(trsm_right_upper(h, Fd, m, r, F->ld, core->R, r, 0, gws, ws_bytes, oz, ozn, digits));
+        GN_TRY(trsm_right_upper(h, Fd, m, r, F->ld, core->R, r, 0, gws, ws_bytes, oz, ozn, digits, AX->data,
+                                AX->dtype == GN_F32, AX->ld));
     } else {
         // F = (AX Q_2) R_2^{-T}
         if (oz && AX->dtype == GN_F32)
@@ -1184,12 +1175,29 @@ size_t apply_ws(long long m, long long n, long long r, long long l, long long kw
            apply_oz_ws(m, n, r, l, kw) + 1024;
 }
 
+// What gn_apply_workspace_size adds for the nine-digit products and the solve on
+// the tensor cores; gn_apply runs them on the FP64 units in a workspace of apply_ws.
+size_t apply_fast_ws(long long r, long long l, long long kw, int sms) {
+    const long long rl = r + l;
+    return align256(trsm_oz_ws_bytes(kw, r, OZ_DIGITS_F64)) +
+           std::max({dgemm_fast_ws_bytes(kw, r, rl, sms), dgemm_fast_ws_bytes(kw, r, r, sms),
+                     dgemm_fast_ws_bytes(kw, rl, r, sms)}) + 512;
+}
+// ... and for the products with FP64 sketches.
+size_t apply_fast64_ws(long long m, long long n, long long r, long long l, long long kw, int sms) {
+    const long long rl = r + l;
+    return align256(trsm_oz_ws_bytes(kw, r, OZ_DIGITS_F64)) +
+           std::max({dgemm_fast_ws_bytes(rl, kw, n, sms), dgemm_fast_ws_bytes(m, kw, r, sms),
+                     dgemm_fast_ws_bytes(kw, r, m, sms), dgemm_fast_ws_bytes(kw, n, rl, sms)}) + 512;
+}
+
 gn_status gn_apply_workspace_size(int64_t m, int64_t n, int64_t r, int64_t l, int64_t kw, int32_t side,
                                   size_t* bytes) {
     if (!bytes || m < 1 || n < 1 || r < 1 || l < 0 || kw < 1 || (side != 0 && side != 1)) return GN_ERR_INVALID_ARG;
     int dev = 0, sms = 148;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    *bytes = apply_ws(m, n, r, l, kw, sms);
+    *bytes = apply_ws(m, n, r, l, kw, sms) +
+             std::max(apply_fast_ws(r, l, kw, sms), apply_fast64_ws(m, n, r, l, kw, sms));
     return GN_OK;
 }
 
@@ -1225,6 +1233,17 @@ gn_status gn_apply(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_co
     if (!cv.ok) return GN_ERR_WORKSPACE;
     size_t gws_bytes = 0;
     double* gws = cv.rest(&gws_bytes);
+    // the core-sized products and the solve: nine digits, in what ws holds beyond the FP64 units' scratch
+    const size_t spare = ws_bytes - apply_ws(m, n, r, l, kw, h->sm_count);
+    const size_t fast_need = apply_fast_ws(r, l, kw, h->sm_count);
+    const bool fast = h->fp64_tc && spare >= fast_need;
+    void* sol = nullptr;
+    const size_t sol_bytes = trsm_oz_ws_bytes(kw, r, OZ_DIGITS_F64);
+    if (fast) {   // the front of the remaining scratch to the solve
+        sol = gws;
+        gws = reinterpret_cast<double*>(reinterpret_cast<char*>(gws) + align256(sol_bytes));
+        gws_bytes -= align256(sol_bytes);
+    }
     const double* Wd = static_cast<const double*>(W->data);
     double* Od = static_cast<double*>(out->data);
     if (side == 0) {
@@ -1235,18 +1254,18 @@ gn_status gn_apply(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_co
             GN_TRY(dgemm_a32(h, rl, kw, n, 1.0, static_cast<const float*>(YtA->data), YtA->ld, 0, Wd, W->ld, 0, 0.0,
                              B1, kw, gws, gws_bytes));
         else
-            GN_TRY(dgemm(h, rl, kw, n, 1.0, static_cast<const double*>(YtA->data), YtA->ld, 0, Wd, W->ld, 0, 0.0, B1,
+            GN_TRY(dgemm_fast(h, rl, kw, n, 1.0, static_cast<const double*>(YtA->data), YtA->ld, 0, Wd, W->ld, 0, 0.0, B1,
                          kw, gws, gws_bytes));
         // B2 = (Q_1^T B1)^T = B1^T Q_1   (kw x k)
-        GN_TRY(dgemm(h, kw, k, rl, 1.0, B1, kw, 1, core->Q, r, 0, 0.0, B2, k, gws, gws_bytes));
+        GN_TRY(dgemm_fast(h, kw, k, rl, 1.0, B1, kw, 1, core->Q, r, 0, 0.0, B2, k, gws, gws_bytes));
         const double* Zt = B2;   // Z^T (kw x r) with Z the core pseudoinverse applied to Y^T A W
         if (!trunc) {
             // (R^{-1} Q^T B1)^T = B2 R^{-T}
-            GN_TRY(trsm_right_upper(h, B2, kw, r, k, core->R, r, 1, gws, gws_bytes));
+            GN_TRY(trsm_right_upper(h, B2, kw, r, k, core->R, r, 1, gws, gws_bytes, sol, sol_bytes, OZ_DIGITS_F64));
         } else {
             // (R_2^{-T} Q_1^T B1)^T = B2 R_2^{-1}, then Z^T = that Q_2^T (kw x r)
-            GN_TRY(trsm_right_upper(h, B2, kw, k, k, core->R2, r, 0, gws, gws_bytes));
-            GN_TRY(dgemm(h, kw, r, k, 1.0, B2, k, 0, core->Q2, r, 1, 0.0, B1, r, gws, gws_bytes));
+            GN_TRY(trsm_right_upper(h, B2, kw, k, k, core->R2, r, 0, gws, gws_bytes, sol, sol_bytes, OZ_DIGITS_F64));
+            GN_TRY(dgemm_fast(h, kw, r, k, 1.0, B2, k, 0, core->Q2, r, 1, 0.0, B1, r, gws, gws_bytes));
             Zt = B1;
         }
         // out = AX Z = AX (Z^T)^T   (m x kw)
@@ -1256,7 +1275,7 @@ gn_status gn_apply(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_co
             GN_TRY(dgemm_a32(h, m, kw, r, 1.0, static_cast<const float*>(AX->data), AX->ld, 0, Zt, r, 1, 0.0, Od,
                              out->ld, gws, gws_bytes));
         else
-            GN_TRY(dgemm(h, m, kw, r, 1.0, static_cast<const double*>(AX->data), AX->ld, 0, Zt, r, 1, 0.0, Od, out->ld,
+            GN_TRY(dgemm_fast(h, m, kw, r, 1.0, static_cast<const double*>(AX->data), AX->ld, 0, Zt, r, 1, 0.0, Od, out->ld,
                          gws, gws_bytes));
         return GN_OK;
     }
@@ -1268,20 +1287,20 @@ gn_status gn_apply(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_co
         GN_TRY(dgemm_b32(h, kw, r, m, 1.0, Wd, W->ld, 0, static_cast<const float*>(AX->data), AX->ld, 0, 0.0, B1, r,
                          gws, gws_bytes));
     else
-        GN_TRY(dgemm(h, kw, r, m, 1.0, Wd, W->ld, 0, static_cast<const double*>(AX->data), AX->ld, 0, 0.0, B1, r,
+        GN_TRY(dgemm_fast(h, kw, r, m, 1.0, Wd, W->ld, 0, static_cast<const double*>(AX->data), AX->ld, 0, 0.0, B1, r,
                      gws, gws_bytes));
     const double* P = B1;   // (kw x k): (W AX) times the core pseudoinverse's left part
     if (!trunc) {
-        GN_TRY(trsm_right_upper(h, B1, kw, r, r, core->R, r, 0, gws, gws_bytes));
+        GN_TRY(trsm_right_upper(h, B1, kw, r, r, core->R, r, 0, gws, gws_bytes, sol, sol_bytes, OZ_DIGITS_F64));
     } else {
-        GN_TRY(dgemm(h, kw, k, r, 1.0, B1, r, 0, core->Q2, r, 0, 0.0, B2, k, gws, gws_bytes));
-        GN_TRY(trsm_right_upper(h, B2, kw, k, k, core->R2, r, 1, gws, gws_bytes));
+        GN_TRY(dgemm_fast(h, kw, k, r, 1.0, B1, r, 0, core->Q2, r, 0, 0.0, B2, k, gws, gws_bytes));
+        GN_TRY(trsm_right_upper(h, B2, kw, k, k, core->R2, r, 1, gws, gws_bytes, sol, sol_bytes, OZ_DIGITS_F64));
         P = B2;
     }
     const long long ldp = trunc ? k : r;
     // B = P Q_1^T   (kw x (r+l)), into the buffer P does not occupy
     double* Bq = trunc ? B1 : B2;
-    GN_TRY(dgemm(h, kw, rl, k, 1.0, P, ldp, 0, core->Q, r, 1, 0.0, Bq, rl, gws, gws_bytes));
+    GN_TRY(dgemm_fast(h, kw, rl, k, 1.0, P, ldp, 0, core->Q, r, 1, 0.0, Bq, rl, gws, gws_bytes));
     // out = B Y^T A   (kw x n)
     if (yta32 && oz) {   // (B Y^T A)^T = (Y^T A)^T B^T, then transposed
         GN_TRY(oz_dgemm(h, n, kw, rl, 1.0, YtA->data, 1, YtA->ld, 1, Bq, rl, 1, 0.0, T2, kw, ozw, ozb));
@@ -1290,7 +1309,7 @@ gn_status gn_apply(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_co
         GN_TRY(dgemm_b32(h, kw, n, rl, 1.0, Bq, rl, 0, static_cast<const float*>(YtA->data), YtA->ld, 0, 0.0, Od,
                          out->ld, gws, gws_bytes));
     else
-        GN_TRY(dgemm(h, kw, n, rl, 1.0, Bq, rl, 0, static_cast<const double*>(YtA->data), YtA->ld, 0, 0.0, Od, out->ld,
+        GN_TRY(dgemm_fast(h, kw, n, rl, 1.0, Bq, rl, 0, static_cast<const double*>(YtA->data), YtA->ld, 0, 0.0, Od, out->ld,
                      gws, gws_bytes));
     return GN_OK;
 }

@@ -2210,58 +2210,300 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
     return dgemm_ws_bytes(m, TB, k, sm_count) + 256;
 }
 
+// ---------------------------------------------------------------------------
+// Triangular solve with the products on the tensor cores.  With blocks J of 128
+// columns, F R = B gives
+//     F_J = (B_J - F_{<J} R_{<J,J}) R_JJ^{-1} = [F_{<J}, B_J] W_J,
+//     W_J = [-R_{<J,J} R_JJ^{-1}; R_JJ^{-1}],
+// and, with the blocks from the last one back, F R^T = B gives
+//     F_J = [B_J, F_{>J}] W_J,   W_J = [R_JJ^{-T}; -R_{J,>J}^T R_JJ^{-T}].
+// F_{<J} and B_J are adjacent columns of F, so each block is one product in
+// place (its operand is sliced before C is written).  The rows of every W_J are
+// triangular solves of 128 unknowns, independent of one another: all of them
+// run in the launch below, in FP64 by substitution.
+// In this form the rows of [F, B_J] and the columns of W_J mix magnitudes: B_J is
+// |R_:J| times F, and the slices are relative to the largest entry.  So B's
+// column j is scaled by 2^-e_j beforehand, e_j the exponent of max_i |R_ij|
+// (trans: max_i |R_ji|), and the inverse's rows by 2^e_j: exact, and every term
+// of a product is then of one size (without it the error grew from 2e-10 to 8e-10
+// of F at r = 2000).
+// Against 32-column substitution steps with a wide update per 128 columns this
+// leaves three launches per 128 columns and no substitution over the m rows
+// (16 m k multiply-adds on the FP64 units).  m = 32768, k = 1000 (launches
+// summed): 5.83 -> 3.69 ms; gn_apply at m, n, k = 32768, 16384, 1000, 64
+// vectors: 4.90 -> 1.49 ms; gn_apply's solve alone (m = 64) 3.5 -> 0.5 ms.
+// Error of F against FP64 substitution at m = 32768, k = 1000: 2.5e-12 with 8
+// digits (2.6e-10 with the seven-digit updates before).
+// ---------------------------------------------------------------------------
+constexpr int TW = 128;              // columns per block
+constexpr int TW_ROWS = 32;          // rows of W per CTA
+constexpr int TW_THREADS = 512;      // a warp carries TW_ROWS / 16 rows
+constexpr long long TRSM_ROWS = 32768;   // rows of F solved together (bounds the slices' scratch)
+
+// Rows of W_J in the stacked W, and its first row.
+__host__ __device__ inline long long tw_rows(long long J, long long k, int trans) {
+    return trans ? k - J * TW : (J * TW + TW < k ? J * TW + TW : k);
+}
+__host__ __device__ inline long long tw_base(long long J, long long k, int trans) {
+    return trans ? J * k - TW * (J * (J - 1) / 2) : TW * (J * (J + 1) / 2);
+}
+
+// e_j = exponent of the largest |R_ij|, i <= j (trans: |R_ji|, i >= j); 0 for a zero
+// or non-finite column.  A CTA takes 32 columns (trans: rows).
+__global__ void __launch_bounds__(1024) tri_scale_kernel(const double* __restrict__ R, long long ldr, int k, int trans,
+                                                        int* __restrict__ e) {
+    __shared__ unsigned long long red[32][33];
+    const int c0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long m = 0;   // |x| as an unsigned integer orders like |x|
+    if (!trans) {
+        const int j = c0 + lane;
+        if (j < k)
+            for (int i = warp; i <= j; i += 32)
+                m = max(m, static_cast<unsigned long long>(__double_as_longlong(R[static_cast<long long>(i) * ldr + j])) & 0x7FFFFFFFFFFFFFFFull);
+        red[warp][lane] = m;
+    } else {
+        const int j = c0 + warp;
+        if (j < k)
+            for (int i = j + lane; i < k; i += 32)
+                m = max(m, static_cast<unsigned long long>(__double_as_longlong(R[static_cast<long long>(j) * ldr + i])) & 0x7FFFFFFFFFFFFFFFull);
+        red[lane][warp] = m;
+    }
+    __syncthreads();
+    if (warp == 0 && c0 + lane < k) {
+        for (int w = 1; w < 32; ++w) m = max(m, red[w][lane]);
+        m = max(m, red[0][lane]);
+        const int E = static_cast<int>(m >> 52);
+        e[c0 + lane] = E == 0 || E == 0x7FF ? 0 : max(-500, min(500, E - 1023));
+    }
+}
+
+// F[:, j] = 2^-e_j src[:, j] (src FP32, FP64 or F itself).  A thread takes four
+// rows of a column (coalesced along the row).
+template <typename T>
+__global__ void __launch_bounds__(256) tri_scale_copy_kernel(const T* src, long long lds, double* F, long long ldf,
+                                                            long long m, int k, const int* __restrict__ e) {
+    const int j = blockIdx.x * 64 + (threadIdx.x & 63);
+    if (j >= k) return;
+    const double s = __longlong_as_double(static_cast<long long>(1023 - e[j]) << 52);
+    for (long long i = blockIdx.y * 16LL + (threadIdx.x >> 6) * 4; i < m; i += gridDim.y * 16LL) {
+        T v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) v[u] = i + u < m ? src[(i + u) * lds + j] : T(0);
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if (i + u < m) F[(i + u) * ldf + j] = static_cast<double>(v[u]) * s;
+    }
+}
+
+// Row kk of W_J solves x R_JJ = e_c (kk in J) or x R_JJ = -R[kk, J] (forward over
+// the columns), trans: x R_JJ^T = e_c or -R[J, kk]^T (backward).  With the
+// coefficients scaled by the reciprocal pivots, Cs[a][b] = R_ab / R_aa, the
+// unknowns before their own scaling follow x_b -= x_a Cs[a][b], one shuffle and
+// one FMA per step of the chain; x_a / R_aa at the end.  A CTA keeps Cs in
+// shared memory for its 32 rows, two per warp (one row's shuffle overlaps the
+// other's FMA).  Bound by the FP64 rate: k = 1000: 38 M multiply-adds.
+__global__ void __launch_bounds__(TW_THREADS) tri_w_kernel(const double* __restrict__ R, long long ldr, int k,
+                                                          int trans, const int* __restrict__ e,
+                                                          double* __restrict__ W) {
+    extern __shared__ double tw_sm[];
+    double* Cs = tw_sm;              // [TW][TW + 1]
+    double* rd = Cs + TW * (TW + 1); // [TW]
+    const int J = blockIdx.y, J0 = J * TW, bw = min(TW, k - J0);
+    const int rows = static_cast<int>(tw_rows(J, k, trans));
+    const int r0 = blockIdx.x * TW_ROWS;
+    if (r0 >= rows) return;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (tid < TW) rd[tid] = tid < bw ? 1.0 / R[static_cast<long long>(J0 + tid) * (ldr + 1)] : 0.0;
+    __syncthreads();
+    for (int e = tid; e < TW * TW; e += TW_THREADS) {
+        const int a = e / TW, b = e % TW;   // R_ab, a < b: read along rows
+        const double v = a < b && b < bw ? R[static_cast<long long>(J0 + a) * ldr + J0 + b] : 0.0;
+        if (trans) Cs[b * (TW + 1) + a] = v * rd[b];   // eliminates x_b from x_a, a < b
+        else Cs[a * (TW + 1) + b] = v * rd[a];
+    }
+    __syncthreads();
+    constexpr int NR = TW_ROWS / (TW_THREADS / 32), NT = TW / 32;
+    double x[NR][NT];
+    // row kk's position: its column inside J, or its row / column of R outside
+    const int in0 = trans ? 0 : J0;   // rows [in0, in0 + bw) of W_J are the inverse's
+    int kk[NR];
+    bool any = false;
+#pragma unroll
+    for (int u = 0; u < NR; ++u) {
+        kk[u] = r0 + NR * warp + u;
+        const int c = kk[u] - in0;
+        const bool unit = c >= 0 && c < bw;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) {
+            const int b = 32 * t + lane;
+            double v = 0.0;
+            if (unit) v = b == c ? 1.0 : 0.0;
+            else if (kk[u] < rows && b < bw)
+                v = trans ? -R[static_cast<long long>(J0 + b) * ldr + J0 + kk[u]]
+                          : -R[static_cast<long long>(kk[u]) * ldr + J0 + b];
+            x[u][t] = v;
+        }
+        any |= kk[u] < rows;
+    }
+    if (!any) return;   // warp-uniform; no barrier follows
+    if (!trans) {
+#pragma unroll
+        for (int p = 0; p < NT; ++p) {
+            if (32 * p >= bw) break;
+#pragma unroll 8
+            for (int s = 0; s < 32; ++s) {
+                const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+#pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
+#pragma unroll
+                    for (int t = p; t < NT; ++t)
+                        if (t > p || lane > s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
+                }
+            }
+        }
+    } else {
+#pragma unroll
+        for (int p = NT - 1; p >= 0; --p) {
+            if (32 * p >= bw) continue;
+#pragma unroll 8
+            for (int s = 31; s >= 0; --s) {
+                const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+#pragma unroll
+                for (int u = 0; u < NR; ++u) {
+                    const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
+#pragma unroll
+                    for (int t = 0; t <= p; ++t)
+                        if (t < p || lane < s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
+                }
+            }
+        }
+    }
+    double* out = W + tw_base(J, k, trans) * TW;
+#pragma unroll
+    for (int u = 0; u < NR; ++u)
+        if (kk[u] < rows) {
+            const int c = kk[u] - in0;
+            const double sc = c >= 0 && c < bw ? __longlong_as_double(static_cast<long long>(1023 + e[J0 + c]) << 52) : 1.0;
+#pragma unroll
+            for (int t = 0; t < NT; ++t)
+                if (32 * t + lane < bw)
+                    out[static_cast<long long>(kk[u]) * TW + 32 * t + lane] = x[u][t] * rd[32 * t + lane] * sc;
+        }
+}
+
+size_t tw_bytes(long long k) {   // the stacked W of either direction
+    const long long nb = (k + TW - 1) / TW;
+    const long long rows = std::max(tw_base(nb - 1, k, 0) + tw_rows(nb - 1, k, 0), tw_base(nb - 1, k, 1) + tw_rows(nb - 1, k, 1));
+    return ((sizeof(double) * rows * TW + 255) & ~static_cast<size_t>(255)) +
+           ((sizeof(int) * k + 255) & ~static_cast<size_t>(255));   // and the exponents
+}
+
+size_t trsm_oz_ws_bytes(long long m, long long k, int digits) {
+    return tw_bytes(k) + oz_ws_bytes(std::min(m, TRSM_ROWS), std::min<long long>(k, TW), k, 0, digits) + 256;
+}
+
+gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ldf, const double* R, long long ldr,
+                  int trans, char* oz, size_t oz_bytes, int digits, const void* src, int src_f32, long long lds) {
+    const long long nb = (k + TW - 1) / TW;
+    const size_t wb = tw_bytes(k);
+    double* W = reinterpret_cast<double*>(oz);
+    int* e = reinterpret_cast<int*>(oz + wb - ((sizeof(int) * k + 255) & ~static_cast<size_t>(255)));
+    oz += wb;
+    oz_bytes -= wb;
+    // rows at a time: as many as the scratch holds
+    long long rows = std::min(m, TRSM_ROWS);
+    while (oz_ws_bytes(rows, std::min<long long>(k, TW), k, 0, digits) > oz_bytes) rows = (rows + 1) / 2;
+    constexpr size_t smem = sizeof(double) * (TW * (TW + 1) + TW);
+    static bool attr = false;
+    if (!attr) {
+        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(smem)));
+        attr = true;
+    }
+    const int ki = static_cast<int>(k);
+    tri_scale_kernel<<<static_cast<unsigned>((k + 31) / 32), 1024, 0, h->stream>>>(R, ldr, ki, trans, e);
+    count_launch();
+    GN_CUDA_TRY(cudaGetLastError());
+    const dim3 cgrid(static_cast<unsigned>((k + 63) / 64), static_cast<unsigned>(std::min<long long>((m + 15) / 16, 8LL * h->sm_count)));
+    if (src_f32)
+        tri_scale_copy_kernel<float><<<cgrid, 256, 0, h->stream>>>(static_cast<const float*>(src), lds, F, ldf, m, ki, e);
+    else
+        tri_scale_copy_kernel<double><<<cgrid, 256, 0, h->stream>>>(static_cast<const double*>(src), lds, F, ldf, m, ki, e);
+    count_launch();
+    GN_CUDA_TRY(cudaGetLastError());
+    tri_w_kernel<<<dim3(static_cast<unsigned>((k + TW_ROWS - 1) / TW_ROWS), static_cast<unsigned>(nb)), TW_THREADS,
+                   smem, h->stream>>>(R, ldr, ki, trans, e, W);
+    count_launch();
+    GN_CUDA_TRY(cudaGetLastError());
+    constexpr long long KG = 4096;   // K of one in-place product: sliced whole before C is written
+    for (long long i0 = 0; i0 < m; i0 += rows) {
+        const long long mm = std::min(rows, m - i0);
+        double* Fi = F + i0 * ldf;
+        for (long long b = 0; b < nb; ++b) {
+            const long long J = trans ? nb - 1 - b : b, J0 = J * TW, bw = std::min<long long>(TW, k - J0);
+            const long long K = tw_rows(J, k, trans), c0 = trans ? J0 : 0;   // operand columns [c0, c0 + K)
+            const double* Wj = W + tw_base(J, k, trans) * TW;
+            // the part of K that holds B_J first (in place), then the rest onto it
+            const long long k0 = trans ? 0 : std::max<long long>(0, K - KG), k1 = trans ? std::min(K, KG) : K;
+            GN_TRY(oz_dgemm(h, mm, bw, k1 - k0, 1.0, Fi + c0 + k0, 0, ldf, 0, Wj + k0 * TW, TW, 0, 0.0, Fi + J0, ldf,
+                            oz, oz_bytes, digits));
+            const long long q0 = trans ? k1 : 0, q1 = trans ? K : k0;
+            if (q1 > q0)
+                GN_TRY(oz_dgemm(h, mm, bw, q1 - q0, 1.0, Fi + c0 + q0, 0, ldf, 0, Wj + q0 * TW, TW, 0, 1.0, Fi + J0,
+                                ldf, oz, oz_bytes, digits));
+        }
+    }
+    return GN_OK;
+}
+
 gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, long long ldf,
                            const double* R, long long ldr, int trans, double* ws, size_t ws_bytes, void* oz,
-                           size_t oz_bytes, int digits) {
+                           size_t oz_bytes, int digits, const void* src, int src_f32, long long lds) {
     if (m <= 0 || k <= 0) return GN_OK;
-    // Two levels of blocking: 128-column outer blocks take the bulk of the
-    // update as one wide FP64 GEMM each; inside, 32-column blocks take a narrow
-    // GEMM over the outer block and the per-row triangular solve.
+    if (!src) {
+        src = F;
+        src_f32 = 0;
+        lds = ldf;
+    }
+    if (oz && k > TB) {   // (one 32-column block is one substitution launch)
+        const size_t pad = (256 - (reinterpret_cast<uintptr_t>(oz) & 255)) & 255;
+        if (oz_bytes >= pad + tw_bytes(k) + oz_ws_bytes(std::min<long long>(m, 256), std::min<long long>(k, TW), k, 0, digits))
+            return trsm_oz(h, F, m, k, ldf, R, ldr, trans, static_cast<char*>(oz) + pad, oz_bytes - pad, digits,
+                           src, src_f32, lds);
+    }
+    if (src_f32)
+        GN_TRY(copy_f32_to_f64(h, static_cast<const float*>(src), m, k, lds, F, ldf));
+    else if (src != F)
+        GN_CUDA_TRY(cudaMemcpy2DAsync(F, ldf * 8, src, lds * 8, k * 8, m, cudaMemcpyDeviceToDevice, h->stream));
+    // FP64 units.  Two levels of blocking: 128-column outer blocks take the bulk
+    // of the update as one wide FP64 GEMM each; inside, 32-column blocks take a
+    // narrow GEMM over the outer block and the per-row triangular solve.
     constexpr long long OB = 128;
     const long long nob = (k + OB - 1) / OB;
     const int blocks = static_cast<int>((m + 127) / 128);
     for (long long obi = 0; obi < nob; ++obi) {
         const long long ob = trans ? nob - 1 - obi : obi;
         const long long J0 = ob * OB, JB = std::min<long long>(OB, k - J0);
-        // (oz: these and the inner updates below on the tensor cores by exact digit slicing)
-        if (!trans && J0 > 0) {   // F[:, J] -= F[:, 0:J0] R[0:J0, J]
-            if (oz)
-                GN_TRY(oz_dgemm(h, m, JB, J0, -1.0, F, 0, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, oz, oz_bytes, digits));
-            else
-                GN_TRY(dgemm(h, m, JB, J0, -1.0, F, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, ws, ws_bytes));
-        }
+        if (!trans && J0 > 0)   // F[:, J] -= F[:, 0:J0] R[0:J0, J]
+            GN_TRY(dgemm(h, m, JB, J0, -1.0, F, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, ws, ws_bytes));
         if (trans && J0 + JB < k) {   // F[:, J] -= F[:, J+] R[J, J+]^T
             const long long kk = k - J0 - JB;
-            if (oz)
-                GN_TRY(oz_dgemm(h, m, JB, kk, -1.0, F + J0 + JB, 0, ldf, 0, R + J0 * ldr + J0 + JB, ldr, 1, 1.0,
-                                F + J0, ldf, oz, oz_bytes, digits));
-            else
-                GN_TRY(dgemm(h, m, JB, kk, -1.0, F + J0 + JB, ldf, 0, R + J0 * ldr + J0 + JB, ldr, 1, 1.0, F + J0,
-                             ldf, ws, ws_bytes));
+            GN_TRY(dgemm(h, m, JB, kk, -1.0, F + J0 + JB, ldf, 0, R + J0 * ldr + J0 + JB, ldr, 1, 1.0, F + J0,
+                         ldf, ws, ws_bytes));
         }
         const long long nb = (JB + TB - 1) / TB;
         for (long long bi = 0; bi < nb; ++bi) {
             const long long b = trans ? nb - 1 - bi : bi;
             const long long j0 = J0 + b * TB;
             const int jb = static_cast<int>(std::min<long long>(TB, J0 + JB - j0));
-            if (!trans && j0 > J0) {
-                // F[:, j] -= F[:, J0:j0] R[J0:j0, j]
-                if (oz)
-                    GN_TRY(oz_dgemm(h, m, jb, j0 - J0, -1.0, F + J0, 0, ldf, 0, R + J0 * ldr + j0, ldr, 0, 1.0,
-                                    F + j0, ldf, oz, oz_bytes, digits));
-                else
-                    GN_TRY(dgemm(h, m, jb, j0 - J0, -1.0, F + J0, ldf, 0, R + J0 * ldr + j0, ldr, 0, 1.0, F + j0, ldf,
-                                 ws, ws_bytes));
-            }
-            if (trans && j0 + jb < J0 + JB) {
-                // F[:, j] -= F[:, j+ .. J0+JB] R[j, j+ ..]^T
+            if (!trans && j0 > J0)   // F[:, j] -= F[:, J0:j0] R[J0:j0, j]
+                GN_TRY(dgemm(h, m, jb, j0 - J0, -1.0, F + J0, ldf, 0, R + J0 * ldr + j0, ldr, 0, 1.0, F + j0, ldf,
+                             ws, ws_bytes));
+            if (trans && j0 + jb < J0 + JB) {   // F[:, j] -= F[:, j+ .. J0+JB] R[j, j+ ..]^T
                 const long long kk = J0 + JB - j0 - jb;
-                if (oz)
-                    GN_TRY(oz_dgemm(h, m, jb, kk, -1.0, F + j0 + jb, 0, ldf, 0, R + j0 * ldr + j0 + jb, ldr, 1, 1.0,
-                                    F + j0, ldf, oz, oz_bytes, digits));
-                else
-                    GN_TRY(dgemm(h, m, jb, kk, -1.0, F + j0 + jb, ldf, 0, R + j0 * ldr + j0 + jb, ldr, 1, 1.0, F + j0,
-                                 ldf, ws, ws_bytes));
+                GN_TRY(dgemm(h, m, jb, kk, -1.0, F + j0 + jb, ldf, 0, R + j0 * ldr + j0 + jb, ldr, 1, 1.0,
+                             F + j0, ldf, ws, ws_bytes));
             }
             trsm_diag_kernel<<<blocks, 128, 0, h->stream>>>(F, m, ldf, static_cast<int>(j0), jb, R, ldr, trans); count_launch();
             GN_CUDA_TRY(cudaGetLastError());

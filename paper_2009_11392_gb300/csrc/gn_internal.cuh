@@ -200,21 +200,32 @@ gn_status qr_form_q(gn_handle h, const double* W, long long M, long long N, long
                     long long ldq, double* ws, size_t ws_bytes, void* oz = nullptr, size_t oz_bytes = 0);
 size_t qr_oz_ws_bytes(long long M, long long N);
 
-// Right triangular solves, FP64, in place on F (m x k):
+// Digits per operand of the FP64 path's products, and of the solves that follow
+// FP32 sketches (the conditioning of R amplifies their rounding: 8 digits keep it
+// at the FP64 units' size, 7 would not).
+constexpr int OZ_DIGITS_F64 = 9;
+constexpr int OZ_DIGITS_SOLVE = 8;
+
+// Right triangular solves, FP64, on F (m x k), in place or from src (m x k, FP32 or
+// FP64, ld lds, not overlapping F):
 //   upper == 1, trans == 0: F <- F R^{-1}   (R upper, k x k)
 //   upper == 1, trans == 1: F <- F R^{-T}
-// oz (optional): workspace of oz_dgemm for the outer-block updates (>= oz_ws_bytes(m,
-// 128, k, 0)); null keeps every update on the FP64 units.
+// oz (optional; trsm_oz_ws_bytes(m, k, digits) solves up to 32768 rows together,
+// less takes fewer rows at a time, too little the FP64 units): the products by
+// digit slicing with `digits` (8 or 9) digits; null: the FP64 units.
+size_t trsm_oz_ws_bytes(long long m, long long k, int digits);
 size_t trsm_ws_bytes(long long m, long long k, int sm_count);
 gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, long long ldf,
                            const double* R, long long ldr, int trans, double* ws, size_t ws_bytes,
-                           void* oz = nullptr, size_t oz_bytes = 0, int digits = 7);
+                           void* oz = nullptr, size_t oz_bytes = 0, int digits = OZ_DIGITS_SOLVE,
+                           const void* src = nullptr, int src_f32 = 0, long long lds = 0);
 
 // FP64 product on the BF16 tensor cores by exact digit slicing (gn_ozaki.cu);
 // same operand conventions as dgemm, A FP64 or (a_f32) FP32.  digits: BF16
 // digits per operand row / column (7: FP64 accuracy; d < 7: every term carries
-// an error of about 2^(1 - 7d) max|a_i.| max|b_.j|).
-constexpr int OZ_DIGITS_F64 = 9;
+// an error of about 2^(1 - 7d) max|a_i.| max|b_.j|).  8 or 9 digits (FP64 A): a
+// 63-bit window, and infinities and NaN propagate.  C may overlap A or B when
+// K <= 4096 (both are sliced before C is written).
 size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32, int digits = 7);
 gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double alpha, const void* A, int a_f32,
                    long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
