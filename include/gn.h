@@ -188,8 +188,8 @@ gn_status gn_set_fp64_accum(gn_handle h, int64_t part_k);
  * element); 0: on the FP64 units.  The panels, the small diagonal-block solves
  * and the detector stay in FP64 either way.
  * For GN_F64 operands the switch covers gn_sketch (and the calls built on it),
- * the core product C, the factors and gn_hmt's two products: 1 (default) forms
- * them from nine digits per operand (63 bits below the largest entry of each
+ * the core product C, the factors, gn_apply and gn_hmt's two products: 1
+ * (default) forms those of more than 2^24 multiply-adds from nine digits per operand (63 bits below the largest entry of each
  * row of the left and column of the right operand: the error per element is
  * about 2^-60 sqrt(K) max_k |a_ik| max_k |b_kj|, below the rounding error of an
  * FP64 sum), infinities and NaN as the FP64 units give them; a workspace too

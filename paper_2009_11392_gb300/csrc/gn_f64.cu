@@ -189,6 +189,125 @@ __global__ void reduce_sum_kernel(const double* __restrict__ part, long long n, 
     }
 }
 
+// --------------------------------------------------------------------------
+// Small FP64 products.  The FP64 units take ~64 cycles per warp instruction and
+// sub-partition, so a product of a few million multiply-adds is bound by how
+// evenly it spreads over the SMs: tiles of 32 rows by 4 NC columns (a lane per
+// row, NC columns per warp, nothing wasted beyond the next multiple), and K
+// split over a cluster whose partial sums are added in rank order through
+// distributed shared memory (one launch, a fixed order of additions).
+// 1000 x 20 x 500: 94 + 5 us as 64 x 64 tiles with split K and a reduction
+// launch, 28 us here (10 M multiply-adds: 21 us at the units' rate); 30 x 500 x
+// 1000: 95 + 6 and 43 us (31); both sketch products at 64 x 64, r = 8: 108 and 14.
+// The columns of A from ka on come from A2 (an operand in two buffers).
+// --------------------------------------------------------------------------
+constexpr int SG_THREADS = 128;
+constexpr int SG_BM = 32;
+constexpr int SG_KC = 32;
+constexpr int SG_MAX_SPLIT = 8;
+
+struct SmallGemm {
+    int M, N, K, ka, kchunk;
+    double alpha, beta;
+    const double *A, *A2, *B;
+    long long lda, lda2, ldb, ldc;
+    int ta, tb;
+    double* C;
+};
+
+template <int NC>
+__global__ void __launch_bounds__(SG_THREADS) dgemm_small_kernel(const __grid_constant__ SmallGemm g) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cluster = cg::this_cluster();
+    constexpr int BN = 4 * NC;
+    __shared__ double As[SG_KC][SG_BM + 1];
+    __shared__ double Bs[SG_KC][BN];
+    __shared__ double part[BN][SG_BM];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int n0 = blockIdx.x * BN, m0 = blockIdx.y * SG_BM;
+    const int S = gridDim.z, rank = blockIdx.z;
+    const int kbeg = rank * g.kchunk, kend = min(g.K, kbeg + g.kchunk);
+    constexpr int LA = SG_BM * SG_KC / SG_THREADS, LB = (BN * SG_KC + SG_THREADS - 1) / SG_THREADS;
+    double ra[LA], rb[LB];
+    auto load = [&](int k0) {   // the next stage's elements into registers (hides their latency behind the FMAs)
+#pragma unroll
+        for (int u = 0; u < LA; ++u) {
+            const int e = tid + u * SG_THREADS;
+            const int mm = g.ta ? e & 31 : e >> 5, kk = g.ta ? e >> 5 : e & 31;
+            const int i = m0 + mm, k = k0 + kk;
+            double v = 0.0;
+            if (i < g.M && k < kend) {
+                const double* p = k < g.ka ? g.A : g.A2;
+                const long long ld = k < g.ka ? g.lda : g.lda2;
+                v = g.ta ? p[k * ld + i] : p[i * ld + k];
+            }
+            ra[u] = v;
+        }
+#pragma unroll
+        for (int u = 0; u < LB; ++u) {
+            const int e = tid + u * SG_THREADS;
+            const int nn = g.tb ? e >> 5 : e % BN, kk = g.tb ? e & 31 : e / BN;
+            const int j = n0 + nn, k = k0 + kk;
+            double v = 0.0;
+            if (e < BN * SG_KC && j < g.N && k < kend)
+                v = g.tb ? g.B[j * g.ldb + k] : g.B[k * g.ldb + j];
+            rb[u] = v;
+        }
+    };
+    double acc[NC];
+#pragma unroll
+    for (int c = 0; c < NC; ++c) acc[c] = 0.0;
+    load(kbeg);
+    for (int k0 = kbeg; k0 < kend; k0 += SG_KC) {
+        __syncthreads();
+#pragma unroll
+        for (int u = 0; u < LA; ++u) {
+            const int e = tid + u * SG_THREADS;
+            if (g.ta) As[e >> 5][e & 31] = ra[u];
+            else As[e & 31][e >> 5] = ra[u];
+        }
+#pragma unroll
+        for (int u = 0; u < LB; ++u) {
+            const int e = tid + u * SG_THREADS;
+            if (e < BN * SG_KC) {
+                if (g.tb) Bs[e & 31][e >> 5] = rb[u];
+                else Bs[e / BN][e % BN] = rb[u];
+            }
+        }
+        __syncthreads();
+        if (k0 + SG_KC < kend) load(k0 + SG_KC);
+        const int kn = min(SG_KC, kend - k0);
+#pragma unroll 4
+        for (int kk = 0; kk < kn; ++kk) {
+            const double a = As[kk][lane];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) acc[c] = fma(a, Bs[kk][warp * NC + c], acc[c]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < NC; ++c) part[warp * NC + c][lane] = acc[c];
+    if (S > 1) cluster.sync();
+    else __syncthreads();
+    // outputs e = rank, rank + S, ... of the tile (rows of 32 by columns), summed in rank order
+    for (int e = rank * SG_THREADS + tid; e < BN * SG_BM; e += S * SG_THREADS) {
+        const int mm = e / BN, nn = e % BN, i = m0 + mm, j = n0 + nn;
+        double s = 0.0;
+        if (S > 1) {
+            double v[SG_MAX_SPLIT];
+#pragma unroll
+            for (int q = 0; q < SG_MAX_SPLIT; ++q) v[q] = q < S ? cluster.map_shared_rank(&part[nn][mm], q)[0] : 0.0;
+            for (int q = 0; q < S; ++q) s += v[q];
+        } else {
+            s = part[nn][mm];
+        }
+        if (i < g.M && j < g.N) {
+            double* c = g.C + i * g.ldc + j;
+            *c = g.beta == 0.0 ? g.alpha * s : fma(g.beta, *c, g.alpha * s);
+        }
+    }
+    if (S > 1) cluster.sync();   // peers read this CTA's partial sums
+}
+
 // Tile shape: 16 x 128 or 32 x 128 for panel-width products (M <= 32), else 64 x 64.
 inline int tile_m(long long M) { return M <= 16 ? 16 : (M <= 32 ? 32 : GT); }
 
@@ -233,6 +352,47 @@ gn_status dgemm_launch(gn_handle h, long long M, long long N, long long K, doubl
         splitk_reduce_kernel<<<blocks, 256, 0, h->stream>>>((int)M, (int)N, splits, ws, beta, C, ldc); count_launch();
     }
     GN_CUDA_TRY(cudaGetLastError());
+    return GN_OK;
+}
+
+// Products of at most this many multiply-adds take the small kernel: up to here
+// its time (about MNK / 400e9 s plus 5 us) is below the three launches of a digit-
+// sliced product (40-60 us) and below 64 x 64 tiles at any size that leaves SMs idle.
+constexpr long long SG_MAX_MACS = 16LL << 20;
+
+gn_status dgemm_small(gn_handle h, long long M, long long N, long long K, double alpha, const double* A, long long lda,
+                      int ta, const double* A2, long long lda2, long long ka, const double* B, long long ldb, int tb,
+                      double beta, double* C, long long ldc) {
+    // columns per warp: the widest that wastes nothing over the next narrower and keeps a few tiles per SM
+    int nc = 1;
+    for (int c : {2, 4}) {
+        const long long w0 = (N + 4 * nc - 1) / (4 * nc) * nc, w1 = (N + 4 * c - 1) / (4 * c) * c;
+        if (w1 <= w0 && (M + SG_BM - 1) / SG_BM * ((N + 4 * c - 1) / (4 * c)) * std::max<long long>(1, K / 64) >= 2LL * h->sm_count)
+            nc = c;
+    }
+    const long long tiles = (M + SG_BM - 1) / SG_BM * ((N + 4 * nc - 1) / (4 * nc));
+    // K parts: enough CTAs for four per SM (one per sub-partition's worth of warps), at least 32 of K each
+    long long S = std::max<long long>(1, std::min<long long>(SG_MAX_SPLIT, (4LL * h->sm_count + tiles - 1) / tiles));
+    S = std::max<long long>(1, std::min(S, K / SG_KC));
+    const long long kchunk = ((K + S - 1) / S + SG_KC - 1) / SG_KC * SG_KC;
+    S = (K + kchunk - 1) / kchunk;
+    SmallGemm g{static_cast<int>(M), static_cast<int>(N), static_cast<int>(K), static_cast<int>(ka),
+                static_cast<int>(kchunk), alpha, beta, A, A2, B, lda, lda2, ldb, ldc, ta, tb, C};
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((N + 4 * nc - 1) / (4 * nc)), static_cast<unsigned>((M + SG_BM - 1) / SG_BM),
+                       static_cast<unsigned>(S));
+    cfg.blockDim = dim3(SG_THREADS);
+    cfg.stream = h->stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = static_cast<unsigned>(S);
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    auto* kern = nc == 4 ? dgemm_small_kernel<4> : nc == 2 ? dgemm_small_kernel<2> : dgemm_small_kernel<1>;
+    GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, g));
+    count_launch();
     return GN_OK;
 }
 
@@ -1457,9 +1617,15 @@ size_t dgemm_ws_bytes(long long M, long long N, long long K, int sm_count) {
     return static_cast<size_t>(choose_splits(M, N, K, sm_count)) * M * N * sizeof(double);
 }
 
+bool small_gemm(long long M, long long N, long long K) {
+    return K >= 1 && M * N * K <= SG_MAX_MACS && (M + SG_BM - 1) / SG_BM <= 65535;
+}
+
 gn_status dgemm(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
                 long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                 long long ldc, double* ws, size_t ws_bytes) {
+    if (M > 0 && N > 0 && small_gemm(M, N, K))
+        return dgemm_small(h, M, N, K, alpha, A, lda, ta, A, lda, K, B, ldb, tb, beta, C, ldc);
     return dgemm_impl<double, double>(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, ws, ws_bytes);
 }
 
@@ -2230,8 +2396,8 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 // Against 32-column substitution steps with a wide update per 128 columns this
 // leaves three launches per 128 columns and no substitution over the m rows
 // (16 m k multiply-adds on the FP64 units).  m = 32768, k = 1000 (launches
-// summed): 5.83 -> 3.69 ms; gn_apply at m, n, k = 32768, 16384, 1000, 64
-// vectors: 4.90 -> 1.49 ms; gn_apply's solve alone (m = 64) 3.5 -> 0.5 ms.
+// summed): 5.83 -> 3.69 ms; m = 64, k = 1000: 3.5 -> 0.25 ms (its products on the
+// FP64 units), gn_apply there (32768 x 16384, 64 vectors) 4.90 -> 1.27 ms.
 // Error of F against FP64 substitution at m = 32768, k = 1000: 2.5e-12 with 8
 // digits (2.6e-10 with the seven-digit updates before).
 // ---------------------------------------------------------------------------
@@ -2403,6 +2569,24 @@ size_t trsm_oz_ws_bytes(long long m, long long k, int digits) {
     return tw_bytes(k) + oz_ws_bytes(std::min(m, TRSM_ROWS), std::min<long long>(k, TW), k, 0, digits) + 256;
 }
 
+// Few rows: the same block products on the FP64 units (dgemm_small), B's scaled
+// copy kept apart from F so that no product reads what another CTA writes.
+gn_status trsm_small(gn_handle h, double* F, long long m, long long k, long long ldf, const double* R, long long ldr,
+                     int trans, const double* W, const double* Bs) {
+    const long long nb = (k + TW - 1) / TW;
+    for (long long b = 0; b < nb; ++b) {
+        const long long J = trans ? nb - 1 - b : b, J0 = J * TW, bw = std::min<long long>(TW, k - J0);
+        const long long K = tw_rows(J, k, trans);
+        const double* Wj = W + tw_base(J, k, trans) * TW;
+        // operand columns: F_{<J} then B_J, or (trans) B_J then F_{>J}
+        const double* lo = trans ? Bs + J0 : F;
+        const double* hi = trans ? F + J0 : Bs;
+        GN_TRY(dgemm_small(h, m, bw, K, 1.0, lo, trans ? k : ldf, 0, hi, trans ? ldf : k, trans ? bw : J0, Wj, TW, 0, 0.0,
+                           F + J0, ldf));
+    }
+    return GN_OK;
+}
+
 gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ldf, const double* R, long long ldr,
                   int trans, char* oz, size_t oz_bytes, int digits, const void* src, int src_f32, long long lds) {
     const long long nb = (k + TW - 1) / TW;
@@ -2411,6 +2595,8 @@ gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ld
     int* e = reinterpret_cast<int*>(oz + wb - ((sizeof(int) * k + 255) & ~static_cast<size_t>(255)));
     oz += wb;
     oz_bytes -= wb;
+    const bool few = small_gemm(m, std::min<long long>(k, TW), k) &&
+                     sizeof(double) * m * k <= oz_bytes;   // few rows: FP64 units
     // rows at a time: as many as the scratch holds
     long long rows = std::min(m, TRSM_ROWS);
     while (oz_ws_bytes(rows, std::min<long long>(k, TW), k, 0, digits) > oz_bytes) rows = (rows + 1) / 2;
@@ -2425,17 +2611,20 @@ gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ld
     tri_scale_kernel<<<static_cast<unsigned>((k + 31) / 32), 1024, 0, h->stream>>>(R, ldr, ki, trans, e);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
+    double* Fs = few ? reinterpret_cast<double*>(oz) : F;   // the scaled B
+    const long long lds_f = few ? k : ldf;
     const dim3 cgrid(static_cast<unsigned>((k + 63) / 64), static_cast<unsigned>(std::min<long long>((m + 15) / 16, 8LL * h->sm_count)));
     if (src_f32)
-        tri_scale_copy_kernel<float><<<cgrid, 256, 0, h->stream>>>(static_cast<const float*>(src), lds, F, ldf, m, ki, e);
+        tri_scale_copy_kernel<float><<<cgrid, 256, 0, h->stream>>>(static_cast<const float*>(src), lds, Fs, lds_f, m, ki, e);
     else
-        tri_scale_copy_kernel<double><<<cgrid, 256, 0, h->stream>>>(static_cast<const double*>(src), lds, F, ldf, m, ki, e);
+        tri_scale_copy_kernel<double><<<cgrid, 256, 0, h->stream>>>(static_cast<const double*>(src), lds, Fs, lds_f, m, ki, e);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
     tri_w_kernel<<<dim3(static_cast<unsigned>((k + TW_ROWS - 1) / TW_ROWS), static_cast<unsigned>(nb)), TW_THREADS,
                    smem, h->stream>>>(R, ldr, ki, trans, e, W);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
+    if (few) return trsm_small(h, F, m, k, ldf, R, ldr, trans, W, Fs);
     constexpr long long KG = 4096;   // K of one in-place product: sliced whole before C is written
     for (long long i0 = 0; i0 < m; i0 += rows) {
         const long long mm = std::min(rows, m - i0);

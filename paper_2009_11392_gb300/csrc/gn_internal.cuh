@@ -234,6 +234,8 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
 // dgemm for FP64 operands through oz_dgemm with nine digits (63 bits below each
 // row's largest entry) where the product is large enough, ws holds
 // dgemm_fast_ws_bytes and gn_set_fp64_tc is on; dgemm otherwise.
+// Whether dgemm takes its kernel for products of few multiply-adds (no workspace).
+bool small_gemm(long long M, long long N, long long K);
 size_t dgemm_fast_ws_bytes(long long M, long long N, long long K, int sm_count);
 gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
                      long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,

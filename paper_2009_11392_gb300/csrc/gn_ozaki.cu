@@ -594,14 +594,12 @@ namespace {
 // Blocks of C per digit-sliced product: the scratch (the slices of up to 4096 of K)
 // stays near 2 GB however large the matrices are.
 constexpr long long OZ_MBLK = 8192, OZ_NBLK = 16384;
-// Least K for the tensor cores.  Three launches take about 20 us; on the FP64
-// units a 64 x 64 tile takes 1.1 us per element of K (256 multiply-adds per
-// sub-partition at ~64 cycles each per warp instruction), so K decides, not M
-// and N: both products of a sketch at m, n, r = 40, 32, 8: 41 us in slices and
-// 68 on the units; 64, 64, 8: 42 and 108; 500, 400, 16: 86 and 187; 4096, 2048,
-// 100: 436 and 5246; 20000, 10000, 500: 28.0 and 428.5 ms.
-constexpr long long OZ_F64_MIN_K = 24;
-bool oz_f64_pays(long long M, long long N, long long K) { return M >= 1 && N >= 1 && K >= OZ_F64_MIN_K; }
+// Digit slicing takes ~40 us of launches whatever the size; the FP64 units take
+// MNK / 485e9 s when the product spreads over the SMs (dgemm's small kernel), so
+// they keep products of up to 16 M multiply-adds.  Both products of a sketch at
+// m, n, r = 1000, 500, 20: 115 us in slices, 73 on the units; 4096, 2048, 100: 0.44 ms in slices and 5.25
+// on the units; 20000, 10000, 500: 28.0 and 428.5 ms.
+bool oz_f64_pays(long long M, long long N, long long K) { return M >= 1 && N >= 1 && K >= 1 && !small_gemm(M, N, K); }
 }  // namespace
 
 size_t dgemm_fast_ws_bytes(long long M, long long N, long long K, int sm_count) {

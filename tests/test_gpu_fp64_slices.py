@@ -1,6 +1,7 @@
-"""The FP64 path's products with nine digits per operand (gn_sketch on GN_F64
-operands) at the sizes where the blocking can go wrong, against exact integer
-products and against the FP64 units."""
+"""The FP64 path's products (gn_sketch on GN_F64 operands), with nine digits per
+operand above 2^24 multiply-adds and on the FP64 units below, at the sizes where
+the blocking can go wrong, against exact integer products and against the FP64
+units."""
 import numpy as np
 import pytest
 import torch
@@ -36,14 +37,17 @@ def run(gn, H, A, X, Y, ws=None, units=False):
     return AX, YtA
 
 
-# one pass and several, ragged tiles, blocks of C past 8192 rows and 16384 columns,
-# a leading dimension longer than a row (padded operands)
-@pytest.mark.parametrize("m,n,r,l,pad", [(300, 257, 31, 3, 0), (1025, 1024, 17, 8, 3), (2049, 513, 40, 1, 5),
-                                         (8193, 130, 9, 4, 0), (66, 16385, 33, 1, 0), (5000, 4099, 16, 8, 1)])
+# the first four on the FP64 units (K of one element, one row or column more than a
+# tile, K split eight ways); then one pass and several, ragged tiles, blocks of C past
+# 8192 rows and 16384 columns, a leading dimension longer than a row (padded operands)
+@pytest.mark.parametrize("m,n,r,l,pad", [(4, 1, 1, 1, 0), (300, 257, 31, 3, 0), (33, 65, 17, 1, 2),
+                                         (97, 4099, 5, 4, 1), (1025, 1024, 17, 8, 3), (2049, 513, 40, 1, 5),
+                                         (8193, 260, 9, 4, 0), (66, 16385, 33, 1, 0), (5000, 4099, 16, 8, 1)])
 def test_fp64_sketch_exact_on_scaled_integers(gn, H, m, n, r, l, pad):
     """30-bit integers times per-row or per-column powers of two: every product is
     exact in the digits, so a pass of 1024 rounds once and the sum of p passes at
-    most p - 1 times more, each relative to a partial sum of absolute values."""
+    most p - 1 times more, each relative to a partial sum of absolute values.  The
+    FP64 units round once per term."""
     g = torch.Generator().manual_seed(m + n)
     ints = lambda a, b, bits: torch.randint(-(1 << bits), 1 << bits, (a, b), generator=g)
     Ai, Xi, Yi = ints(m, n, 30), ints(n, r, 20), ints(m, r + l, 20)
@@ -59,7 +63,8 @@ def test_fp64_sketch_exact_on_scaled_integers(gn, H, m, n, r, l, pad):
         exact = (hi @ B).astype(np.longdouble) * 65536 + (lo @ B).astype(np.longdouble)
         size = left[at].abs().double().numpy() @ right.abs().double().numpy()
         err = np.abs(got[at].numpy().astype(np.longdouble) - exact).astype(np.float64)
-        passes = (left.shape[1] + 1023) // 1024
+        K = left.shape[1]
+        passes = (K + 1023) // 1024 if K * got.shape[0] * got.shape[1] > 1 << 24 else K + 8
         # (np.longdouble carries 64 bits or more: the reference itself rounds below 2^-64)
         assert np.all(err <= 2.0 ** -53 * (2 * passes) * size)
 
@@ -89,7 +94,7 @@ def test_fp64_sketch_propagates_nonfinite_like_the_units(gn, H):
 def test_fp64_sketch_runs_in_the_smallest_workspace(gn, H):
     """Without room for the slices the product runs on the FP64 units, and with
     an unaligned workspace the slices start at the next 256-byte boundary."""
-    m, n, r, l = 700, 600, 20, 10
+    m, n, r, l = 1500, 1100, 20, 10
     torch.manual_seed(4)
     A = torch.randn(m, n, dtype=torch.float64, device="cuda")
     X = torch.randn(n, r, dtype=torch.float64, device="cuda")
