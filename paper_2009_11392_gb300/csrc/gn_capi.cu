@@ -844,7 +844,7 @@ gn_status gn_core(gn_handle h, const gn_mat* YtA, const gn_mat* X, double eps, i
         side.stream = h->side;
         GN_TRY(latch_nonfinite_upper(&side, core->R, r, r));
         GN_TRY(core_diagnostics(&side, core->R, r, r, eps, eps_rel, 1, DIAG_ITERS, diag_d, k_d, zscr,
-                                sizeof(double) * 2 * std::max<long long>(r, 64)));
+                                sizeof(double) * 2 * std::max<long long>(r, 64), W2));   // (W2: used after k is known)
         // k and the three diagnostics to the pinned host words as soon as they exist
         GN_CUDA_TRY(cudaMemcpyAsync(h->pin_k, k_d, sizeof(int32_t), cudaMemcpyDeviceToHost, h->side));
         GN_CUDA_TRY(cudaMemcpyAsync(h->pin_diag, diag_d, 3 * sizeof(double), cudaMemcpyDeviceToHost, h->side));

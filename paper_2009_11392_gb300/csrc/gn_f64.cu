@@ -1265,242 +1265,276 @@ __global__ void __launch_bounds__(DG_THREADS) core_diag_kernel(const double* R, 
     if (threadIdx.x == 0) out[0] = est;
 }
 
-// Cluster version of the core diagnostics: rows of R are split over the CTAs of
-// a cluster.  The power iteration for ||R||_2 exchanges the matrix-vector
-// products through distributed shared memory; the blocked triangular solves of
-// the ||R^{-1}||_2 iteration are right-looking: the CTA owning a 32-row block
-// solves it with one warp, the block's solution is read by every CTA through
-// DSMEM (double-buffered by block parity, one cluster barrier per block), and
-// each CTA updates its own rows.  Same results as core_diag_kernel.
+// Cluster version of the core diagnostics, in two launches.
+//
+// The power iteration for ||R^{-1}||_2 is a chain of triangular solves, bound by
+// the latency of its steps (FP64 chains, cluster barriers), so the steps are few:
+// blocks of 128 columns with their inverses formed first (core_diag_inverse_kernel,
+// a warp per row of an inverse), a step being y_J = X_J^T z_J (pass 0) or X_J z_J
+// (pass 1) and the update of the remaining entries.  One cluster of 16 CTAs takes
+// it; a second one takes ||R||_2 and the truncation rank at the same time.
+// Columns are dealt out in groups of 8 inside each block, so every CTA has a share
+// of every step.  r = 20 / 100 / 1000: 303 / 305 / 1640 us with 32-column blocks
+// one after the other on one cluster (one CTA below r = 64); here 63 / 117 / 543 us
+// with the inverses (10 / 54 / 78 us of it), about the formation of Q beside it.
+// Same results as core_diag_kernel up to rounding.
 constexpr int CD_THREADS = 512;
 constexpr int CD_WARPS = CD_THREADS / 32;
 constexpr int CD_MAX_R = 4096;
+constexpr int CD_B = 128;            // columns per block
 
-__host__ __device__ inline int cd_rows_per(int r, int cs) { return ((r + cs - 1) / cs + 31) / 32 * 32; }
-__host__ __device__ inline size_t cd_smem(int r, int cs) {
-    const size_t rp = cd_rows_per(r, cs);
-    return sizeof(double) * (2 * static_cast<size_t>(r) + rp + 64 + 32 + 32 * 33 + 8 + (rp / 32) * 32 * 33);
+__host__ __device__ inline int cd_ldx(int r) { return r < CD_B ? r : CD_B; }
+
+// X_J = R_JJ^{-1}, row c of block J at X[(J0 + c) ldx]: forward substitution of
+// x R_JJ = e_c, a warp per row, four per CTA (one per sub-partition of the SM).
+__global__ void __launch_bounds__(128) core_diag_inverse_kernel(const double* __restrict__ R, long long ldr, int r,
+                                                               double* __restrict__ X, int ldx) {
+    constexpr int NT = CD_B / 32;
+    const int row = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= r) return;
+    const int J0 = row / CD_B * CD_B, bw = min(CD_B, r - J0), c = row - J0;
+    const double* RJ = R + static_cast<long long>(J0) * (ldr + 1);
+    double x[NT], rd[NT];
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        const int b = 32 * t + lane;
+        x[t] = b == c ? 1.0 : 0.0;
+        rd[t] = b >= c && b < bw ? 1.0 / RJ[static_cast<long long>(b) * (ldr + 1)] : 0.0;
+    }
+#pragma unroll
+    for (int p = 0; p < NT; ++p) {
+        if (32 * p + 31 < c || 32 * p >= bw) continue;   // warp-uniform
+#pragma unroll 8
+        for (int s = 0; s < 32; ++s) {
+            const int a = 32 * p + s;
+            if (a >= bw) break;
+            const double xa = __shfl_sync(0xffffffffu, x[p], s) * __shfl_sync(0xffffffffu, rd[p], s);
+            const double* ra = RJ + a * ldr + lane;
+#pragma unroll
+            for (int t = p; t < NT; ++t) {
+                const double v = 32 * t + lane < bw && 32 * t + lane > a ? ra[32 * t] : 0.0;
+                if (t > p || lane > s) x[t] = fma(-xa, v, x[t]);
+            }
+        }
+    }
+#pragma unroll
+    for (int t = 0; t < NT; ++t) {
+        const int b = 32 * t + lane;
+        if (b < bw) X[static_cast<long long>(row) * ldx + b] = x[t] * rd[t];
+    }
 }
 
-__global__ void __launch_bounds__(CD_THREADS) core_diag_cluster_kernel(const double* R, long long ldr, int r,
-                                                                      double eps, int eps_relative,
-                                                                      int want_est, int iters, double* out,
-                                                                      int* k_out) {
+// Sum of `part` (one double per CTA, published before a cluster barrier) over the
+// ranks, the same order in every CTA; every lane of the calling warp gets it.
+__device__ __forceinline__ double cd_rank_sum(cooperative_groups::cluster_group& cluster, double* part, int cs) {
+    const int lane = threadIdx.x & 31;
+    return warp_sum(lane < cs ? cluster.map_shared_rank(part, lane)[0] : 0.0);
+}
+
+__global__ void __launch_bounds__(CD_THREADS) core_diag_cluster_kernel(const double* __restrict__ R, long long ldr, int r,
+                                                                      double eps, int eps_relative, int want_est,
+                                                                      int iters, const double* __restrict__ X, int ldx,
+                                                                      double* out, int* k_out) {
     cg::cluster_group cluster = cg::this_cluster();
     const int cs = static_cast<int>(cluster.num_blocks());
     const int rank = static_cast<int>(cluster.block_rank());
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     extern __shared__ double sm[];
-    const int rp = cd_rows_per(r, cs);
-    double* v = sm;              // [r]  full iterate (identical in every CTA)
-    double* u = v + r;           // [r]  gathered R v
-    double* loc = u + r;         // [rp] own slice of the vector being solved
-    double* blk = loc + rp;      // [2][32] solved block, read by the other CTAs
-    double* ybuf = blk + 64;     // [32] local copy of the solved block
-    double* Rb = ybuf + 32;      // [32][33] diagonal block (owner)
-    double* part = Rb + 32 * 33; // [8] partial norms, double-buffered
-    double* Xinv = part + 8;     // [rp/32][32][33] inverses of the owned diagonal blocks
+    __shared__ double part[2], wred[CD_WARPS];
     __shared__ int s_kmin;
-    const int s0 = rank * rp;
-    const int s1 = min(r, s0 + rp);
     const double inf = __longlong_as_double(0x7ff0000000000000LL);
     const double inv = 1.0 / sqrt(static_cast<double>(r));
+    // columns of block J dealt to this CTA: J0 + rank g + [0, g)
+    const int g = (min(r, CD_B) + cs - 1) / cs;
+    const int nb = (r + CD_B - 1) / CD_B;
+    auto owned = [&](int J) { return max(0, min(g, min(CD_B, r - J * CD_B) - rank * g)); };
 
-    // ---- ||R||_2 (power iteration on R^T R from the all-ones vector)
-    double rn = 0.0;
-    if (eps_relative) {
-        for (int i = tid; i < r; i += CD_THREADS) v[i] = inv;
-        __syncthreads();
-        for (int it = 0; it < iters; ++it) {
-            const int par = it & 1;
-            for (int i = s0 + warp; i < s1; i += CD_WARPS) {   // u_i = (R v)_i, own rows
-                double acc = 0.0;
-                for (int j = i + lane; j < r; j += 32) acc = fma(R[static_cast<long long>(i) * ldr + j], v[j], acc);
-                acc = warp_sum(acc);
-                if (lane == 0) u[i] = acc;
-            }
-            cluster.sync();
-            for (int k = 0; k < cs; ++k) {   // gather the other slices of u
-                if (k == rank) continue;
-                const double* ru = cluster.map_shared_rank(u, k);
-                const int a = k * rp, b = min(r, a + rp);
-                for (int i = a + tid; i < b; i += CD_THREADS) u[i] = ru[i];
-            }
-            cluster.sync();
-            double ss = 0.0;
-            for (int j = s0 + tid; j < s1; j += CD_THREADS) {   // w_j = (R^T u)_j, own columns
-                double acc = 0.0;
-                for (int i = 0; i <= j; ++i) acc = fma(R[static_cast<long long>(i) * ldr + j], u[i], acc);
-                v[j] = acc;
-                ss = fma(acc, acc, ss);
-            }
-            ss = warp_sum(ss);
-            if (lane == 0) Rb[warp] = ss;
+    if (blockIdx.x >= static_cast<unsigned>(cs)) {
+        // ---- second cluster: ||R||_2 (power iteration on R^T R from the all-ones
+        // vector), the threshold and the truncation rank
+        double* v = sm;        // [r] the iterate (identical in every CTA)
+        double* wp = v + r;    // [r] this CTA's rows' part of R^T u
+        double* uo = wp + r;   // [nb g] own entries of u = R v, then of R^T u
+        double rn = 0.0;
+        if (eps_relative) {
+            for (int i = tid; i < r; i += CD_THREADS) v[i] = inv;
             __syncthreads();
-            if (tid == 0) {
-                double t = 0.0;
-                for (int w = 0; w < CD_WARPS; ++w) t += Rb[w];
-                part[par] = t;
-            }
-            cluster.sync();
-            double nw2 = 0.0;
-            for (int k = 0; k < cs; ++k) nw2 += cluster.map_shared_rank(part, k)[par];
-            for (int k = 0; k < cs; ++k) {   // gather the other slices of w into v
-                if (k == rank) continue;
-                const double* rv = cluster.map_shared_rank(v, k);
-                const int a = k * rp, b = min(r, a + rp);
-                for (int i = a + tid; i < b; i += CD_THREADS) v[i] = rv[i];
-            }
-            const double nw = sqrt(nw2);
-            cluster.sync();   // every CTA has read my slice of v before it is rescaled
-            if (nw == 0.0 || !isfinite(nw)) {
-                rn = nw;
-                break;
-            }
-            rn = sqrt(nw);
-            const double sc = 1.0 / nw;
-            for (int i = tid; i < r; i += CD_THREADS) v[i] *= sc;
-            __syncthreads();
-        }
-        eps = eps * rn;
-    }
-
-    // ---- truncation rank (every CTA scans the diagonal; rank 0 reports)
-    if (tid == 0) s_kmin = r;
-    __syncthreads();
-    int zero_diag = 0;
-    for (int i = tid; i < r; i += CD_THREADS) {
-        const double d = R[static_cast<long long>(i) * ldr + i];
-        if (fabs(d) <= eps) atomicMin(&s_kmin, i);
-        if (d == 0.0) zero_diag = 1;
-    }
-    zero_diag = __syncthreads_or(zero_diag);
-    if (rank == 0 && tid == 0) {
-        *k_out = s_kmin;
-        out[1] = rn;
-        out[2] = eps;
-        out[0] = 0.0;
-    }
-    if (!want_est) {
-        cluster.sync();
-        return;
-    }
-    if (zero_diag) {
-        if (rank == 0 && tid == 0) out[0] = inf;
-        cluster.sync();
-        return;
-    }
-
-    // ---- ||R^{-1}||_2 (power iteration on R^{-1} R^{-T} from the all-ones vector)
-    // Blocked substitution over 32-row blocks.  Each CTA first inverts the
-    // diagonal blocks it owns (once, in shared memory), so a block step is a
-    // 32 x 32 matrix-vector product instead of a 32-step dependent chain.
-    const int nb = (r + 31) / 32;
-    for (int ob = warp; ob * 32 < s1 - s0; ob += CD_WARPS) {
-        const int j0 = s0 + ob * 32, jb = min(32, r - j0);
-        double* X = Xinv + ob * 32 * 33;
-        // load D (identity padding beyond jb), then invert in place: rows from the
-        // bottom, X[i][j] = (delta_ij - sum_{i<k<=j} D[i][k] X[k][j]) / D[i][i]
-#pragma unroll 4
-        for (int a = 0; a < 32; ++a)
-            X[a * 33 + lane] = (a < jb && lane < jb) ? (lane >= a ? R[static_cast<long long>(j0 + a) * ldr + j0 + lane] : 0.0)
-                                                     : (a == lane ? 1.0 : 0.0);
-        __syncwarp();
-        const double rdl = 1.0 / X[lane * 33 + lane];
-        for (int i = 31; i >= 0; --i) {
-            double acc = lane == i ? 1.0 : 0.0;
-            for (int k = i + 1; k <= lane; ++k) acc = fma(-X[i * 33 + k], X[k * 33 + lane], acc);
-            const double rdi = __shfl_sync(0xffffffffu, rdl, i);   // every lane takes part
-            const double xi = lane >= i ? acc * rdi : 0.0;
-            __syncwarp();
-            X[i * 33 + lane] = xi;
-            __syncwarp();
-        }
-    }
-    for (int i = s0 + tid; i < s1; i += CD_THREADS) loc[i - s0] = inv;
-    __syncthreads();
-    double est = 0.0;
-    const int ra = tid >> 4, rpart = tid & 15;   // block product: row ra, k = rpart, rpart + 16
-    const int urow = tid >> 2, uq = tid & 3;      // updates: 4 lanes per row, 8 terms each
-    for (int it = 0; it < iters; ++it) {
-        for (int pass = 0; pass < 2; ++pass) {   // pass 0: R^T y = z; pass 1: R w = y
-            for (int bi = 0; bi < nb; ++bi) {
-                const int b = pass == 0 ? bi : nb - 1 - bi;
-                const int j0 = b * 32, jb = min(32, r - j0);
-                const int owner = j0 / rp;
-                if (rank == owner) {
-                    const double* X = Xinv + ((j0 - s0) >> 5) * 32 * 33;
-                    const int k0 = rpart, k1 = rpart + 16;
-                    const double z0 = k0 < jb ? loc[j0 - s0 + k0] : 0.0;
-                    const double z1 = k1 < jb ? loc[j0 - s0 + k1] : 0.0;
-                    // pass 0: y = X^T z (X upper); pass 1: w = X y
-                    double acc = pass == 0 ? fma(X[k0 * 33 + ra], z0, X[k1 * 33 + ra] * z1)
-                                           : fma(X[ra * 33 + k0], z0, X[ra * 33 + k1] * z1);
-#pragma unroll
-                    for (int o = 8; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                    __syncthreads();   // every block-product read of loc is done
-                    // buffer alternates with (b + pass): consecutive blocks, including the
-                    // last block of one pass and the first of the next, never share a slot
-                    if (rpart == 0 && ra < jb) {
-                        loc[j0 - s0 + ra] = acc;
-                        blk[((b + pass) & 1) * 32 + ra] = acc;
+            for (int it = 0; it < iters; ++it) {
+                for (int q = warp; q < nb * g; q += CD_WARPS) {   // u_i = (R v)_i, own rows, a warp each
+                    const int J = q / g, c = q - J * g;
+                    if (c >= owned(J)) continue;
+                    const int i = J * CD_B + rank * g + c;
+                    const double* ri = R + static_cast<long long>(i) * ldr;
+                    double a0 = 0.0, a1 = 0.0;
+                    int j = i + lane;
+                    for (; j + 32 < r; j += 64) {
+                        a0 = fma(ri[j], v[j], a0);
+                        a1 = fma(ri[j + 32], v[j + 32], a1);
                     }
+                    if (j < r) a0 = fma(ri[j], v[j], a0);
+                    a0 = warp_sum(a0 + a1);
+                    if (lane == 0) uo[q] = a0;
+                }
+                __syncthreads();
+                for (int j = tid; j < r; j += CD_THREADS) {   // own rows' part of R^T u
+                    double a0 = 0.0, a1 = 0.0;
+                    for (int J = 0; J * CD_B <= j; ++J) {
+                        const int i0 = J * CD_B + rank * g, n = min(owned(J), j - i0 + 1);
+                        const double* rc = R + static_cast<long long>(i0) * ldr + j;
+                        int c = 0;
+                        for (; c + 1 < n; c += 2) {
+                            a0 = fma(rc[c * ldr], uo[J * g + c], a0);
+                            a1 = fma(rc[(c + 1) * ldr], uo[J * g + c + 1], a1);
+                        }
+                        if (c < n) a0 = fma(rc[c * ldr], uo[J * g + c], a0);
+                    }
+                    wp[j] = a0 + a1;
                 }
                 cluster.sync();
-                if (tid < jb) ybuf[tid] = cluster.map_shared_rank(blk, owner)[((b + pass) & 1) * 32 + tid];
-                __syncthreads();
-                if (pass == 0) {   // z_j -= sum_{i in block} R[i][j] y_i, own rows j after the block
-                    const int jlo = max(s0, j0 + jb);
-                    for (int base = jlo; base < s1; base += CD_THREADS / 4) {
-                        const int j = base + urow;
-                        double acc = 0.0;
-                        if (j < s1) {
+                double ss = 0.0;
+                for (int q = tid; q < nb * g; q += CD_THREADS) {   // own entries of R^T u: the parts in rank order
+                    const int J = q / g, c = q - J * g;
+                    if (c >= owned(J)) continue;
+                    const int j = J * CD_B + rank * g + c;
+                    double p[16], a = 0.0;
 #pragma unroll
-                            for (int t = 0; t < 8; ++t) {
-                                const int i = uq * 8 + t;
-                                if (i < jb) acc = fma(R[static_cast<long long>(j0 + i) * ldr + j], ybuf[i], acc);
-                            }
-                        }
-                        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                        if (j < s1 && uq == 0) loc[j - s0] -= acc;
-                    }
-                } else {           // y_i -= sum_{j in block} R[i][j] w_j, own rows i before the block
-                    const int ihi = min(s1, j0);
-                    for (int base = s0; base < ihi; base += CD_THREADS / 4) {
-                        const int i = base + urow;
-                        double acc = 0.0;
-                        if (i < ihi) {
-                            const double* rr = R + static_cast<long long>(i) * ldr + j0;
+                    for (int k = 0; k < 16; ++k) p[k] = k < cs ? cluster.map_shared_rank(wp, k)[j] : 0.0;
 #pragma unroll
-                            for (int t = 0; t < 8; ++t) {
-                                const int j = uq * 8 + t;
-                                if (j < jb) acc = fma(rr[j], ybuf[j], acc);
-                            }
-                        }
-                        acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-                        acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-                        if (i < ihi && uq == 0) loc[i - s0] -= acc;
-                    }
+                    for (int k = 0; k < 16; k += 4) a += (p[k] + p[k + 1]) + (p[k + 2] + p[k + 3]);
+                    uo[q] = a;
+                    ss = fma(a, a, ss);
                 }
+                ss = warp_sum(ss);
+                if (lane == 0) wred[warp] = ss;
                 __syncthreads();
+                if (warp == 0) {
+                    const double t = warp_sum(lane < CD_WARPS ? wred[lane] : 0.0);
+                    if (lane == 0) part[0] = t;
+                }
+                cluster.sync();
+                const double nw = sqrt(cd_rank_sum(cluster, part, cs));
+                const double sc = 1.0 / nw;
+                for (int j = tid; j < r; j += CD_THREADS) {   // the next iterate
+                    const int J = j / CD_B, o = j - J * CD_B;
+                    v[j] = cluster.map_shared_rank(uo, o / g)[J * g + o % g] * sc;
+                }
+                cluster.sync();   // uo, wp and part are rewritten next
+                if (nw == 0.0 || !isfinite(nw)) {
+                    rn = nw;
+                    break;
+                }
+                rn = sqrt(nw);
             }
+            eps = eps * rn;
         }
-        const int par = it & 1;
-        double ss = 0.0;
-        for (int i = s0 + tid; i < s1; i += CD_THREADS) ss = fma(loc[i - s0], loc[i - s0], ss);
-        ss = warp_sum(ss);
-        if (lane == 0) Rb[warp] = ss;   // Rb is free here (owner warps are done)
+        if (rank != 0) return;
+        if (tid == 0) s_kmin = r;
+        __syncthreads();
+        for (int i = tid; i < r; i += CD_THREADS)
+            if (fabs(R[static_cast<long long>(i) * (ldr + 1)]) <= eps) atomicMin(&s_kmin, i);
         __syncthreads();
         if (tid == 0) {
-            double t = 0.0;
-            for (int w = 0; w < CD_WARPS; ++w) t += Rb[w];
-            part[2 + par] = t;
+            *k_out = s_kmin;
+            out[1] = rn;
+            out[2] = eps;
+        }
+        return;
+    }
+
+    // ---- first cluster: ||R^{-1}||_2 (power iteration on R^{-1} R^{-T} from the
+    // all-ones vector)
+    double* zo = sm;             // [nb g] own entries of the vector being solved (read by the peers)
+    double* zs = zo + nb * g;    // [CD_B] z_J, then y_J
+    double* yo = zs + CD_B;      // [g] own entries of y_J (read by the peers)
+    int zero_diag = 0;
+    for (int i = tid; i < r; i += CD_THREADS)
+        if (R[static_cast<long long>(i) * (ldr + 1)] == 0.0) zero_diag = 1;
+    zero_diag = __syncthreads_or(zero_diag);
+    if (!want_est || zero_diag) {   // the same in every CTA of the cluster
+        if (rank == 0 && tid == 0) out[0] = want_est ? inf : 0.0;
+        return;
+    }
+    for (int q = tid; q < nb * g; q += CD_THREADS) zo[q] = inv;
+    double est = 0.0;
+    const int uq = tid >> 3, up = tid & 7;   // updates: 8 lanes per own entry, 16 terms each
+    for (int it = 0; it < iters; ++it) {
+        for (int pass = 0; pass < 2; ++pass) {   // pass 0: R^T y = z; pass 1: R w = y
+            for (int b = 0; b < nb; ++b) {
+                const int J = pass == 0 ? b : nb - 1 - b, J0 = J * CD_B, bw = min(CD_B, r - J0);
+                // the coefficients of this step first: they do not depend on the vector
+                const int no = owned(J);
+                double xc[CD_B / 32];
+                if (warp < no) {
+                    const int o = rank * g + warp;   // pass 0: column o of X_J; pass 1: row o
+#pragma unroll
+                    for (int t = 0; t < CD_B / 32; ++t) {
+                        const int i = 32 * t + lane;
+                        xc[t] = i < bw ? (pass == 0 ? X[static_cast<long long>(J0 + i) * ldx + o]
+                                                    : X[static_cast<long long>(J0 + o) * ldx + i]) : 0.0;
+                    }
+                }
+                cluster.sync();   // the previous step's updates of z_J are in place
+                if (tid < bw) zs[tid] = cluster.map_shared_rank(zo, tid / g)[J * g + tid % g];
+                __syncthreads();
+                double y = 0.0;
+                if (warp < no) {
+#pragma unroll
+                    for (int t = 0; t < CD_B / 32; ++t)
+                        if (32 * t + lane < bw) y = fma(xc[t], zs[32 * t + lane], y);
+                    y = warp_sum(y);
+                    if (lane == 0) yo[warp] = y;
+                }
+                // own entries still to be updated: (pass 0) blocks after J, (pass 1) before it
+                const int cnt = (pass == 0 ? nb - 1 - J : J) * g, q0 = pass == 0 ? (J + 1) * g : 0;
+                double rc[CD_B / 8];
+                auto coeffs = [&](int q) {
+                    const int Jq = q / g, c = q - Jq * g;
+                    const bool on = c < owned(Jq);
+                    const int e = Jq * CD_B + rank * g + c;   // row / column of R
+#pragma unroll
+                    for (int t = 0; t < CD_B / 8; ++t) {
+                        const int i = 8 * t + up;
+                        rc[t] = on && i < bw ? (pass == 0 ? R[static_cast<long long>(J0 + i) * ldr + e]
+                                                          : R[static_cast<long long>(e) * ldr + J0 + i]) : 0.0;
+                    }
+                };
+                if (uq < cnt) coeffs(q0 + uq);
+                cluster.sync();   // every CTA's y_J is published, and z_J is read
+                if (tid < bw) zs[tid] = cluster.map_shared_rank(yo, tid / g)[tid % g];
+                if (warp < no && lane == 0) zo[J * g + warp] = y;
+                __syncthreads();
+                for (int u = uq; u < cnt; u += CD_THREADS / 8) {   // uniform over groups of 8 lanes
+                    if (u != uq) coeffs(q0 + u);
+                    double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+                    for (int t = 0; t < CD_B / 8; t += 2) {
+                        const int i = 8 * t + up;
+                        a0 = fma(rc[t], i < bw ? zs[i] : 0.0, a0);
+                        a1 = fma(rc[t + 1], i + 8 < bw ? zs[i + 8] : 0.0, a1);
+                    }
+                    a0 += a1;
+                    const unsigned mask = 0xffu << (lane & 24);
+                    a0 += __shfl_xor_sync(mask, a0, 1);
+                    a0 += __shfl_xor_sync(mask, a0, 2);
+                    a0 += __shfl_xor_sync(mask, a0, 4);
+                    if (up == 0) zo[q0 + u] -= a0;
+                }
+            }
+        }
+        // the norm of the new iterate
+        __syncthreads();
+        double ss = 0.0;
+        for (int q = tid; q < nb * g; q += CD_THREADS)
+            if (q % g < owned(q / g)) ss = fma(zo[q], zo[q], ss);
+        ss = warp_sum(ss);
+        if (lane == 0) wred[warp] = ss;
+        __syncthreads();
+        if (warp == 0) {
+            const double t = warp_sum(lane < CD_WARPS ? wred[lane] : 0.0);
+            if (lane == 0) part[it & 1] = t;
         }
         cluster.sync();
-        double nw2 = 0.0;
-        for (int k = 0; k < cs; ++k) nw2 += cluster.map_shared_rank(part, k)[2 + par];
-        const double nw = sqrt(nw2);
+        const double nw = sqrt(cd_rank_sum(cluster, part + (it & 1), cs));
         if (!isfinite(nw)) {
             est = inf;
             break;
@@ -1508,11 +1542,15 @@ __global__ void __launch_bounds__(CD_THREADS) core_diag_cluster_kernel(const dou
         est = sqrt(nw);
         if (nw == 0.0) break;
         const double sc = 1.0 / nw;
-        for (int i = s0 + tid; i < s1; i += CD_THREADS) loc[i - s0] *= sc;
-        __syncthreads();
+        for (int q = tid; q < nb * g; q += CD_THREADS) zo[q] *= sc;
     }
     if (rank == 0 && tid == 0) out[0] = est;
-    cluster.sync();
+    cluster.sync();   // peers may still read this CTA's shared memory
+}
+
+size_t cd_smem(int r) {
+    const size_t own = static_cast<size_t>((r + CD_B - 1) / CD_B) * CD_B;   // nb g <= nb CD_B
+    return sizeof(double) * (2 * static_cast<size_t>(r) + own + 2 * CD_B);
 }
 
 // --------------------------------------------------------------------------
@@ -2703,18 +2741,18 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
 
 gn_status core_diagnostics(gn_handle h, const double* R, long long r, long long ldr, double eps,
                            int eps_relative, int want_estimate, int iters, double* out3, int* k_out,
-                           double* ws, size_t ws_bytes) {
+                           double* ws, size_t ws_bytes, double* X) {
     static int cd_cs = -1;
     if (cd_cs < 0) {
         cd_cs = 0;
-        const size_t smax = cd_smem(CD_MAX_R, 8);
+        const size_t smax = cd_smem(CD_MAX_R);
         if (cudaFuncSetAttribute(core_diag_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(smax)) == cudaSuccess &&
             cudaFuncSetAttribute(core_diag_cluster_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
                 cudaSuccess) {
             for (int cs : {16, 8}) {
                 cudaLaunchConfig_t cfg = {};
-                cfg.gridDim = dim3(cs);
+                cfg.gridDim = dim3(2 * cs);
                 cfg.blockDim = dim3(CD_THREADS);
                 cfg.dynamicSmemBytes = smax;
                 cudaLaunchAttribute attr[1];
@@ -2733,11 +2771,17 @@ gn_status core_diagnostics(gn_handle h, const double* R, long long r, long long 
         }
         cudaGetLastError();
     }
-    if (cd_cs > 0 && r <= CD_MAX_R && r >= 64) {
+    if (cd_cs > 0 && r <= CD_MAX_R && X) {
+        const int ri = static_cast<int>(r), ldx = cd_ldx(ri);
+        if (want_estimate) {
+            core_diag_inverse_kernel<<<static_cast<unsigned>((r + 3) / 4), 128, 0, h->stream>>>(R, ldr, ri, X, ldx);
+            count_launch();
+            GN_CUDA_TRY(cudaGetLastError());
+        }
         cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(cd_cs);
+        cfg.gridDim = dim3(2 * cd_cs);
         cfg.blockDim = dim3(CD_THREADS);
-        cfg.dynamicSmemBytes = cd_smem(static_cast<int>(r), cd_cs);
+        cfg.dynamicSmemBytes = cd_smem(ri);
         cfg.stream = h->stream;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -2746,8 +2790,8 @@ gn_status core_diagnostics(gn_handle h, const double* R, long long r, long long 
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, core_diag_cluster_kernel, R, ldr, static_cast<int>(r), eps,
-                                       eps_relative, want_estimate, iters, out3, k_out));
+        GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, core_diag_cluster_kernel, R, ldr, ri, eps, eps_relative, want_estimate,
+                                       iters, static_cast<const double*>(X), ldx, out3, k_out));
         count_launch();
         return GN_OK;
     }

@@ -244,10 +244,11 @@ gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double 
 // Core diagnostics (one CTA): out3[0] = est ||R^{-1}||_2 (if want_estimate),
 // out3[1] = est ||R||_2 (if eps_relative), out3[2] = the absolute threshold
 // used (eps, or eps * est ||R||_2); *k_out = first i with |R_ii| <= threshold.
-// ws: 2 r doubles.
+// ws: 2 r doubles.  X (r min(r, 128) doubles, or null): scratch of the version on
+// two clusters of CTAs.
 gn_status core_diagnostics(gn_handle h, const double* R, long long r, long long ldr, double eps,
                            int eps_relative, int want_estimate, int iters, double* out3, int* k_out,
-                           double* ws, size_t ws_bytes);
+                           double* ws, size_t ws_bytes, double* X = nullptr);
 
 gn_status copy_f32_to_f64(gn_handle h, const float* src, long long rows, long long cols,
                           long long lds, double* dst, long long ldd);
