@@ -1790,6 +1790,7 @@ gn_status launch_cluster_panel(gn_handle h, const PanelCfg& pc, double* W, long 
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     const int Mi = static_cast<int>(M), j0i = static_cast<int>(j0);
+    if (pc.nb == 32 && panel_push_usable(M)) return launch_panel_push(h, W, ld, M, j0, jb, V, ldv, tau, T);
     if (pc.nb == 32) {
         cfg.dynamicSmemBytes = cluster_panel_smem<32>(rows_per);
         GN_CUDA_TRY(cudaLaunchKernelEx(&cfg, qr_panel_cluster_kernel<32>, W, ld, Mi, j0i, jb, V, ldv, tau, T,

@@ -185,6 +185,12 @@ size_t qr_ws_bytes(long long M, long long N, int sm_count);
 gn_status householder_qr(gn_handle h, double* W, long long M, long long N, long long ld,
                          double* Q, long long ldq, double* R, long long ldr,
                          double* ws, size_t ws_bytes);
+// One panel of the factorization (gn_panel.cu): columns j0 .. j0 + jb (jb <= 32) of
+// W (M x .), rows j0 on, M up to 3072: R and v in place, the explicit reflectors
+// into V (rows j0 on), tau and the compact-WY T (jb x jb).
+bool panel_push_usable(long long M);
+gn_status launch_panel_push(gn_handle h, double* W, long long ld, long long M, long long j0, int jb, double* V,
+                            long long ldv, double* tau, double* T);
 // The two halves of householder_qr: the factorization (R written, reflectors
 // kept in ws) and the formation of the thin Q from them (same W and ws).
 // oz (optional, >= qr_oz_ws_bytes(M, N)): with the look-ahead and at least two
