@@ -415,6 +415,8 @@ gn_status gn_batched_prepare(gn_handle h, int32_t count, const gn_problem* probs
     h->batched_count = count;
     h->batched_sk_tiles = sk_tiles;
     h->batched_mt = sk_mt;
+    h->batched_sk_bn = 0;
+    for (const TcGemm& g : sk) h->batched_sk_bn = std::max(h->batched_sk_bn, g.bn);
     h->batched_c_tiles = c_tiles;
     h->batched_ws = ws;
     return GN_OK;
@@ -485,12 +487,12 @@ gn_status gn_batched_run(gn_handle h, double eps, int32_t mode, void* ws, size_t
     (void)ws_bytes;
     const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(base + o_maps);
     GN_TRY(tc_launch_grouped(h, reinterpret_cast<const TcGemm*>(base + o_sk), 2 * count, maps, h->batched_sk_tiles,
-                             h->batched_mt));
+                             h->batched_mt, h->batched_sk_bn));
     const ProblemDev* pd = reinterpret_cast<const ProblemDev*>(base + o_p);
     batched_split3_kernel<<<dim3(16, count), 256, 0, h->stream>>>(pd);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
-    GN_TRY(tc_launch_grouped(h, reinterpret_cast<const TcGemm*>(base + o_c), 3 * count, maps, h->batched_c_tiles));
+    GN_TRY(tc_launch_grouped(h, reinterpret_cast<const TcGemm*>(base + o_c), 3 * count, maps, h->batched_c_tiles, 1, NMAX));
     static bool attr = false;
     if (!attr) {
         GN_CUDA_TRY(cudaFuncSetAttribute(batched_core_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

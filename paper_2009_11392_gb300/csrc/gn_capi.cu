@@ -208,6 +208,124 @@ gn_status sum_parts(gn_handle h, const float* parts, int nparts, long long strid
     return GN_OK;
 }
 
+// Whether Y^T A's tiles run as two half-K items adding into a zeroed output: when K = m
+// makes them much longer than AX's (bn0: AX's N tile).
+bool sketch_halves(long long m, long long n, long long bn0) { return 2 * 256 * m >= 3 * bn0 * n; }
+
+// K parts of a sketch's two products (stored apart in the workspace and summed): a
+// tile of AX is a chain of n / 64 K blocks on one SM and one of Y^T A of m / 64, and a
+// K block costs about its operand bytes (an SM reads ~60 B per cycle from L2: 48 KB
+// 0.4 us, 24 KB 0.28 us), so a tall, wide or small matrix leaves most SMs waiting for a
+// few long chains.  Parts are taken when the estimate below says so (in units of 128
+// bytes, ~1 ns; ~2.5 us per item, ~5 us for the launch that sums the parts or for
+// zeroing Y^T A under its halves; never below the time of A's passes through HBM).  bf16, m, n, r, l:
+// 20000, 1200, 300, 150: 99 -> 68 us; 2000, 16000, 300, 150: 115 -> 89; 1555, 7831,
+// 28, 14: 42 -> 21; 3001, 1777, 97, 49: 31 -> 21.  Square-ish sketches whose items just
+// fill the SMs gain nothing (12000, 6000, 60, 30) and stay whole, as large ones do.
+struct SketchSplit {
+    int s0, s1;      // parts of AX and of Y^T A (1: whole)
+    size_t b0, b1;   // bytes of their parts
+    size_t bytes() const { return b0 + b1; }
+};
+SketchSplit sketch_split(long long m, long long n, long long r, long long rl, int nsrc, int f8, int sms) {
+    SketchSplit p{1, 1, 0, 0};
+    if (r < 1 || rl < 1) return p;
+    const long long ke = f8 ? 128 : 64;
+    const long long kb0 = nsrc * ((n + ke - 1) / ke), kb1 = nsrc * ((m + ke - 1) / ke);
+    const long long bn0 = f8 ? 128 : std::min<long long>(256, (r + 63) / 64 * 64), bn1 = f8 ? 128 : 256;
+    const double c0 = kb0 * (128.0 + bn0), c1 = kb1 * (128.0 + bn1), item = 2500.0, launch = 5000.0;
+    const double t0 = static_cast<double>((m + 127) / 128 * ((r + bn0 - 1) / bn0));
+    const double t1 = static_cast<double>((rl + 127) / 128 * ((n + bn1 - 1) / bn1));
+    const double a_bytes = static_cast<double>(m) * n * (f8 ? 1 : 2 * nsrc);
+    const double hbm = a_bytes / 6000.0 * (a_bytes > 100e6 ? 2 : 1);   // one pass stays in L2 below ~100 MB
+    auto estimate = [&](int s0, int s1) {   // one round: the longest item; more: the mean load and half an item
+        const double i0 = c0 / s0 + item, i1 = c1 / s1 + item, most = std::max(i0, i1);
+        return std::max(hbm, t0 * s0 + t1 * s1 <= sms ? most : (t0 * s0 * i0 + t1 * s1 * i1) / sms + 0.5 * most);
+    };
+    const bool halves = !f8 && sketch_halves(m, n, bn0);
+    double best = estimate(1, halves ? 2 : 1) + (halves ? launch : 0.0);
+    for (double f : {0.75, 1.0, 1.25, 1.5, 2.0}) {
+        const double len = f * (t0 * c0 + t1 * c1) / sms;
+        const int s0 = static_cast<int>(std::max(1.0, std::min({16.0, kb0 / 8.0, std::ceil(c0 / len)})));
+        const int s1 = static_cast<int>(std::max(1.0, std::min({16.0, kb1 / 8.0, std::ceil(c1 / len)})));
+        const double e = estimate(s0, s1) + launch;
+        if (e < best && s0 + s1 > 2) {
+            best = e;
+            p.s0 = s0;
+            p.s1 = s1;
+        }
+    }
+    if (p.s0 > 1) p.b0 = align256(4 * static_cast<size_t>(p.s0) * m * round4(r));
+    if (p.s1 > 1) p.b1 = align256(4 * static_cast<size_t>(p.s1) * rl * round4(n));
+    return p;
+}
+
+// out = the sum of the parts (part c at parts + c stride, ld ldp, a multiple of 4), in
+// order, FP32; up to two matrices in one launch.
+struct SumJob {
+    const float* parts;
+    float* out;
+    long long stride, ldp, ldo;
+    int nparts, rows, cols, vec;
+};
+struct SumJobs {
+    SumJob j[2];
+};
+__global__ void __launch_bounds__(256) sum_parts_f32_kernel(const __grid_constant__ SumJobs jobs) {
+    const SumJob& s = jobs.j[blockIdx.y];
+    const int c4 = (s.cols + 3) / 4;
+    const long long total = static_cast<long long>(s.rows) * c4;
+    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < total; e += gridDim.x * 256LL) {
+        const int i = static_cast<int>(e / c4), j = static_cast<int>(e - static_cast<long long>(i) * c4) * 4;
+        const float* p = s.parts + i * s.ldp + j;
+        float4 a = *reinterpret_cast<const float4*>(p);
+        for (int c = 1; c < s.nparts; ++c) {
+            const float4 b = *reinterpret_cast<const float4*>(p + c * s.stride);
+            a = make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+        }
+        float* o = s.out + i * s.ldo + j;
+        if (s.vec && j + 4 <= s.cols) {
+            *reinterpret_cast<float4*>(o) = a;
+        } else {
+            o[0] = a.x;
+            if (j + 1 < s.cols) o[1] = a.y;
+            if (j + 2 < s.cols) o[2] = a.z;
+            if (j + 3 < s.cols) o[3] = a.w;
+        }
+    }
+}
+
+// The parts of g[0] (AX) and g[1] (Y^T A) into ws per the plan.
+void sketch_split_apply(const SketchSplit& p, TcGemm* g0, TcGemm* g1, const gn_mat* AX, const gn_mat* YtA, void* ws,
+                        SumJobs* jobs, int* njobs) {
+    *njobs = 0;
+    char* base = static_cast<char*>(ws);
+    auto cut = [&](TcGemm* g, const gn_mat* out, int parts, char* at) {
+        g->ksplit = parts < 2 ? 0 : parts;
+        if (parts < 2) return;
+        g->D = reinterpret_cast<float*>(at);
+        g->ldd = round4(out->cols);
+        g->part_stride = out->rows * g->ldd;
+        SumJob& j = jobs->j[(*njobs)++];
+        j = SumJob{g->D, static_cast<float*>(out->data), g->part_stride, g->ldd, out->ld, parts,
+                   static_cast<int>(out->rows), static_cast<int>(out->cols),
+                   (reinterpret_cast<uintptr_t>(out->data) & 15) == 0 && out->ld % 4 == 0};
+    };
+    cut(g0, AX, p.s0, base);
+    cut(g1, YtA, p.s1, base + p.b0);
+}
+
+gn_status sum_parts_f32(gn_handle h, const SumJobs& jobs, int njobs) {
+    long long most = 1;
+    for (int i = 0; i < njobs; ++i)
+        most = std::max(most, (static_cast<long long>(jobs.j[i].rows) * ((jobs.j[i].cols + 3) / 4) + 255) / 256);
+    const dim3 grid(static_cast<unsigned>(std::min<long long>(most, 16LL * h->sm_count)), static_cast<unsigned>(njobs));
+    sum_parts_f32_kernel<<<grid, 256, 0, h->stream>>>(jobs);
+    count_launch();
+    GN_CUDA_TRY(cudaGetLastError());
+    return GN_OK;
+}
+
 gn_status launch_sketch_tc(gn_handle h, const gn_mat* A, const gn_mat* X, const gn_mat* Y, gn_mat* AX,
                            gn_mat* YtA, void* ws, size_t ws_bytes) {
     const long long m = A->rows, n = A->cols, r = X->cols, rl = Y->cols;
@@ -255,7 +373,7 @@ gn_status launch_sketch_tc(gn_handle h, const gn_mat* A, const gn_mat* X, const 
     // the tiles keep bn = 256 (the fewest L2 bytes per flop) and run as two
     // half-K items each, so that every item costs about the same.
     g1.bn = 256;
-    g1.ksplit = (2 * 256LL * m >= 3LL * g0.bn * n) ? 2 : 1;
+    g1.ksplit = sketch_halves(m, n, g0.bn) ? 2 : 1;
     g1.a_mn = 1;
     g1.b_mn = 1;
     g1.nsrc = nsrc;
@@ -289,7 +407,15 @@ gn_status launch_sketch_tc(gn_handle h, const gn_mat* A, const gn_mat* X, const 
         if (sax < 2) g0.ksplit = 0, g0.part_stride = 0;
         if (syta < 2) g1.ksplit = 0, g1.part_stride = 0;
     }
+    // a few long chains: K parts, where the workspace has room for them
+    SumJobs jobs;
+    int njobs = 0;
+    const SketchSplit split = sketch_split(m, n, r, rl, nsrc, 0, h->sm_count);
+    const size_t pad = (256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255;
+    if (!pax && split.bytes() && ws && ws_bytes >= pad + split.bytes())
+        sketch_split_apply(split, &g0, &g1, AX, YtA, static_cast<char*>(ws) + pad, &jobs, &njobs);
     auto finish = [&]() -> gn_status {
+        if (njobs) return sum_parts_f32(h, jobs, njobs);
         if (!pax) return GN_OK;
         if (r > 0) GN_TRY(sum_parts(h, pax, sax, m * ldpx, m, r, ldpx, static_cast<float*>(AX->data), AX->ld));
         if (rl > 0) GN_TRY(sum_parts(h, pyta, syta, rl * ldpy, rl, n, ldpy, static_cast<float*>(YtA->data), YtA->ld));
@@ -380,6 +506,13 @@ gn_status launch_sketch_e4m3(gn_handle h, const gn_mat* A, const gn_mat* X, cons
         p.f8 = 1;
         return tc_launch(h, &p);
     }
+    SumJobs jobs;
+    int njobs = 0;
+    const SketchSplit split = sketch_split(m, n, r, rl, 1, 1, h->sm_count);
+    char* rest = static_cast<char*>(ws) + cv.off;
+    const size_t pad = (256 - (reinterpret_cast<uintptr_t>(rest) & 255)) & 255;
+    if (split.bytes() && ws_bytes >= cv.off + pad + split.bytes())
+        sketch_split_apply(split, &g0, &g1, AX, YtA, rest + pad, &jobs, &njobs);
     if (m >= n) {   // the longer-K GEMM first
         TcGemm t = p.g[0];
         p.g[0] = p.g[1];
@@ -387,7 +520,8 @@ gn_status launch_sketch_e4m3(gn_handle h, const gn_mat* A, const gn_mat* X, cons
     }
     p.ngemm = 2;
     p.f8 = 1;
-    return tc_launch(h, &p);
+    GN_TRY(tc_launch(h, &p));
+    return njobs ? sum_parts_f32(h, jobs, njobs) : GN_OK;
 }
 
 // dst (rows x cols, ldd) += src (rows x cols, lds), FP32 or FP64.
@@ -425,9 +559,11 @@ size_t update_scratch(long long m, long long n, long long r, long long l, int op
 
 // Scratch of sketch_block for an m x n block with rx = X's and ry = Y's columns.
 size_t block_sketch_ws(long long m, long long n, long long rx, long long ry, int op_dtype, int sms) {
-    if (op_dtype == GN_E4M3) return sketch_e4m3_ws(m, n, rx, ry - rx);
+    const size_t split = op_dtype == GN_F64 ? 0 : sketch_split(m, n, rx, ry, op_dtype == GN_BF16X2 ? 2 : 1,
+                                                               op_dtype == GN_E4M3, sms).bytes() + 256;
+    if (op_dtype == GN_E4M3) return sketch_e4m3_ws(m, n, rx, ry - rx) + split;
     if (op_dtype == GN_F64) return std::max(dgemm_fast_ws_bytes(m, rx, n, sms), dgemm_fast_ws_bytes(ry, n, m, sms)) + 1024;
-    return 1024;
+    return 1024 + split;
 }
 
 // The sketch products A X (m x rx) and Y^T A (ry x n) of any block A (m, n >= 1);
@@ -530,6 +666,7 @@ gn_status gn_create(gn_handle* out, void* stream) {
     h->batched_ws = nullptr;
     h->batched_count = h->batched_sk_tiles = h->batched_c_tiles = 0;
     h->batched_mt = 1;
+    h->batched_sk_bn = 256;
     h->batched_policy = 0;
     h->fp64_g = 0;
     h->fp64_tc = 1;
@@ -672,6 +809,9 @@ gn_status gn_workspace_size(int64_t m, int64_t n, int64_t r, int64_t l, int32_t 
     b = std::max(b, factors_ws(m, n, r, l, mixed, sms));
     b = std::max(b, hmt_ws(m, n, r, sms));
     b = std::max(b, error_ws_bytes(m, n, sms));
+    if (mixed)   // (gn_sketch runs its products whole without room for their K parts)
+        b = std::max(b, (op_dtype == GN_E4M3 ? sketch_e4m3_ws(m, n, r, l) : 0) + 512 +
+                            sketch_split(m, n, r, r + l, op_dtype == GN_BF16X2 ? 2 : 1, op_dtype == GN_E4M3, sms).bytes());
     if (!mixed) b = std::max(b, f64_fast_ws(m, n, r, l, sms));
     // (the factors' own check asks for less: the solve then takes fewer rows at a time)
     if (mixed) b = std::max(b, factors_ws(m, n, r, l, 1, sms) + trsm_oz_ws_bytes(m, r, OZ_DIGITS_SOLVE));

@@ -23,7 +23,7 @@ struct gn_handle_s {
     uint64_t wait_limit_ns;
     // batched path: the tables gn_batched_prepare uploaded into batched_ws
     void* batched_ws;
-    int batched_count, batched_sk_tiles, batched_c_tiles, batched_mt;
+    int batched_count, batched_sk_tiles, batched_c_tiles, batched_mt, batched_sk_bn;
     int batched_policy;        // tile policy of the next gn_batched_prepare
     int fp64_g;                // gn_factors: FP64 G even for FP32 Y^T A
     int fp64_tc;               // gn_factors: digit-sliced tensor-core FP64 products (FP32 AX)
@@ -130,6 +130,7 @@ struct TcParams {
     int snake_groups;
     int snake;   // set by tc_launch from snake_groups
     int max_ctas;
+    int stages, stage_bytes;   // BF16 ring (set by the launch)
 };
 
 // Host helpers (gn_tc.cu).
@@ -154,9 +155,9 @@ gn_status e4m3_sf_image(gn_handle h, const uint8_t* scale, long long tiles, uint
 gn_status e4m3_t_to_bf16(gn_handle h, const uint8_t* data_t, long long ld_t, const uint8_t* scale,
                          long long rows, long long cols, __nv_bfloat16* out, long long ldo);
 // Grouped launch: descriptors (tile_base ascending) and tensor maps already in
-// device memory; any number of GEMMs.
+// device memory; any number of GEMMs, N tiles of at most bn_max.
 gn_status tc_launch_grouped(gn_handle h, const TcGemm* dev_gemms, int ngemm, const CUtensorMap* dev_maps,
-                            int total_tiles, int mt = 1);
+                            int total_tiles, int mt, int bn_max);
 
 // --------------------------------------------------------------------------
 // FP64 / FP32 helper kernels (gn_f64.cu)

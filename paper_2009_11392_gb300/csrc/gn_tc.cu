@@ -7,15 +7,18 @@
 // optionally as K parts (added into D, or stored apart, K-aligned or not):
 //
 //   warp 0      : TMA producer -- cp.async.bulk.tensor tiles of both operands
-//                 into a shared-memory ring (128B swizzle; 4 stages of 48 KB
-//                 for 128-row tiles, 3 of 64 KB for 256-row tiles), one
+//                 into a shared-memory ring (128B swizzle; 3 to 12 stages by
+//                 the tile: tc_stages), one
 //                 mbarrier with a transaction count per stage;
 //   warp 1      : tcgen05.mma issuer (one thread) -- 128 x bn x 16 BF16 MMAs
 //                 with FP32 accumulators in tensor memory, two accumulator
 //                 buffers of 256 columns so the epilogue of one tile overlaps
 //                 the main loop of the next; also owns the TMEM allocation;
-//   warps 2..5  : epilogue -- tcgen05.ld 32 lanes x 32 columns per warp,
-//                 FP32 stores to global memory.
+//   warps 2..5  : epilogue -- tcgen05.ld 32 lanes x 32 columns per warp, turned
+//                 in shared memory so that a store instruction writes whole
+//                 128-byte row pieces (a lane holds a row: stored as it comes,
+//                 every instruction touches 32 rows: 1-3 % of a sketch, 8 % of
+//                 the nine-digit products, whose tiles have K = 1024).
 //
 // Operands are used in their natural row-major layout: the A operand of a
 // GEMM may be K-major (rows of A contiguous along K) or MN-major, likewise B.
@@ -27,6 +30,8 @@
 #include "gn_internal.cuh"
 
 #include <string.h>
+
+#include <algorithm>
 
 namespace gn {
 namespace {
@@ -63,9 +68,24 @@ struct Cfg {
     static constexpr int NACC = MT == 2 ? 1 : 2;
     static constexpr int TM = BM * MT;
     static constexpr int SF_STAGE = F8 ? (MT + 1) * 512 : 0;
-    static constexpr int SMEM = STG * STAGE + 1024 + (F8 ? 1024 + STG * SF_STAGE : 256);
+    static constexpr int BAR_BLOCK = F8 ? 1024 + STG * SF_STAGE : 256;
+    static constexpr int EPI_BYTES = 4 * 32 * 32 * 4;   // a 32 x 32 block per epilogue warp
+    static constexpr int SMEM = STG * STAGE + 1024 + BAR_BLOCK + EPI_BYTES;
 };
 constexpr uint32_t SF_TMEM_COL = 384;
+constexpr int MAX_STG = 12;   // stages at most (the barrier block has room for 2 MAX_STG + 7)
+
+// Stages of a BF16 launch whose widest N tile is bn: a stage takes ~1.3 us from its
+// load's issue to its MMAs' completion, so a narrow tile (its MMAs finish in 0.06 us
+// per 64 columns) is bound by the stages in flight.  The ring holds as many as fit:
+// 3 of 64 KB for 256 x 256 tiles, 4 of 48 KB for 128 x 256, 8 of 24 KB for 128 x 64
+// (a 128 x 64 tile, K block after K block: 0.34 us with 4 stages and the tile's fields
+// read again for every K block, 0.28 us with 8 and the fields in registers, about the
+// 60 B per cycle an SM reads from L2; e4m3 at 16384 x 8192, r = 500: 244 -> 197 us).
+void tc_stages(TcParams* p, int mt, int bn) {
+    p->stage_bytes = mt * BM * BK * 2 + bn * BK * 2;
+    p->stages = std::min(MAX_STG, (mt == 2 ? Cfg<2>::STG * Cfg<2>::STAGE : Cfg<1>::STG * Cfg<1>::STAGE) / p->stage_bytes);
+}
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
@@ -347,22 +367,23 @@ template <bool GROUPED, int MT, bool F8>
 __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __grid_constant__ TcParams p) {
     using K = Cfg<MT, F8>;
     constexpr int KE = F8 ? 128 : BK;                     // K elements per stage (128 bytes per row)
-    constexpr int STAGES = K::STG;
-    constexpr int STAGE_BYTES = K::STAGE;
+    // BF16 launches size their stages by the widest N tile (see tc_stages); e4m3 ones are fixed
+    const int STAGES = F8 ? K::STG : p.stages;
+    const int STAGE_BYTES = F8 ? K::STAGE : p.stage_bytes;
     constexpr int A_STAGE_BYTES = K::A_BYTES;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t base = (raw + 1023u) & ~1023u;            // 1024-aligned stage ring
     uint8_t* base_ptr = smem_raw + (base - raw);
-    const uint32_t bars = base + STAGES * STAGE_BYTES;        // barrier block
+    const uint32_t bars = base + K::STG * K::STAGE;           // barrier block
     const uint32_t sfs = bars + 1024;                         // F8: scale-factor images per stage
     auto full_bar = [&](int s) { return bars + 8u * s; };
-    auto empty_bar = [&](int s) { return bars + 8u * (STAGES + s); };
-    auto tfull_bar = [&](int a) { return bars + 8u * (2 * STAGES + a); };
-    auto tempty_bar = [&](int a) { return bars + 8u * (2 * STAGES + 2 + a); };
-    const uint32_t final_bar = bars + 8u * (2 * STAGES + 4);
-    const uint32_t stall_bar = bars + 8u * (2 * STAGES + 6);   // never completed (timeout-path test)
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + STAGES * STAGE_BYTES + 8 * (2 * STAGES + 5));
+    auto empty_bar = [&](int s) { return bars + 8u * (MAX_STG + s); };
+    auto tfull_bar = [&](int a) { return bars + 8u * (2 * MAX_STG + a); };
+    auto tempty_bar = [&](int a) { return bars + 8u * (2 * MAX_STG + 2 + a); };
+    const uint32_t final_bar = bars + 8u * (2 * MAX_STG + 4);
+    const uint32_t stall_bar = bars + 8u * (2 * MAX_STG + 6);   // never completed (timeout-path test)
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(base_ptr + K::STG * K::STAGE + 8 * (2 * MAX_STG + 5));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x >> 5;
@@ -412,25 +433,43 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                 const TileCoord c = decode_tile<GROUPED>(p, t);
                 const TcGemm& G = *gemm_of<GROUPED>(p, c.g);
                 const KRange kr = k_range(G, c.half);
-                const uint32_t bytes = A_STAGE_BYTES + G.bn * BK * 2 + K::SF_STAGE;
+                // Everything of the tile in registers: the loop below issues the loads of one K
+                // block, and a narrow tile's MMAs take less than reading these fields again (the
+                // asm statements' memory clobbers make the compiler reload them) and a division.
+                const bool a_mn = !F8 && G.a_mn, b_mn = G.b_mn;
+                const int bn = G.bn, nsrc = G.nsrc, n0 = c.tn * bn, m0 = c.tm * K::TM, nk = kr.nk;
+                const uint32_t bytes = A_STAGE_BYTES + bn * BK * 2 + K::SF_STAGE;
+                const uint8_t *sf_a[MT], *sf_b = nullptr;   // scale-factor images: K block 0, then a step per block
+                long long sf_astep = 0, sf_bstep = 0;
+                if (F8) {
+                    sf_astep = 512LL * (G.sfa_tr ? G.sfa_ld : 1);
+                    sf_bstep = 512LL * (G.sfb_tr ? G.sfb_ld : 1);
+#pragma unroll
+                    for (int hh = 0; hh < MT; ++hh) {
+                        const long long rb = min(m0 / BM + hh, G.sfa_rows - 1);
+                        sf_a[hh] = G.sfa + 512 * (G.sfa_tr ? rb : rb * G.sfa_ld);
+                    }
+                    const long long rb = min(n0 / BM, G.sfb_rows - 1);   // bn = 128: one tile
+                    sf_b = G.sfb + 512 * (G.sfb_tr ? rb : rb * G.sfb_ld);
+                }
+                int src = kr.kb0 / nk, kk = kr.kb0 - src * nk;   // source and K block inside its range
+                const CUtensorMap* ma = map_of<GROUPED>(p, G.a_map[src]);
+                const CUtensorMap* mb = map_of<GROUPED>(p, G.b_map[src]);
+                if (GROUPED) {   // maps written to device memory before the launch (grouped GEMMs have one source)
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
+                                     reinterpret_cast<uint64_t>(ma))
+                                 : "memory");
+                    asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
+                                     reinterpret_cast<uint64_t>(mb))
+                                 : "memory");
+                }
                 for (int kb = kr.kb0; kb < kr.kb1; ++kb) {
                     if (!mbar_wait(empty_bar(stage), ephase ^ 1u, limit, abort_flag)) {
                         latch(p.status, GN_ERR_TIMEOUT, 1, abort_flag);
                         ok = false;
                         break;
                     }
-                    const int src = kb / kr.nk;
-                    const int kk = kr.kk0 + (kb - src * kr.nk);
-                    const CUtensorMap* ma = map_of<GROUPED>(p, G.a_map[src]);
-                    const CUtensorMap* mb = map_of<GROUPED>(p, G.b_map[src]);
-                    if (GROUPED && kk == 0) {   // maps written to device memory before the launch
-                        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
-                                         reinterpret_cast<uint64_t>(ma))
-                                     : "memory");
-                        asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
-                                         reinterpret_cast<uint64_t>(mb))
-                                     : "memory");
-                    }
+                    const int kx = kr.kk0 + kk;   // K block
                     const uint32_t sa = base + stage * STAGE_BYTES;
                     const uint32_t sb = sa + A_STAGE_BYTES;
                     const uint32_t fb = full_bar(stage);
@@ -439,35 +478,31 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                     last_parity = (last_parity & ~(1u << stage)) | (ephase << stage);
 #pragma unroll
                     for (int hh = 0; hh < MT; ++hh) {
-                        const int m0 = c.tm * K::TM + hh * BM;
-                        if (!F8 && G.a_mn) {
-                            tma_load_2d(sa + hh * 16384, ma, fb, m0, kk * BK);
-                            tma_load_2d(sa + hh * 16384 + 8192, ma, fb, m0 + 64, kk * BK);
+                        const int mr = m0 + hh * BM;
+                        if (a_mn) {
+                            tma_load_2d(sa + hh * 16384, ma, fb, mr, kx * BK);
+                            tma_load_2d(sa + hh * 16384 + 8192, ma, fb, mr + 64, kx * BK);
                         } else {
-                            tma_load_2d(sa + hh * 16384, ma, fb, kk * KE, m0);
+                            tma_load_2d(sa + hh * 16384, ma, fb, kx * KE, mr);
                         }
-                        if (F8) {   // scale-factor image of this A tile
-                            const int rb = min(m0 / BM, G.sfa_rows - 1);
-                            const long long ti = G.sfa_tr ? static_cast<long long>(kk) * G.sfa_ld + rb
-                                                          : static_cast<long long>(rb) * G.sfa_ld + kk;
-                            bulk_load(sfs + stage * K::SF_STAGE + hh * 512, G.sfa + ti * 512, 512, fb);
-                        }
+                        if (F8) bulk_load(sfs + stage * K::SF_STAGE + hh * 512, sf_a[hh] + kx * sf_astep, 512, fb);
                     }
-                    if (F8) {       // and of the B tile (bn = 128: one tile)
-                        const int rb = min(c.tn * G.bn / BM, G.sfb_rows - 1);
-                        const long long ti = G.sfb_tr ? static_cast<long long>(kk) * G.sfb_ld + rb
-                                                      : static_cast<long long>(rb) * G.sfb_ld + kk;
-                        bulk_load(sfs + stage * K::SF_STAGE + MT * 512, G.sfb + ti * 512, 512, fb);
-                    }
-                    if (G.b_mn) {
-                        for (int j = 0; j < G.bn / 64; ++j)
-                            tma_load_2d(sb + 8192 * j, mb, fb, c.tn * G.bn + 64 * j, kk * BK);
+                    if (F8) bulk_load(sfs + stage * K::SF_STAGE + MT * 512, sf_b + kx * sf_bstep, 512, fb);
+                    if (b_mn) {
+                        for (int j = 0; j < bn; j += 64) tma_load_2d(sb + 128 * j, mb, fb, n0 + j, kx * BK);
                     } else {
-                        tma_load_2d(sb, mb, fb, kk * KE, c.tn * G.bn);
+                        tma_load_2d(sb, mb, fb, kx * KE, n0);
                     }
                     if (++stage == STAGES) {
                         stage = 0;
                         ephase ^= 1u;
+                    }
+                    if (++kk == nk) {   // the next source
+                        kk = 0;
+                        if (++src < nsrc) {
+                            ma = map_of<GROUPED>(p, G.a_map[src]);
+                            mb = map_of<GROUPED>(p, G.b_map[src]);
+                        }
                     }
                 }
             }
@@ -494,6 +529,13 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                 const KRange kr = k_range(G, c.half);
                 const int kb0 = kr.kb0, kb1 = kr.kb1;
                 const uint32_t idesc = F8 ? 0u : instr_desc_bf16(BM, G.bn, G.a_mn, G.b_mn);
+                const uint32_t idesc8 = F8 ? instr_desc_mxf8(BM, G.bn, 0, 0) : 0u;
+                // operand descriptors of stage 0 and their step per MMA (in 16-byte units: the
+                // address field is the low one), so that the loop only adds
+                const bool a_mn = !F8 && G.a_mn, b_mn = !F8 && G.b_mn;
+                const uint64_t adesc0 = smem_desc(base, a_mn ? 8192u : 16u, 1024u);
+                const uint64_t bdesc0 = smem_desc(base + A_STAGE_BYTES, b_mn ? 8192u : 16u, 1024u);
+                const uint32_t astep = a_mn ? 2048u / 16 : 32u / 16, bstep = b_mn ? 2048u / 16 : 32u / 16;
                 if (!mbar_wait(tempty_bar(acc), aphase ^ 1u, limit, abort_flag)) {
                     latch(p.status, GN_ERR_TIMEOUT, 3, abort_flag);
                     break;
@@ -507,8 +549,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                         break;
                     }
                     tc_fence_after();
-                    const uint32_t sa = base + stage * STAGE_BYTES;
-                    const uint32_t sb = sa + A_STAGE_BYTES;
+                    const uint32_t soff = static_cast<uint32_t>(stage * STAGE_BYTES) >> 4;
+                    const uint64_t ad0 = adesc0 + soff, bd0 = bdesc0 + soff;
                     if (F8) {
                         // scale factors of this stage into tensor memory (ordered
                         // before the MMAs below: same issuing thread), then
@@ -520,25 +562,19 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                         tc_cp_32x128b_x4(tsf + 8u, smem_desc_plain(sfs_s + 512u * MT));
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
-                            const uint64_t bd = smem_desc(sb + 32u * k, 16u, 1024u);
-                            const uint32_t id = instr_desc_mxf8(BM, G.bn, k, k);
+                            const uint32_t id = idesc8 | (static_cast<uint32_t>(k) << 4) | (static_cast<uint32_t>(k) << 29);
 #pragma unroll
                             for (int hh = 0; hh < MT; ++hh)
-                                tc_mma_mxf8(d_tmem + 256u * hh, smem_desc(sa + 16384u * hh + 32u * k, 16u, 1024u), bd, id,
-                                            tsf + 4u * hh, tsf + 8u, (kb != kb0 || k != 0) ? 1u : 0u);
+                                tc_mma_mxf8(d_tmem + 256u * hh, ad0 + 1024u * hh + 2u * k, bd0 + 2u * k, id, tsf + 4u * hh,
+                                            tsf + 8u, (kb != kb0 || k != 0) ? 1u : 0u);
                         }
                     } else {
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) {
-                            const uint64_t bd = G.b_mn ? smem_desc(sb + 2048u * k, 8192u, 1024u)
-                                                       : smem_desc(sb + 32u * k, 16u, 1024u);
 #pragma unroll
-                            for (int hh = 0; hh < MT; ++hh) {
-                                const uint32_t sah = sa + 16384u * hh;
-                                const uint64_t ad = G.a_mn ? smem_desc(sah + 2048u * k, 8192u, 1024u)
-                                                           : smem_desc(sah + 32u * k, 16u, 1024u);
-                                tc_mma_bf16(d_tmem + 256u * hh, ad, bd, idesc, (kb != kb0 || k != 0) ? 1u : 0u);
-                            }
+                            for (int hh = 0; hh < MT; ++hh)
+                                tc_mma_bf16(d_tmem + 256u * hh, ad0 + 1024u * hh + astep * k, bd0 + bstep * k, idesc,
+                                            (kb != kb0 || k != 0) ? 1u : 0u);
                         }
                     }
                     issued_any = true;
@@ -566,6 +602,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
     } else {
         // ------------------------------------------------------------ epilogue
         const int q = warp & 3;   // TMEM lane quarter this warp may access
+        float* epi = reinterpret_cast<float*>(base_ptr + K::STG * K::STAGE + K::BAR_BLOCK) + q * 1024;
         int acc = 0;
         uint32_t aphase = 0;
         bool stalled = false;
@@ -587,40 +624,58 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
             const bool stored_part = c.half && G.ksplit >= 2 && G.part_stride > 0;
             float* Dbase = stored_part ? G.D + (c.half - 1) * G.part_stride : G.D;
             for (int hh = 0; hh < MT; ++hh) {
-                const int row = c.tm * K::TM + hh * BM + q * 32 + lane;
-                const bool row_ok = row < G.M;
-                float* drow = Dbase + static_cast<long long>(row_ok ? row : 0) * G.ldd;
+                const int row0 = c.tm * K::TM + hh * BM + q * 32;   // this warp's 32 rows
+                const int nrow = min(32, G.M - row0);
                 for (int c0 = 0; c0 < G.bn; c0 += 32) {
                     uint32_t v[32];
                     tmem_ld32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + (acc * MT + hh) * 256 + c0, v);
                     const int col0 = c.tn * G.bn + c0;
-                    if (!row_ok || col0 >= G.N) continue;
+                    if (nrow <= 0 || col0 >= G.N) continue;   // warp-uniform
                     // columns of this chunk inside both the tile and D
                     const int ncol = min(min(32, G.bn - c0), G.N - col0);
-                    if (c.half && !stored_part) {   // part of the K range: add into the pre-zeroed D
-                        if (G.vec4 && ncol == 32) {
-                            float4* dst = reinterpret_cast<float4*>(drow + col0);
+                    // row `lane` into the block, its 16-byte pieces permuted by the row (no bank conflicts
+                    // either way)
 #pragma unroll
-                            for (int j = 0; j < 8; ++j)
-                                atomicAdd(dst + j, make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                               __uint_as_float(v[4 * j + 2]),
-                                                               __uint_as_float(v[4 * j + 3])));
-                        } else {
+                    for (int j = 0; j < 8; ++j)
+                        *reinterpret_cast<float4*>(epi + lane * 32 + ((j ^ (lane & 7)) << 2)) =
+                            make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
+                                        __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
+                    __syncwarp();
+                    const bool add = c.half && !stored_part;   // part of the K range: add into the pre-zeroed D
+                    float* d0 = Dbase + static_cast<long long>(row0) * G.ldd + col0;
+                    if (G.vec4 && ncol == 32) {   // four rows of eight 16-byte pieces per instruction
+                        const int j = lane & 7;
 #pragma unroll
-                            for (int j = 0; j < 32; ++j)
-                                if (j < ncol) atomicAdd(drow + col0 + j, __uint_as_float(v[j]));
+                        for (int it = 0; it < 8; ++it) {
+                            const int r = it * 4 + (lane >> 3);
+                            const float4 x = *reinterpret_cast<const float4*>(epi + r * 32 + ((j ^ (r & 7)) << 2));
+                            float4* dst = reinterpret_cast<float4*>(d0 + r * G.ldd) + j;
+                            if (r < nrow) {
+                                if (add) atomicAdd(dst, x);
+                                else *dst = x;
+                            }
                         }
-                    } else if (G.vec4 && ncol == 32) {
-                        float4* dst = reinterpret_cast<float4*>(drow + col0);
+                    } else if (ncol > 16) {       // a row per instruction
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            dst[j] = make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
-                                                 __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
-                    } else {
+                        for (int r = 0; r < 32; ++r) {
+                            const float f = epi[r * 32 + (((lane >> 2) ^ (r & 7)) << 2) + (lane & 3)];
+                            if (lane < ncol && r < nrow) {
+                                if (add) atomicAdd(d0 + r * G.ldd + lane, f);
+                                else d0[r * G.ldd + lane] = f;
+                            }
+                        }
+                    } else {                      // two short rows
 #pragma unroll
-                        for (int j = 0; j < 32; ++j)
-                            if (j < ncol) drow[col0 + j] = __uint_as_float(v[j]);
+                        for (int it = 0; it < 16; ++it) {
+                            const int r = 2 * it + (lane >> 4), x = lane & 15;
+                            const float f = epi[r * 32 + (((x >> 2) ^ (r & 7)) << 2) + (x & 3)];
+                            if (x < ncol && r < nrow) {
+                                if (add) atomicAdd(d0 + r * G.ldd + x, f);
+                                else d0[r * G.ldd + x] = f;
+                            }
+                        }
                     }
+                    __syncwarp();
                 }
             }
             tc_fence_before();
@@ -765,6 +820,9 @@ gn_status tc_launch(gn_handle h, TcParams* p) {
             }
         }
     }
+    int bn_max = 0;
+    for (int i = 0; i < p->ngemm; ++i) bn_max = std::max(bn_max, p->g[i].bn);
+    tc_stages(p, MT, bn_max);
     p->total_tiles = total;
     p->gg = nullptr;
     p->gmaps = nullptr;
@@ -788,10 +846,11 @@ gn_status tc_prepare_gemm(TcGemm* G, int tile_base, int mt, int f8) {
 }
 
 gn_status tc_launch_grouped(gn_handle h, const TcGemm* dev_gemms, int ngemm, const CUtensorMap* dev_maps,
-                            int total_tiles, int mt) {
+                            int total_tiles, int mt, int bn_max) {
     if (total_tiles <= 0 || ngemm <= 0) return GN_OK;
     TcParams p;
     memset(&p, 0, sizeof(p));
+    tc_stages(&p, mt, bn_max);
     p.gg = dev_gemms;
     p.gmaps = dev_maps;
     p.ngemm = ngemm;
