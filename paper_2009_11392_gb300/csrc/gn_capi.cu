@@ -667,6 +667,7 @@ gn_status gn_create(gn_handle* out, void* stream) {
     h->batched_count = h->batched_sk_tiles = h->batched_c_tiles = 0;
     h->batched_mt = 1;
     h->batched_sk_bn = 256;
+    h->batched_cluster = 0;
     h->batched_policy = 0;
     h->fp64_g = 0;
     h->fp64_tc = 1;

@@ -23,7 +23,7 @@ struct gn_handle_s {
     uint64_t wait_limit_ns;
     // batched path: the tables gn_batched_prepare uploaded into batched_ws
     void* batched_ws;
-    int batched_count, batched_sk_tiles, batched_c_tiles, batched_mt, batched_sk_bn;
+    int batched_count, batched_sk_tiles, batched_c_tiles, batched_mt, batched_sk_bn, batched_cluster;
     int batched_policy;        // tile policy of the next gn_batched_prepare
     int fp64_g;                // gn_factors: FP64 G even for FP32 Y^T A
     int fp64_tc;               // gn_factors: digit-sliced tensor-core FP64 products (FP32 AX)

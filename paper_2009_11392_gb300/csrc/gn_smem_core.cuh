@@ -219,13 +219,14 @@ __device__ inline void smem_form_q(const Smem& sm, int M, int N) {
 // lower: R^T y = z (forward); else R w = z (backward); z in shared memory.
 // 32 x 32 diagonal blocks are solved by warp 0 from a shared-memory copy with
 // reciprocal diagonals; the other rows are updated by the whole CTA.
+template <int T = BT>   // threads of the CTA
 __device__ inline void smem_tri_solve(const double* R, int ld, int N, double* z, int lower, double* Rb /*[32*33]*/) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nb = (N + 31) / 32;
     for (int bi = 0; bi < nb; ++bi) {
         const int b = lower ? bi : nb - 1 - bi;
         const int j0 = b * 32, jb = min(32, N - j0);
-        for (int e = tid; e < 32 * 32; e += BT) {
+        for (int e = tid; e < 32 * 32; e += T) {
             const int a = e >> 5, c = e & 31;
             Rb[a * 33 + c] = (a < jb && c < jb) ? R[(j0 + a) * ld + j0 + c] : 0.0;
         }
@@ -255,7 +256,7 @@ __device__ inline void smem_tri_solve(const double* R, int ld, int N, double* z,
         __syncthreads();
         // four partial sums per update (short FP64 dependency chains)
         if (lower) {
-            for (int jj = j0 + jb + tid; jj < N; jj += BT) {
+            for (int jj = j0 + jb + tid; jj < N; jj += T) {
                 double a[4] = {z[jj], 0.0, 0.0, 0.0};
 #pragma unroll
                 for (int i = 0; i < 32; ++i)
@@ -263,7 +264,7 @@ __device__ inline void smem_tri_solve(const double* R, int ld, int N, double* z,
                 z[jj] = (a[0] + a[1]) + (a[2] + a[3]);
             }
         } else {
-            for (int i = tid; i < j0; i += BT) {
+            for (int i = tid; i < j0; i += T) {
                 double a[4] = {z[i], 0.0, 0.0, 0.0};
                 const double* rr = R + i * ld + j0;
 #pragma unroll
@@ -276,7 +277,8 @@ __device__ inline void smem_tri_solve(const double* R, int ld, int N, double* z,
     }
 }
 
-__device__ inline double block_sum512(double s, double* red) {
+template <int T = BT>
+__device__ inline double block_sum(double s, double* red) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -284,7 +286,7 @@ __device__ inline double block_sum512(double s, double* red) {
     if (lane == 0) red[warp] = s;
     __syncthreads();
     double t = 0.0;
-    for (int w = 0; w < BW; ++w) t += red[w];
+    for (int w = 0; w < T / 32; ++w) t += red[w];
     return t;
 }
 
