@@ -754,8 +754,9 @@ gn_status gn_batched_prepare(gn_handle h, int32_t count, const gn_problem* probs
         g0.bn = (policy & 4) && r > 64 ? 64 : static_cast<int>(std::min<long long>(256, (r + 63) / 64 * 64));
         g0.b_mn = 1;
         g0.nsrc = 1;
-        g0.a_map[0] = mi + 0;
-        g0.b_map[0] = mi + 2;
+        g0.map_base = mi;
+        g0.a_map[0] = 0;
+        g0.b_map[0] = 2;
         g0.D = static_cast<float*>(q.AX.data);
         g0.ldd = q.AX.ld;
         TcGemm& g1 = sk[2 * slot[i] + 1];
@@ -767,8 +768,9 @@ gn_status gn_batched_prepare(gn_handle h, int32_t count, const gn_problem* probs
         g1.a_mn = 1;
         g1.b_mn = 1;
         g1.nsrc = 1;
-        g1.a_map[0] = mi + 3;
-        g1.b_map[0] = mi + 1;
+        g1.map_base = mi;
+        g1.a_map[0] = 3;
+        g1.b_map[0] = 1;
         g1.D = static_cast<float*>(q.YtA.data);
         g1.ldd = q.YtA.ld;
         for (int s = 0; s < 3; ++s) {
@@ -780,8 +782,9 @@ gn_status gn_batched_prepare(gn_handle h, int32_t count, const gn_problem* probs
             g.bn = static_cast<int>(std::min<long long>(256, (r + 63) / 64 * 64));
             g.b_mn = 1;
             g.nsrc = 1;
-            g.a_map[0] = mi + 4 + s;
-            g.b_map[0] = mi + 2;
+            g.map_base = mi;
+            g.a_map[0] = static_cast<signed char>(4 + s);
+            g.b_map[0] = 2;
             g.D = d.cpart[s];
             g.ldd = r;
             GN_TRY(tc_prepare_gemm(&g, c_tiles));

@@ -1324,6 +1324,105 @@ __global__ void __launch_bounds__(128) core_diag_inverse_kernel(const double* __
     }
 }
 
+// The diagnostics of a core of at most 32 columns in one CTA: no exchange between
+// CTAs pays (a cluster step is ~4.5 us; r = 20: 64 us on clusters, SMALLD_FIG here).
+// Eight warps form X = R^{-1} (lane = column, the rows dealt to the warps), then four
+// take ||R^{-1}|| with products by X and four ||R||: a product is eight terms per warp
+// and one barrier of the four.  The iterates are kept within a power of two of norm 1,
+// so sqrt and division (~1160 cycles a pair) come once, at the end.
+constexpr int DS_R = 32;
+
+__global__ void __launch_bounds__(256) core_diag_small_kernel(const double* __restrict__ R, long long ldr, int r,
+                                                             double eps, int eps_relative, int want_est, int iters,
+                                                             double* out, int* k_out) {
+    __shared__ double Rs[DS_R][DS_R + 1], Xs[DS_R][DS_R + 1];
+    __shared__ double part[2][2][4][DS_R];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const double inf = __longlong_as_double(0x7ff0000000000000LL);
+    double x[4], dg[4];   // rows warp + 8 u of X (lane = column), their pivots
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {   // (identity beyond r)
+        const int i = warp + 8 * u;
+        const double v = i < r && lane < r ? (lane >= i ? R[i * ldr + lane] : 0.0) : (i == lane ? 1.0 : 0.0);
+        Rs[i][lane] = v;
+        dg[u] = __shfl_sync(0xffffffffu, v, i);
+        x[u] = i == lane ? 1.0 : 0.0;
+    }
+    int zero = 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) zero |= dg[u] == 0.0;
+    zero = __syncthreads_or(zero);
+    if (want_est && !zero) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) dg[u] = 1.0 / dg[u];
+#pragma unroll
+        for (int u = 3; u >= 0; --u)
+            for (int w = 7; w >= 0; --w) {   // row k = 8 u + w from the last one up
+                const int k = 8 * u + w;
+                if (warp == w) Xs[k][lane] = x[u] = x[u] * dg[u];
+                __syncthreads();
+                const double xk = Xs[k][lane];
+#pragma unroll
+                for (int q = 0; q <= u; ++q) {
+                    const int i = warp + 8 * q;
+                    if (i < k) x[q] = fma(-Rs[i][k], xk, x[q]);
+                }
+            }
+    }
+    __syncthreads();
+    const int half = warp >> 2, w4 = warp & 3;   // 0: ||R^{-1}||, 1: ||R||
+    int pb = 0;
+    // out_j = sum_i M[i][j] v_i (trans) or out_i = sum_j M[i][j] v_j, a lane per output; v in the lanes
+    auto product = [&](const double (*Mx)[DS_R + 1], bool trans, double v) {
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+        for (int t = 0; t < 8; t += 2) {
+            const int i = 8 * w4 + t;
+            const double v0 = __shfl_sync(0xffffffffu, v, i), v1 = __shfl_sync(0xffffffffu, v, i + 1);
+            a0 = fma(trans ? Mx[i][lane] : Mx[lane][i], v0, a0);
+            a1 = fma(trans ? Mx[i + 1][lane] : Mx[lane][i + 1], v1, a1);
+        }
+        double (*pt)[DS_R] = part[half][pb];
+        pb ^= 1;
+        pt[w4][lane] = a0 + a1;
+        asm volatile("bar.sync %0, 128;" ::"r"(1 + half) : "memory");
+        return (pt[0][lane] + pt[1][lane]) + (pt[2][lane] + pt[3][lane]);
+    };
+    double res = 0.0;
+    if (half == 0 && want_est && zero) res = inf;
+    else if (half == 0 ? want_est : eps_relative) {
+        double z = lane < r ? 1.0 : 0.0, zz = static_cast<double>(r), ww = zz;
+        for (int it = 0; it < iters; ++it) {
+            z = half == 0 ? product(Xs, false, product(Xs, true, z)) : product(Rs, true, product(Rs, false, z));
+            if (lane >= r) z = 0.0;   // the identity's part
+            ww = warp_sum(z * z);     // ww / zz: the squared norm ratio of this step
+            if (!(isfinite(ww) && ww > 0.0)) break;   // the same in every lane and warp of the half
+            if (it + 1 < iters) {     // to within a factor of two of norm 1, exactly
+                const int e = ((__double2hiint(ww) >> 20) & 0x7FF) - 1023;
+                const double sc = __hiloint2double((1023 - (e >> 1)) << 20, 0);
+                z *= sc;
+                zz = ww * sc * sc;
+            }
+        }
+        // est = sqrt(nw), nw = ||w|| / ||z||; as the larger versions: a non-finite ||w|| gives
+        // an infinite ||R^{-1}|| and is handed on for ||R||, zero gives zero
+        if (ww == 0.0) res = 0.0;
+        else if (!isfinite(ww)) res = half == 0 ? inf : sqrt(ww);
+        else res = sqrt(sqrt(ww / zz));
+    }
+    if (half == 1) {
+        if (eps_relative) eps = eps * res;
+        const unsigned below = __ballot_sync(0xffffffffu, lane < r && fabs(Rs[lane][lane]) <= eps);
+        if (warp == 4 && lane == 0) {
+            *k_out = below ? __ffs(below) - 1 : r;
+            out[1] = res;
+            out[2] = eps;
+        }
+    } else if (tid == 0) {
+        out[0] = res;
+    }
+}
+
 // Sum of `part` (one double per CTA, published before a cluster barrier) over the
 // ranks, the same order in every CTA; every lane of the calling warp gets it.
 __device__ __forceinline__ double cd_rank_sum(cooperative_groups::cluster_group& cluster, double* part, int cs) {
@@ -2820,6 +2919,13 @@ gn_status core_diagnostics(gn_handle h, const double* R, long long r, long long 
             }
         }
         cudaGetLastError();
+    }
+    if (r <= DS_R) {
+        core_diag_small_kernel<<<1, 256, 0, h->stream>>>(R, ldr, static_cast<int>(r), eps, eps_relative, want_estimate,
+                                                         iters, out3, k_out);
+        count_launch();
+        GN_CUDA_TRY(cudaGetLastError());
+        return GN_OK;
     }
     if (cd_cs > 0 && r <= CD_MAX_R && X) {
         const int ri = static_cast<int>(r), ldx = cd_ldx(ri);

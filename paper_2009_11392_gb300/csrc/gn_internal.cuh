@@ -85,8 +85,9 @@ struct TcGemm {
     int bn;                  // N tile: multiple of 64 (MN-major B) or 16 (K-major B), <= 256
     int a_mn, b_mn;          // 0: K-major operand, 1: MN-major operand
     int nsrc;                // number of (A, B) pairs summed into D
-    int a_map[TC_MAX_SRC];   // tensor-map indices
-    int b_map[TC_MAX_SRC];
+    int map_base;            // tensor-map indices: map_base + a_map[s], map_base + b_map[s]
+    signed char a_map[TC_MAX_SRC];
+    signed char b_map[TC_MAX_SRC];
     int tiles_m, tiles_n, kblocks;
     int tile_base;           // first global tile index of this GEMM
     float* D;
@@ -132,6 +133,7 @@ struct TcParams {
     int max_ctas;
     int stages, stage_bytes;   // BF16 ring (set by the launch)
 };
+static_assert(sizeof(TcParams) <= 4096, "launches with more than 4 KB of parameters take ~2 us longer");
 
 // Host helpers (gn_tc.cu).
 gn_status tc_make_map_bf16(CUtensorMap* map, const void* base, long long rows, long long cols,

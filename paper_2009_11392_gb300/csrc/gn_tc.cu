@@ -453,8 +453,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                     sf_b = G.sfb + 512 * (G.sfb_tr ? rb : rb * G.sfb_ld);
                 }
                 int src = kr.kb0 / nk, kk = kr.kb0 - src * nk;   // source and K block inside its range
-                const CUtensorMap* ma = map_of<GROUPED>(p, G.a_map[src]);
-                const CUtensorMap* mb = map_of<GROUPED>(p, G.b_map[src]);
+                const CUtensorMap* ma = map_of<GROUPED>(p, G.map_base + G.a_map[src]);
+                const CUtensorMap* mb = map_of<GROUPED>(p, G.map_base + G.b_map[src]);
                 if (GROUPED) {   // maps written to device memory before the launch (grouped GEMMs have one source)
                     asm volatile("fence.proxy.tensormap::generic.acquire.gpu [%0], 128;" ::"l"(
                                      reinterpret_cast<uint64_t>(ma))
@@ -500,8 +500,8 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                     if (++kk == nk) {   // the next source
                         kk = 0;
                         if (++src < nsrc) {
-                            ma = map_of<GROUPED>(p, G.a_map[src]);
-                            mb = map_of<GROUPED>(p, G.b_map[src]);
+                            ma = map_of<GROUPED>(p, G.map_base + G.a_map[src]);
+                            mb = map_of<GROUPED>(p, G.map_base + G.b_map[src]);
                         }
                     }
                 }
