@@ -1325,7 +1325,7 @@ __global__ void __launch_bounds__(128) core_diag_inverse_kernel(const double* __
 }
 
 // The diagnostics of a core of at most 32 columns in one CTA: no exchange between
-// CTAs pays (a cluster step is ~4.5 us; r = 20: 64 us on clusters, SMALLD_FIG here).
+// CTAs pays (a cluster step is ~4.5 us; r = 20: 64 us on clusters, 31 here).
 // Eight warps form X = R^{-1} (lane = column, the rows dealt to the warps), then four
 // take ||R^{-1}|| with products by X and four ||R||: a product is eight terms per warp
 // and one barrier of the four.  The iterates are kept within a power of two of norm 1,

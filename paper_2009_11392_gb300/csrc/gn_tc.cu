@@ -69,7 +69,8 @@ struct Cfg {
     static constexpr int TM = BM * MT;
     static constexpr int SF_STAGE = F8 ? (MT + 1) * 512 : 0;
     static constexpr int BAR_BLOCK = F8 ? 1024 + STG * SF_STAGE : 256;
-    static constexpr int EPI_BYTES = 4 * 32 * 32 * 4;   // a 32 x 32 block per epilogue warp
+    static constexpr int EPI_BUFS = F8 ? 1 : 2;
+    static constexpr int EPI_BYTES = EPI_BUFS * 4 * 32 * 32 * 4;   // 32 x 32 blocks per epilogue warp
     static constexpr int SMEM = STG * STAGE + 1024 + BAR_BLOCK + EPI_BYTES;
 };
 constexpr uint32_t SF_TMEM_COL = 384;
@@ -195,7 +196,7 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
         : "memory");
 }
 
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
         "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -207,7 +208,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
           "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]),
           "=r"(v[31])
         : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+}
+
+// Waits for the warp's loads from tensor memory; v depends on it, so that no use moves above.
+__device__ __forceinline__ void tmem_wait(uint32_t (&v)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]), "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]), "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]), "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+                 :
+                 : "memory");
 }
 
 // Shared-memory matrix descriptor for tcgen05 (128B swizzle, version 1).
@@ -602,7 +610,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
     } else {
         // ------------------------------------------------------------ epilogue
         const int q = warp & 3;   // TMEM lane quarter this warp may access
-        float* epi = reinterpret_cast<float*>(base_ptr + K::STG * K::STAGE + K::BAR_BLOCK) + q * 1024;
+        float* epi = reinterpret_cast<float*>(base_ptr + K::STG * K::STAGE + K::BAR_BLOCK) + q * (1024 * K::EPI_BUFS);
         int acc = 0;
         uint32_t aphase = 0;
         bool stalled = false;
@@ -626,29 +634,30 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
             for (int hh = 0; hh < MT; ++hh) {
                 const int row0 = c.tm * K::TM + hh * BM + q * 32;   // this warp's 32 rows
                 const int nrow = min(32, G.M - row0);
-                for (int c0 = 0; c0 < G.bn; c0 += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(tmem_base + (static_cast<uint32_t>(q * 32) << 16) + (acc * MT + hh) * 256 + c0, v);
-                    const int col0 = c.tn * G.bn + c0;
-                    if (nrow <= 0 || col0 >= G.N) continue;   // warp-uniform
-                    // columns of this chunk inside both the tile and D
-                    const int ncol = min(min(32, G.bn - c0), G.N - col0);
+                // Columns of this tile inside D, 32 at a time: the next block's load from tensor memory
+                // is under way while this one is stored.
+                const int ncols = min(G.bn, G.N - c.tn * G.bn);
+                if (nrow <= 0) continue;                           // warp-uniform
+                const bool add = c.half && !stored_part;           // part of the K range: add into the pre-zeroed D
+                const uint32_t t0 = tmem_base + (static_cast<uint32_t>(q * 32) << 16) + (acc * MT + hh) * 256;
+                auto store = [&](const uint32_t (&v)[32], int c0) {
+                    const int col0 = c.tn * G.bn + c0, ncol = min(32, ncols - c0);
+                    float* blk = epi + (K::EPI_BUFS == 2 ? (c0 & 32) * 32 : 0);
                     // row `lane` into the block, its 16-byte pieces permuted by the row (no bank conflicts
                     // either way)
 #pragma unroll
                     for (int j = 0; j < 8; ++j)
-                        *reinterpret_cast<float4*>(epi + lane * 32 + ((j ^ (lane & 7)) << 2)) =
+                        *reinterpret_cast<float4*>(blk + lane * 32 + ((j ^ (lane & 7)) << 2)) =
                             make_float4(__uint_as_float(v[4 * j]), __uint_as_float(v[4 * j + 1]),
                                         __uint_as_float(v[4 * j + 2]), __uint_as_float(v[4 * j + 3]));
                     __syncwarp();
-                    const bool add = c.half && !stored_part;   // part of the K range: add into the pre-zeroed D
                     float* d0 = Dbase + static_cast<long long>(row0) * G.ldd + col0;
                     if (G.vec4 && ncol == 32) {   // four rows of eight 16-byte pieces per instruction
                         const int j = lane & 7;
 #pragma unroll
                         for (int it = 0; it < 8; ++it) {
                             const int r = it * 4 + (lane >> 3);
-                            const float4 x = *reinterpret_cast<const float4*>(epi + r * 32 + ((j ^ (r & 7)) << 2));
+                            const float4 x = *reinterpret_cast<const float4*>(blk + r * 32 + ((j ^ (r & 7)) << 2));
                             float4* dst = reinterpret_cast<float4*>(d0 + r * G.ldd) + j;
                             if (r < nrow) {
                                 if (add) atomicAdd(dst, x);
@@ -658,7 +667,7 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                     } else if (ncol > 16) {       // a row per instruction
 #pragma unroll
                         for (int r = 0; r < 32; ++r) {
-                            const float f = epi[r * 32 + (((lane >> 2) ^ (r & 7)) << 2) + (lane & 3)];
+                            const float f = blk[r * 32 + (((lane >> 2) ^ (r & 7)) << 2) + (lane & 3)];
                             if (lane < ncol && r < nrow) {
                                 if (add) atomicAdd(d0 + r * G.ldd + lane, f);
                                 else d0[r * G.ldd + lane] = f;
@@ -668,15 +677,28 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
 #pragma unroll
                         for (int it = 0; it < 16; ++it) {
                             const int r = 2 * it + (lane >> 4), x = lane & 15;
-                            const float f = epi[r * 32 + (((x >> 2) ^ (r & 7)) << 2) + (x & 3)];
+                            const float f = blk[r * 32 + (((x >> 2) ^ (r & 7)) << 2) + (x & 3)];
                             if (x < ncol && r < nrow) {
                                 if (add) atomicAdd(d0 + r * G.ldd + x, f);
                                 else d0[r * G.ldd + x] = f;
                             }
                         }
                     }
-                    __syncwarp();
+                    if (K::EPI_BUFS == 1) __syncwarp();   // (two blocks: the next barrier comes first)
+                };
+                uint32_t va[32], vb[32];
+                tmem_ld32_issue(t0, va);
+                for (int c0 = 0; c0 < ncols; c0 += 64) {
+                    tmem_wait(va);
+                    if (c0 + 32 < ncols) tmem_ld32_issue(t0 + c0 + 32, vb);
+                    store(va, c0);
+                    if (c0 + 32 < ncols) {
+                        tmem_wait(vb);
+                        if (c0 + 64 < ncols) tmem_ld32_issue(t0 + c0 + 64, va);
+                        store(vb, c0 + 32);
+                    }
                 }
+                if (K::EPI_BUFS == 2) __syncwarp();
             }
             tc_fence_before();
             mbar_arrive(tempty_bar(acc));
