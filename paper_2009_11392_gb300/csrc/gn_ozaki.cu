@@ -125,6 +125,16 @@ __device__ __forceinline__ unsigned long long digit_bias(int S) {
     return b;
 }
 
+// The digit u_s of U in slice s as a float, d_s 2^{-7(s+1)}: u below 256 put into the
+// mantissa of 2^23 instead of converted (conversions run at a quarter of the rate), the
+// bias and 2^23 taken off in the multiply-add that scales it; exact.
+template <int W>
+__device__ __forceinline__ float digit_value(unsigned long long U, int s) {
+    const unsigned u = s ? static_cast<unsigned>(U >> (7 * (W - 1 - s))) & 127u : static_cast<unsigned>(U >> (7 * (W - 1)));
+    const float sc = __int_as_float((127 - 7 * (s + 1)) << 23);   // 2^{-7(s+1)}
+    return fmaf(__uint_as_float(0x4B000000u | u), sc, -8388672.0f * sc);
+}
+
 // Digits of two entries adjacent along K, stored as one bf16 pair per slice
 // (out 4-byte aligned, slice_stride even).
 template <int W>
@@ -135,12 +145,22 @@ __device__ __forceinline__ void write_digits2(long long Y0, long long Y1, int S,
 #pragma unroll
     for (int s = 0; s < W; ++s) {
         if (s >= S) break;
-        const int sh = 7 * (W - 1 - s);
-        const unsigned u0 = s ? static_cast<unsigned>(U0 >> sh) & 127u : static_cast<unsigned>(U0 >> sh);
-        const unsigned u1 = s ? static_cast<unsigned>(U1 >> sh) & 127u : static_cast<unsigned>(U1 >> sh);
-        const float sc = __int_as_float((127 - 7 * (s + 1)) << 23);   // 2^{-7(s+1)}
-        const float2 f = make_float2(fmaf(__uint2float_rn(u0), sc, -64.0f * sc), fmaf(__uint2float_rn(u1), sc, -64.0f * sc));
-        *reinterpret_cast<__nv_bfloat162*>(out + s * slice_stride) = __float22bfloat162_rn(f);
+        *reinterpret_cast<__nv_bfloat162*>(out + s * slice_stride) =
+            __floats2bfloat162_rn(digit_value<W>(U0, s), digit_value<W>(U1, s));
+    }
+}
+
+// Eight entries adjacent along K: 16 bytes per slice (out 16-byte aligned).
+template <int W>
+__device__ __forceinline__ void write_digits8(const unsigned long long (&U)[8], int S, __nv_bfloat16* out,
+                                              long long slice_stride) {
+#pragma unroll
+    for (int s = 0; s < W; ++s) {
+        if (s >= S) break;
+        __nv_bfloat162 w[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) w[u] = __floats2bfloat162_rn(digit_value<W>(U[2 * u], s), digit_value<W>(U[2 * u + 1], s));
+        *reinterpret_cast<uint4*>(out + s * slice_stride) = *reinterpret_cast<const uint4*>(w);
     }
 }
 
@@ -157,8 +177,8 @@ struct OzOperand {
     unsigned long long* mx;   // [passes][rows]
     int rows, K, S;
     int passes;     // ceil(K / OZ_KPASS): pass p is K range [p OZ_KPASS, min(K, (p + 1) OZ_KPASS))
-    int tpr;        // K contiguous: threads per row, 32 (K <= 256) or 128
-    int rpc;        // rows per cluster: OZ_CS OZ_ST / tpr (K contiguous) or 32 (rows contiguous)
+    int tpr;        // K contiguous: threads per row, a warp per 256 of the pass
+    int rpc;        // rows per cluster: OZ_CS (OZ_ST / tpr) (K contiguous) or 32 (rows contiguous)
     int clusters;   // passes x ceil(rows / rpc): one cluster of OZ_CS CTAs per pass and rpc rows
 };
 struct OzSliceArgs {
@@ -183,10 +203,13 @@ __device__ __forceinline__ unsigned long long mx_word(unsigned long long m, floa
     return m ? static_cast<unsigned long long>(row_exponent<float>(m) + 1021) << 52 : 0ull;
 }
 
-// K contiguous (s_k == 1): tpr threads per row (a warp when K <= 256, else four
-// warps), OZ_ST / tpr rows per CTA, pairs of entries along K (8 entries per
-// thread); the row maximum is a shuffle, plus an exchange between the row's
-// warps when there are four.
+// K contiguous (s_k == 1): tpr threads per row (a warp per 256 entries of the pass, up
+// to four), OZ_ST / tpr rows per CTA, eight adjacent entries along K per thread (16-byte
+// stores per slice, 16-byte loads where the row is aligned); the row maximum is a
+// shuffle, plus an exchange between the row's warps when there are several.  Bound by
+// each CTA's chain (loads, row maximum, digits) as much as by memory: 3.6 GB over the
+// factors' eight launches in 0.95-0.98 ms (0.99 as pairs with converted digits); the
+// slices of a 20000 x 10000 FP64 sketch 3.4 -> 3.1 ms.
 template <int W, typename T>
 __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int q, int rank, OzSmem& sm) {
     const long long koff = static_cast<long long>(pass) * OZ_KPASS;
@@ -194,35 +217,46 @@ __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tpr = o.tpr;   // uniform over the cluster
     const int r = tid / tpr, l = tid - r * tpr;
-    const long long i = static_cast<long long>(q) * o.rpc + rank * (OZ_ST / tpr) + r;
-    const bool live = i < o.rows;
+    const int nw = tpr >> 5, rows = OZ_ST / tpr;   // (with three warps per row the last warp idles)
+    const long long i = static_cast<long long>(q) * o.rpc + rank * rows + r;
+    const bool live = r < rows && i < o.rows;
     const int K = min(OZ_KPASS, o.K - pass * OZ_KPASS);   // <= 8 tpr
     T v[8];
     unsigned long long m = 0;
+    const int k0 = 8 * l;
+    const T* rs = src + i * o.s_row + k0;
+    constexpr int VW = 16 / sizeof(T);
+    if (live && k0 + 8 <= K && (reinterpret_cast<uintptr_t>(rs) & 15) == 0) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int k = 2 * l + 2 * tpr * u;
-        v[2 * u] = live && k < K ? src[i * o.s_row + k] : T(0);
-        v[2 * u + 1] = live && k + 1 < K ? src[i * o.s_row + k + 1] : T(0);
-        m = max(m, max(abs_bits(v[2 * u]), abs_bits(v[2 * u + 1])));
+        for (int u = 0; u < 8; u += VW) {
+            const uint4 w = *reinterpret_cast<const uint4*>(rs + u);
+            const T* p = reinterpret_cast<const T*>(&w);
+#pragma unroll
+            for (int q = 0; q < VW; ++q) v[u + q] = p[q];
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = live && k0 + u < K ? rs[u] : T(0);
     }
 #pragma unroll
+    for (int u = 0; u < 8; ++u) m = max(m, abs_bits(v[u]));
+#pragma unroll
     for (int s = 16; s > 0; s >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, s));
-    if (tpr > 32) {   // four warps per row
+    if (nw > 1) {   // the row's warps
         if (lane == 0) sm.part[warp][0] = m;
         __syncthreads();
-        m = max(max(sm.part[4 * r][0], sm.part[4 * r + 1][0]), max(sm.part[4 * r + 2][0], sm.part[4 * r + 3][0]));
+        if (live)
+            for (int w = 0; w < nw; ++w) m = max(m, sm.part[nw * r + w][0]);
     }
     if (!live) return;   // no barrier follows in this path
     if (l == 0) o.mx[static_cast<long long>(pass) * o.rows + i] = mx_word(m, static_cast<T*>(nullptr));
     const int e = row_exponent<T>(m);
+    if (k0 >= K) return;
     const unsigned long long bias = digit_bias<W>(o.S);
-    __nv_bfloat16* out = o.out + i * o.ldk + koff;
+    unsigned long long U[8];   // entries past K are zero: ldk is K rounded up to 8
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        const int k = 2 * l + 2 * tpr * u;   // k + 1 < ldk: ldk is K rounded up to 8
-        if (k < K) write_digits2<W>(fixed_win<W>(v[2 * u], e), fixed_win<W>(v[2 * u + 1], e), o.S, bias, out + k, o.slice_stride);
-    }
+    for (int u = 0; u < 8; ++u) U[u] = static_cast<unsigned long long>(fixed_win<W>(v[u], e)) + bias;
+    write_digits8<W>(U, o.S, o.out + i * o.ldk + koff + k0, o.slice_stride);
 }
 
 // Rows contiguous (s_row == 1): the cluster's 8 CTAs split K into chunks of
@@ -327,7 +361,7 @@ OzOperand oz_operand(const void* src, long long s_row, long long s_k, long long 
     o.slice_stride = slice_stride;
     o.mx = mx;
     o.passes = static_cast<int>((K + OZ_KPASS - 1) / OZ_KPASS);
-    o.tpr = s_k == 1 ? (K <= 256 ? 32 : 128) : 0;
+    o.tpr = s_k == 1 ? 32 * static_cast<int>((std::min<long long>(K, OZ_KPASS) + 255) / 256) : 0;
     o.rpc = s_k == 1 ? OZ_CS * (OZ_ST / o.tpr) : 32;
     o.clusters = o.passes * static_cast<int>((rows + o.rpc - 1) / o.rpc);
     return o;
@@ -392,38 +426,75 @@ __device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, in
 // of the leading one).  A thread per column and row group (no division per
 // element; narrow products fill a block with more rows); each exact order is
 // an integer below 2^24 units, so it converts through a 32-bit integer.
-template <int NEX>
-__global__ void oz_combine_kernel(const float* __restrict__ D, long long d_stride, long long part_stride,
-                                  long long ldd, int norders, int nparts, int M, int N,
-                                  const unsigned long long* __restrict__ mxa,
-                                  const unsigned long long* __restrict__ mxb, long long mxb_part, double alpha,
-                                  double beta, double* __restrict__ C, long long ldc, int cw,
-                                  const __grid_constant__ OzDirect direct, int j0) {
+template <int NORD>
+__global__ void __launch_bounds__(256) oz_combine_kernel(
+    const float* __restrict__ D, long long d_stride, long long part_stride, long long ldd, int nparts, int M, int N,
+    const unsigned long long* __restrict__ mxa, const unsigned long long* __restrict__ mxb, long long mxb_part,
+    double alpha, double beta, double* __restrict__ C, long long ldc, int cw, const __grid_constant__ OzDirect direct,
+    int j0) {
+    constexpr int NEX = NORD > 7 ? 6 : 4, NEXACT = NORD < NEX ? NORD : NEX;
     // a block is cw columns by blockDim.x / cw rows (cw: a power of two >= min(N, 256), >= 32)
     const int j = blockIdx.x * cw + static_cast<int>(threadIdx.x) % cw;
-    const int rb = static_cast<int>(blockDim.x) / cw;
+    const int rb = static_cast<int>(blockDim.x) / cw, step = gridDim.y * rb;
     if (j >= N) return;
-    const int nexact = norders < NEX ? norders : NEX;
-    for (int i = blockIdx.y * rb + static_cast<int>(threadIdx.x) / cw; i < M; i += gridDim.y * rb) {
+    const bool unit = alpha == 1.0 || alpha == -1.0;
+    const int flip = alpha == -1.0 ? static_cast<int>(0x80000000u) : 0;
+    // one part of one entry from its orders
+    auto value = [&](const float (&d)[NORD], int q, int i) {
+        long long acc = 0;
+#pragma unroll
+        for (int o = 0; o < NEXACT; ++o)   // D_o is an integer number of units 2^{-7(o+2)}
+            acc += static_cast<long long>(__float2int_rn(d[o] * __int_as_float((127 + 7 * (o + 2)) << 23)))
+                   << (7 * (NEX - 1 - o));
+        float low = 0.0f;
+#pragma unroll
+        for (int o = NORD - 1; o >= NEX; --o) low += d[o];
+        // times 2^(ea + eb - 7 (NEX + 1)): a power of two built from its bits when normal
+        const unsigned long long ma = mxa[static_cast<long long>(q) * M + i], mb = mxb[q * mxb_part + j];
+        const int p = row_exponent<double>(ma) + row_exponent<double>(mb) - 7 * (NEX + 1);
+        const double x = fma(static_cast<double>(low), static_cast<double>(1ull << (7 * (NEX + 1))),
+                             static_cast<double>(acc));
+        // times 2^p by the exponent field where x and the result are normal, times alpha = +-1 by the
+        // sign (every FP64 instruction counts: the units run at 1/64 of the FP32 rate)
+        const int ex = ((__double2hiint(x) >> 20) & 0x7FF), er = ex + p;
+        double v = 0.0;
+        if (ex > 0 && er > 0 && er < 0x7FF) {
+            v = __hiloint2double((__double2hiint(x) + p * (1 << 20)) ^ flip, __double2loint(x));
+            if (!unit) v *= alpha;
+        } else if ((__double2hiint(x) << 1 | __double2loint(x)) != 0) {
+            v = alpha * ldexp(x, p);
+        }
+        if (NEX == 6 && direct.A && max(ma, mb) >= 0x7FF0000000000000ull) v = alpha * oz_direct_dot(direct, q, i, j0 + j);
+        return v;
+    };
+    int i = blockIdx.y * rb + static_cast<int>(threadIdx.x) / cw;
+    // one part: two rows at a time, both rows' orders loaded before either is used (32768 x
+    // 128, 8 orders: 80 -> 69 us); several parts already have that many loads in flight
+    if (nparts == 1)
+        for (; i + step < M; i += 2 * step) {
+            double* c = C + static_cast<long long>(i) * ldc + j;
+            double* c2 = c + step * ldc;
+            const float* p = D + static_cast<long long>(i) * ldd + j;
+            const float* p2 = p + step * ldd;
+            float d[NORD], e[NORD];
+#pragma unroll
+            for (int o = 0; o < NORD; ++o) {
+                d[o] = p[o * d_stride];
+                e[o] = p2[o * d_stride];
+            }
+            const double v = value(d, 0, i), v2 = value(e, 0, i + step);
+            *c = beta == 0.0 ? v : fma(beta, *c, v);
+            *c2 = beta == 0.0 ? v2 : fma(beta, *c2, v2);
+        }
+    for (; i < M; i += step) {
         double* c = C + static_cast<long long>(i) * ldc + j;
         double out = 0.0;
         for (int q = 0; q < nparts; ++q) {   // K parts (passes) in order, as separate passes would add them
-            const float* d = D + q * part_stride + static_cast<long long>(i) * ldd + j;
-            long long acc = 0;
-            for (int o = 0; o < nexact; ++o)   // D_o is an integer number of units 2^{-7(o+2)}
-                acc += static_cast<long long>(__float2int_rn(d[o * d_stride] * __int_as_float((127 + 7 * (o + 2)) << 23)))
-                       << (7 * (NEX - 1 - o));
-            float low = 0.0f;
-            for (int o = norders - 1; o >= NEX; --o) low += d[o * d_stride];
-            // times 2^(ea + eb - 7 (NEX + 1)): a power of two built from its bits when normal
-            const unsigned long long ma = mxa[static_cast<long long>(q) * M + i], mb = mxb[q * mxb_part + j];
-            const int p = row_exponent<double>(ma) + row_exponent<double>(mb) - 7 * (NEX + 1);
-            const double x = fma(static_cast<double>(low), static_cast<double>(1ull << (7 * (NEX + 1))),
-                                 static_cast<double>(acc));
-            double v = (p >= -1022 && p <= 1023)
-                           ? x * (alpha * __longlong_as_double(static_cast<long long>(p + 1023) << 52))
-                           : alpha * ldexp(x, p);
-            if (NEX == 6 && direct.A && max(ma, mb) >= 0x7FF0000000000000ull) v = alpha * oz_direct_dot(direct, q, i, j0 + j);
+            const float* p = D + q * part_stride + static_cast<long long>(i) * ldd + j;
+            float d[NORD];
+#pragma unroll
+            for (int o = 0; o < NORD; ++o) d[o] = p[o * d_stride];
+            const double v = value(d, q, i);
             out = q ? out + v : (beta == 0.0 ? v : fma(beta, *c, v));
         }
         *c = out;
@@ -578,10 +649,21 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
             if (digits > 7)
                 dd = OzDirect{static_cast<const double*>(A) + a_off, B + b_off, a_row, a_k, b_row, b_k,
                               in_place ? 0 : static_cast<int>(kc)};
-            auto* combine = digits > 7 ? oz_combine_kernel<6> : oz_combine_kernel<4>;
+            auto combine = [&]() {
+                switch (norders) {
+                    case 2: return oz_combine_kernel<2>;
+                    case 3: return oz_combine_kernel<3>;
+                    case 4: return oz_combine_kernel<4>;
+                    case 5: return oz_combine_kernel<5>;
+                    case 6: return oz_combine_kernel<6>;
+                    case 7: return oz_combine_kernel<7>;
+                    case 8: return oz_combine_kernel<8>;
+                    default: return oz_combine_kernel<9>;
+                }
+            }();
             combine<<<dim3(gx, gy), 256, 0, h->stream>>>(
-                o.d, d_stride, part_stride, o.ldd, norders, S, static_cast<int>(M), static_cast<int>(nb), o.mxa,
-                o.mxb + j0, N, alpha, beta_grp, C + j0, ldc, cw, dd, static_cast<int>(j0));
+                o.d, d_stride, part_stride, o.ldd, S, static_cast<int>(M), static_cast<int>(nb), o.mxa, o.mxb + j0, N,
+                alpha, beta_grp, C + j0, ldc, cw, dd, static_cast<int>(j0));
             count_launch();
             GN_CUDA_TRY(cudaGetLastError());
         }
