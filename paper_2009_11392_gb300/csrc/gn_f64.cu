@@ -1810,7 +1810,10 @@ bool small_gemm(long long M, long long N, long long K) {
 gn_status dgemm(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
                 long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                 long long ldc, double* ws, size_t ws_bytes) {
-    if (M > 0 && N > 0 && small_gemm(M, N, K))
+    // (also larger ones whose 64 x 64 tiles leave SMs idle: the adjoint's three 256 x 256 x 384
+    // products: 0.08 ms less)
+    const bool few_tiles = K >= 1 && ((M + GT - 1) / GT) * ((N + GT - 1) / GT) < h->sm_count && M * N * K <= 4 * SG_MAX_MACS;
+    if (M > 0 && N > 0 && (small_gemm(M, N, K) || few_tiles))
         return dgemm_small(h, M, N, K, alpha, A, lda, ta, A, lda, K, B, ldb, tb, beta, C, ldc);
     return dgemm_impl<double, double>(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, ws, ws_bytes);
 }
@@ -2589,8 +2592,7 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 // digits (2.6e-10 with the seven-digit updates before).
 // ---------------------------------------------------------------------------
 constexpr int TW = 128;              // columns per block
-constexpr int TW_ROWS = 32;          // rows of W per CTA
-constexpr int TW_THREADS = 512;      // a warp carries TW_ROWS / 16 rows
+constexpr int TW_NR = 2;             // rows of W per warp
 constexpr long long TRSM_ROWS = 32768;   // rows of F solved together (bounds the slices' scratch)
 
 // Rows of W_J in the stacked W, and its first row.
@@ -2653,8 +2655,10 @@ __global__ void __launch_bounds__(256) tri_scale_copy_kernel(const T* src, long 
 // coefficients scaled by the reciprocal pivots, Cs[a][b] = R_ab / R_aa, the
 // unknowns before their own scaling follow x_b -= x_a Cs[a][b], one shuffle and
 // one FMA per step of the chain; x_a / R_aa at the end.  A CTA keeps Cs in
-// shared memory for its 32 rows, two per warp (one row's shuffle overlaps the
-// other's FMA).  Bound by the FP64 rate: k = 1000: 38 M multiply-adds.
+// shared memory for its rows, two per warp (one row's shuffle overlaps the other's
+// FMA): 32 rows (16 warps) when that still gives every SM a CTA, else 8 (the CTA's
+// FP64 rate bounds it: 94 us for 32 rows, 28-53 for 8).  k = 1000: 38 M multiply-adds.
+template <int TW_THREADS>
 __global__ void __launch_bounds__(TW_THREADS) tri_w_kernel(const double* __restrict__ R, long long ldr, int k,
                                                           int trans, const int* __restrict__ e,
                                                           double* __restrict__ W) {
@@ -2663,9 +2667,11 @@ __global__ void __launch_bounds__(TW_THREADS) tri_w_kernel(const double* __restr
     double* rd = Cs + TW * (TW + 1); // [TW]
     const int J = blockIdx.y, J0 = J * TW, bw = min(TW, k - J0);
     const int rows = static_cast<int>(tw_rows(J, k, trans));
+    constexpr int TW_ROWS = TW_NR * TW_THREADS / 32;
     const int r0 = blockIdx.x * TW_ROWS;
     if (r0 >= rows) return;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    static_assert(TW_THREADS >= TW, "a thread per pivot");
     if (tid < TW) rd[tid] = tid < bw ? 1.0 / R[static_cast<long long>(J0 + tid) * (ldr + 1)] : 0.0;
     __syncthreads();
     for (int e = tid; e < TW * TW; e += TW_THREADS) {
@@ -2675,7 +2681,7 @@ __global__ void __launch_bounds__(TW_THREADS) tri_w_kernel(const double* __restr
         else Cs[a * (TW + 1) + b] = v * rd[a];
     }
     __syncthreads();
-    constexpr int NR = TW_ROWS / (TW_THREADS / 32), NT = TW / 32;
+    constexpr int NR = TW_NR, NT = TW / 32;
     double x[NR][NT];
     // row kk's position: its column inside J, or its row / column of R outside
     const int in0 = trans ? 0 : J0;   // rows [in0, in0 + bw) of W_J are the inverse's
@@ -2790,7 +2796,9 @@ gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ld
     constexpr size_t smem = sizeof(double) * (TW * (TW + 1) + TW);
     static bool attr = false;
     if (!attr) {
-        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         static_cast<int>(smem)));
+        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem)));
         attr = true;
     }
@@ -2807,8 +2815,12 @@ gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ld
         tri_scale_copy_kernel<double><<<cgrid, 256, 0, h->stream>>>(static_cast<const double*>(src), lds, Fs, lds_f, m, ki, e);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
-    tri_w_kernel<<<dim3(static_cast<unsigned>((k + TW_ROWS - 1) / TW_ROWS), static_cast<unsigned>(nb)), TW_THREADS,
-                   smem, h->stream>>>(R, ldr, ki, trans, e, W);
+    // 8 rows per CTA while one round of CTAs (one per SM: 133 KB) holds all rows
+    const long long w_rows = std::max(tw_base(nb - 1, k, trans) + tw_rows(nb - 1, k, trans), k);
+    const bool narrow = w_rows <= 8LL * h->sm_count;
+    const dim3 wgrid(static_cast<unsigned>((k + (narrow ? 7 : 31)) / (narrow ? 8 : 32)), static_cast<unsigned>(nb));
+    if (narrow) tri_w_kernel<128><<<wgrid, 128, smem, h->stream>>>(R, ldr, ki, trans, e, W);
+    else tri_w_kernel<512><<<wgrid, 512, smem, h->stream>>>(R, ldr, ki, trans, e, W);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
     if (few) return trsm_small(h, F, m, k, ldf, R, ldr, trans, W, Fs);

@@ -47,9 +47,12 @@ constexpr int OZ_PGRP = 4;       // passes per group of launches (slicing, produ
 size_t al256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 
 // Columns of C per GEMM launch: at least 256, more while the FP32 outputs of all
-// orders and K parts stay within 64 MB (short, wide products in one launch).
+// orders and K parts stay within 64 MB (short, wide products in one launch); 160 MB
+// with more than seven digits: their wide products (Y^T A of an FP64 sketch) then have
+// enough 256-row tiles, which need 62 B per cycle and SM from L2 where 128-row ones
+// need 94 of the ~60 there are (20000 x 10000, r = 500: 28.4 -> 26.3 ms).
 long long oz_npanel(long long M, long long N, long long parts, int orders) {
-    long long np = (64LL << 20) / (4LL * orders * std::max<long long>(M, 1) * std::max<long long>(parts, 1));
+    long long np = ((orders > 7 ? 160LL : 64LL) << 20) / (4LL * orders * std::max<long long>(M, 1) * std::max<long long>(parts, 1));
     np = std::max<long long>(np, OZ_NPANEL) / 16 * 16;
     return std::min<long long>(N, np);
 }
