@@ -788,19 +788,44 @@ gn_status launch_cfg(gn_handle h, const TcParams& p, int total_tiles) {
     return GN_OK;
 }
 
-// Tile shape: 256-row tiles (two MMAs sharing each B stage) when every GEMM has
-// at least 256 rows and the launch keeps enough tiles, else 128-row tiles.
-int pick_mt(const TcGemm* g, int ngemm, int sm_count) {
+// Tile shape: 128- or 256-row tiles (two MMAs sharing each B stage; every GEMM needs at
+// least 256 rows).  256-row tiles wherever they give four items per SM; below that by
+// an estimate of the launch.  A K block of an item costs its MMAs (2 bn cycles per 128
+// rows) or its operand bytes at the ~50 per cycle an SM gets from L2 with every SM
+// reading, whichever is more: 128 x 256 tiles ~980 cycles (512 of MMAs), 256 x 256 ones
+// ~1310 (1024).  An item's start and the part of its epilogue that nothing overlaps add
+// ~2500 (one accumulator: ~6000).  BF16's taller tiles have to win by 15 %, and products cut
+// into unaligned K parts keep the short ones (their items are short: 20000 x 1200, r =
+// 300: 58 us, 72 with 256 rows).  bf16 16384 x 8192, r = 500: 283 -> 250 us; e4m3 there:
+// 197 -> 171.
+double launch_cycles(const TcGemm* g, int ngemm, int mt, int f8, int sm_count) {
+    double sum = 0.0, most = 0.0, items = 0.0;
+    for (int i = 0; i < ngemm; ++i) {
+        const double kb = static_cast<double>(g[i].nsrc) * ((g[i].K + (f8 ? 127 : 63)) / (f8 ? 128 : 64));
+        const int s = g[i].ksplit >= 2 ? g[i].ksplit : 1;
+        const double t = kb / s * std::max(2.0 * mt * g[i].bn, (mt * 16384.0 + 128.0 * g[i].bn) / 50.0) + (mt == 2 ? 6000 : 2500);
+        const double n = static_cast<double>((g[i].M + 128 * mt - 1) / (128 * mt)) * ((g[i].N + g[i].bn - 1) / g[i].bn) * s;
+        sum += n * t;
+        items += n;
+        most = std::max(most, t);
+    }
+    return items <= sm_count ? most : sum / sm_count + 0.7 * most;
+}
+
+int pick_mt(const TcGemm* g, int ngemm, int f8, int sm_count) {
+    bool parts = false;
     long long tiles2 = 0;   // work items with 256-row tiles (a K-split tile counts twice)
     for (int i = 0; i < ngemm; ++i) {
         if (g[i].M < 2 * BM) return 1;
+        parts |= g[i].ksplit >= 2 && g[i].part_stride > 0 && g[i].kpart == 0;
         tiles2 += ((g[i].M + 2 * BM - 1) / (2 * BM)) * ((g[i].N + g[i].bn - 1) / g[i].bn) * (g[i].ksplit >= 2 ? g[i].ksplit : 1);
     }
-    return tiles2 >= 4LL * sm_count ? 2 : 1;   // keep enough tiles to fill the GPU
+    if (tiles2 >= 4LL * sm_count) return 2;
+    return !parts && (f8 ? 1.0 : 1.15) * launch_cycles(g, ngemm, 2, f8, sm_count) < launch_cycles(g, ngemm, 1, f8, sm_count) ? 2 : 1;
 }
 
 gn_status tc_launch(gn_handle h, TcParams* p) {
-    const int MT = pick_mt(p->g, p->ngemm, h->sm_count);
+    const int MT = pick_mt(p->g, p->ngemm, p->f8, h->sm_count);
     for (int i = 0; i < p->ngemm; ++i) {
         if (p->f8 && (p->g[i].a_mn || p->g[i].b_mn || p->g[i].bn != 128 || p->g[i].nsrc != 1 || !p->g[i].sfa ||
                       !p->g[i].sfb || p->g[i].sfa_rows < 1 || p->g[i].sfb_rows < 1))
