@@ -2567,7 +2567,7 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 }
 
 // ---------------------------------------------------------------------------
-// Triangular solve with the products on the tensor cores.  With blocks J of 128
+// Triangular solve with the products on the tensor cores.  With blocks J of 128 or 256
 // columns, F R = B gives
 //     F_J = (B_J - F_{<J} R_{<J,J}) R_JJ^{-1} = [F_{<J}, B_J] W_J,
 //     W_J = [-R_{<J,J} R_JJ^{-1}; R_JJ^{-1}],
@@ -2575,7 +2575,7 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 //     F_J = [B_J, F_{>J}] W_J,   W_J = [R_JJ^{-T}; -R_{J,>J}^T R_JJ^{-T}].
 // F_{<J} and B_J are adjacent columns of F, so each block is one product in
 // place (its operand is sliced before C is written).  The rows of every W_J are
-// triangular solves of 128 unknowns, independent of one another: all of them
+// triangular solves of a block's unknowns, independent of one another: all of them
 // run in the launch below, in FP64 by substitution.
 // In this form the rows of [F, B_J] and the columns of W_J mix magnitudes: B_J is
 // |R_:J| times F, and the slices are relative to the largest entry.  So B's
@@ -2584,23 +2584,33 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 // of a product is then of one size (without it the error grew from 2e-10 to 8e-10
 // of F at r = 2000).
 // Against 32-column substitution steps with a wide update per 128 columns this
-// leaves three launches per 128 columns and no substitution over the m rows
+// leaves three launches per block and no substitution over the m rows
 // (16 m k multiply-adds on the FP64 units).  m = 32768, k = 1000 (launches
-// summed): 5.83 -> 3.69 ms; m = 64, k = 1000: 3.5 -> 0.25 ms (its products on the
+// summed): 5.83 -> 3.69 ms (2.8 with blocks of 256 columns); m = 64, k = 1000: 3.5 -> 0.25 ms (its products on the
 // FP64 units), gn_apply there (32768 x 16384, 64 vectors) 4.90 -> 1.27 ms.
 // Error of F against FP64 substitution at m = 32768, k = 1000: 2.5e-12 with 8
 // digits (2.6e-10 with the seven-digit updates before).
 // ---------------------------------------------------------------------------
-constexpr int TW = 128;              // columns per block
+constexpr int TW = 128;              // columns per block, or per half of a wide one
 constexpr int TW_NR = 2;             // rows of W per warp
+// Blocks of 256 columns: half as many products, each F_{<J} sliced half as often, in
+// 256-column tiles (3e-8 m k^2 us saved), against rows of W that cost 3.6 times the
+// multiply-adds of a 128-column block's in a chain twice as long (85-110 us).  They pay
+// from m k^2 = 3e9 on.  gn_factors with 128- / 256-column blocks, us: 8192 x 500 447 / 482,
+// 8192 x 1000 1128 / 937, 12000 x 300 361 / 441, 20000 x 500 852 / 782, 32768 x 200
+// 472 / 518, 32768 x 1000 3406 / 2546, 32768 x 2000 12230 / 8108 (at k = 500 the CTAs of W
+// sized by its rows, below, take 55 us off the 128-column figure).
+inline bool tw_wide(long long m, long long k) {
+    return m >= 8192 && k > TW && static_cast<double>(m) * k * k >= 4e9;
+}
 constexpr long long TRSM_ROWS = 32768;   // rows of F solved together (bounds the slices' scratch)
 
-// Rows of W_J in the stacked W, and its first row.
-__host__ __device__ inline long long tw_rows(long long J, long long k, int trans) {
-    return trans ? k - J * TW : (J * TW + TW < k ? J * TW + TW : k);
+// Rows of W_J in the stacked W, and its first row (blocks of tb columns).
+__host__ __device__ inline long long tw_rows(long long J, long long k, int tb, int trans) {
+    return trans ? k - J * tb : (J * tb + tb < k ? J * tb + tb : k);
 }
-__host__ __device__ inline long long tw_base(long long J, long long k, int trans) {
-    return trans ? J * k - TW * (J * (J - 1) / 2) : TW * (J * (J + 1) / 2);
+__host__ __device__ inline long long tw_base(long long J, long long k, int tb, int trans) {
+    return trans ? J * k - tb * (J * (J - 1) / 2) : tb * (J * (J + 1) / 2);
 }
 
 // e_j = exponent of the largest |R_ij|, i <= j (trans: |R_ji|, i >= j); 0 for a zero
@@ -2654,112 +2664,143 @@ __global__ void __launch_bounds__(256) tri_scale_copy_kernel(const T* src, long 
 // the columns), trans: x R_JJ^T = e_c or -R[J, kk]^T (backward).  With the
 // coefficients scaled by the reciprocal pivots, Cs[a][b] = R_ab / R_aa, the
 // unknowns before their own scaling follow x_b -= x_a Cs[a][b], one shuffle and
-// one FMA per step of the chain; x_a / R_aa at the end.  A CTA keeps Cs in
-// shared memory for its rows, two per warp (one row's shuffle overlaps the other's
-// FMA): 32 rows (16 warps) when that still gives every SM a CTA, else 8 (the CTA's
-// FP64 rate bounds it: 94 us for 32 rows, 28-53 for 8).  k = 1000: 38 M multiply-adds.
-template <int TW_THREADS>
-__global__ void __launch_bounds__(TW_THREADS) tri_w_kernel(const double* __restrict__ R, long long ldr, int k,
-                                                          int trans, const int* __restrict__ e,
-                                                          double* __restrict__ W) {
+// one FMA per step of the chain; x_a / R_aa at the end.  A wide block is solved in two
+// halves of 128 columns, the first one's unknowns taken off the second's right-hand
+// side in between.  A CTA keeps Cs in shared memory for its rows, two per warp (one
+// row's shuffle overlaps the other's FMA), as many warps as let one round of CTAs (one
+// per SM: 133 KB) hold all rows, 4 to 16: the CTA's FP64 rate bounds it (128 columns:
+// 94 us for 32 rows, 28-53 for 8).  k = 1000: 38 M multiply-adds (wide: 92 M).
+template <int NH>
+__global__ void __launch_bounds__(512) tri_w_kernel(const double* __restrict__ R, long long ldr, int k,
+                                                   int trans, const int* __restrict__ e,
+                                                   double* __restrict__ W) {
     extern __shared__ double tw_sm[];
     double* Cs = tw_sm;              // [TW][TW + 1]
     double* rd = Cs + TW * (TW + 1); // [TW]
-    const int J = blockIdx.y, J0 = J * TW, bw = min(TW, k - J0);
-    const int rows = static_cast<int>(tw_rows(J, k, trans));
-    constexpr int TW_ROWS = TW_NR * TW_THREADS / 32;
-    const int r0 = blockIdx.x * TW_ROWS;
+    constexpr int TBW = NH * TW;
+    const int J = blockIdx.y, J0 = J * TBW, bw = min(TBW, k - J0);
+    const int rows = static_cast<int>(tw_rows(J, k, TBW, trans));
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x;
+    const int r0 = blockIdx.x * (TW_NR * nthr / 32);
     if (r0 >= rows) return;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    static_assert(TW_THREADS >= TW, "a thread per pivot");
-    if (tid < TW) rd[tid] = tid < bw ? 1.0 / R[static_cast<long long>(J0 + tid) * (ldr + 1)] : 0.0;
-    __syncthreads();
-    for (int e = tid; e < TW * TW; e += TW_THREADS) {
-        const int a = e / TW, b = e % TW;   // R_ab, a < b: read along rows
-        const double v = a < b && b < bw ? R[static_cast<long long>(J0 + a) * ldr + J0 + b] : 0.0;
-        if (trans) Cs[b * (TW + 1) + a] = v * rd[b];   // eliminates x_b from x_a, a < b
-        else Cs[a * (TW + 1) + b] = v * rd[a];
-    }
-    __syncthreads();
     constexpr int NR = TW_NR, NT = TW / 32;
-    double x[NR][NT];
-    // row kk's position: its column inside J, or its row / column of R outside
     const int in0 = trans ? 0 : J0;   // rows [in0, in0 + bw) of W_J are the inverse's
-    int kk[NR];
-    bool any = false;
+    double x[NR][NT], x1[NR][NT];     // this half's unknowns; the first half's
+    double* out = W + tw_base(J, k, TBW, trans) * TBW;
 #pragma unroll
-    for (int u = 0; u < NR; ++u) {
-        kk[u] = r0 + NR * warp + u;
-        const int c = kk[u] - in0;
-        const bool unit = c >= 0 && c < bw;
+    for (int q = 0; q < NH; ++q) {
+        const int hh = trans ? NH - 1 - q : q;
+        const int H0 = J0 + hh * TW, hw = min(TW, k - H0);   // hw <= 0: the last block's missing half
+        // row kk's right-hand side in this half: its column inside J, or its row / column of R outside
 #pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            const int b = 32 * t + lane;
-            double v = 0.0;
-            if (unit) v = b == c ? 1.0 : 0.0;
-            else if (kk[u] < rows && b < bw)
-                v = trans ? -R[static_cast<long long>(J0 + b) * ldr + J0 + kk[u]]
-                          : -R[static_cast<long long>(kk[u]) * ldr + J0 + b];
-            x[u][t] = v;
+        for (int u = 0; u < NR; ++u) {
+            const int kk = r0 + NR * warp + u, c = kk - in0;
+            const bool unit = c >= 0 && c < bw;
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                const int b = 32 * t + lane;
+                double v = 0.0;
+                if (unit) v = hh * TW + b == c ? 1.0 : 0.0;
+                else if (kk < rows && b < hw)
+                    v = trans ? -R[static_cast<long long>(H0 + b) * ldr + J0 + kk]
+                              : -R[static_cast<long long>(kk) * ldr + H0 + b];
+                x[u][t] = v;
+            }
         }
-        any |= kk[u] < rows;
-    }
-    if (!any) return;   // warp-uniform; no barrier follows
-    if (!trans) {
+        if (NH == 2 && q == 1) {   // x -= x1 R_12 (trans: x1 R_12^T), R_12 = R[J0.., J0 + TW..]
+            const int w2 = min(TW, k - J0 - TW);
+            if (w2 > 0) {
+                __syncthreads();
+                for (int i = tid; i < TW * TW; i += nthr) {
+                    const int a = i / TW, b = i % TW;
+                    const double v = b < w2 ? R[static_cast<long long>(J0 + a) * ldr + J0 + TW + b] : 0.0;
+                    if (trans) Cs[b * (TW + 1) + a] = v;
+                    else Cs[a * (TW + 1) + b] = v;
+                }
+                __syncthreads();
 #pragma unroll
-        for (int p = 0; p < NT; ++p) {
-            if (32 * p >= bw) break;
+                for (int p = 0; p < NT; ++p)
 #pragma unroll 8
-            for (int s = 0; s < 32; ++s) {
-                const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+                    for (int s = 0; s < 32; ++s) {
+                        const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
 #pragma unroll
-                for (int u = 0; u < NR; ++u) {
-                    const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
+                        for (int u = 0; u < NR; ++u) {
+                            const double xa = __shfl_sync(0xffffffffu, x1[u][p], s);
 #pragma unroll
-                    for (int t = p; t < NT; ++t)
-                        if (t > p || lane > s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
+                            for (int t = 0; t < NT; ++t) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
+                        }
+                    }
+            }
+        }
+        if (q > 0) __syncthreads();
+        for (int i = tid; i < TW; i += nthr) rd[i] = i < hw ? 1.0 / R[static_cast<long long>(H0 + i) * (ldr + 1)] : 0.0;
+        __syncthreads();
+        for (int i = tid; i < TW * TW; i += nthr) {
+            const int a = i / TW, b = i % TW;   // R_ab, a < b: read along rows
+            const double v = a < b && b < hw ? R[static_cast<long long>(H0 + a) * ldr + H0 + b] : 0.0;
+            if (trans) Cs[b * (TW + 1) + a] = v * rd[b];   // eliminates x_b from x_a, a < b
+            else Cs[a * (TW + 1) + b] = v * rd[a];
+        }
+        __syncthreads();
+        if (!trans) {
+#pragma unroll
+            for (int p = 0; p < NT; ++p) {
+                if (32 * p >= hw) break;
+#pragma unroll 8
+                for (int s = 0; s < 32; ++s) {
+                    const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+#pragma unroll
+                    for (int u = 0; u < NR; ++u) {
+                        const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
+#pragma unroll
+                        for (int t = p; t < NT; ++t)
+                            if (t > p || lane > s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
+                    }
+                }
+            }
+        } else {
+#pragma unroll
+            for (int p = NT - 1; p >= 0; --p) {
+                if (32 * p >= hw) continue;
+#pragma unroll 8
+                for (int s = 31; s >= 0; --s) {
+                    const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+#pragma unroll
+                    for (int u = 0; u < NR; ++u) {
+                        const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
+#pragma unroll
+                        for (int t = 0; t <= p; ++t)
+                            if (t < p || lane < s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
+                    }
                 }
             }
         }
-    } else {
 #pragma unroll
-        for (int p = NT - 1; p >= 0; --p) {
-            if (32 * p >= bw) continue;
-#pragma unroll 8
-            for (int s = 31; s >= 0; --s) {
-                const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
-#pragma unroll
-                for (int u = 0; u < NR; ++u) {
-                    const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
-#pragma unroll
-                    for (int t = 0; t <= p; ++t)
-                        if (t < p || lane < s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
-                }
-            }
-        }
-    }
-    double* out = W + tw_base(J, k, trans) * TW;
-#pragma unroll
-    for (int u = 0; u < NR; ++u)
-        if (kk[u] < rows) {
-            const int c = kk[u] - in0;
+        for (int u = 0; u < NR; ++u) {
+            const int kk = r0 + NR * warp + u, c = kk - in0;
             const double sc = c >= 0 && c < bw ? __longlong_as_double(static_cast<long long>(1023 + e[J0 + c]) << 52) : 1.0;
 #pragma unroll
-            for (int t = 0; t < NT; ++t)
-                if (32 * t + lane < bw)
-                    out[static_cast<long long>(kk[u]) * TW + 32 * t + lane] = x[u][t] * rd[32 * t + lane] * sc;
+            for (int t = 0; t < NT; ++t) {
+                const int b = 32 * t + lane;
+                const double v = x[u][t] * rd[b];
+                if (NH == 2 && q == 0) x1[u][t] = b < hw ? v : 0.0;
+                if (kk < rows && b < hw) out[static_cast<long long>(kk) * TBW + hh * TW + b] = v * sc;
+            }
         }
+    }
 }
 
-size_t tw_bytes(long long k) {   // the stacked W of either direction
-    const long long nb = (k + TW - 1) / TW;
-    const long long rows = std::max(tw_base(nb - 1, k, 0) + tw_rows(nb - 1, k, 0), tw_base(nb - 1, k, 1) + tw_rows(nb - 1, k, 1));
-    return ((sizeof(double) * rows * TW + 255) & ~static_cast<size_t>(255)) +
+size_t tw_bytes(long long k, int tb) {   // the stacked W of either direction
+    const long long nb = (k + tb - 1) / tb;
+    const long long rows = std::max(tw_base(nb - 1, k, tb, 0) + tw_rows(nb - 1, k, tb, 0),
+                                    tw_base(nb - 1, k, tb, 1) + tw_rows(nb - 1, k, tb, 1));
+    return ((sizeof(double) * rows * tb + 255) & ~static_cast<size_t>(255)) +
            ((sizeof(int) * k + 255) & ~static_cast<size_t>(255));   // and the exponents
 }
 
 size_t trsm_oz_ws_bytes(long long m, long long k, int digits) {
-    return tw_bytes(k) + oz_ws_bytes(std::min(m, TRSM_ROWS), std::min<long long>(k, TW), k, 0, digits) + 256;
+    const int tb = tw_wide(m, k) ? 2 * TW : TW;
+    return tw_bytes(k, tb) + oz_ws_bytes(std::min(m, TRSM_ROWS), std::min<long long>(k, tb), k, 0, digits) + 256;
 }
 
 // Few rows: the same block products on the FP64 units (dgemm_small), B's scaled
@@ -2769,8 +2810,8 @@ gn_status trsm_small(gn_handle h, double* F, long long m, long long k, long long
     const long long nb = (k + TW - 1) / TW;
     for (long long b = 0; b < nb; ++b) {
         const long long J = trans ? nb - 1 - b : b, J0 = J * TW, bw = std::min<long long>(TW, k - J0);
-        const long long K = tw_rows(J, k, trans);
-        const double* Wj = W + tw_base(J, k, trans) * TW;
+        const long long K = tw_rows(J, k, TW, trans);
+        const double* Wj = W + tw_base(J, k, TW, trans) * TW;
         // operand columns: F_{<J} then B_J, or (trans) B_J then F_{>J}
         const double* lo = trans ? Bs + J0 : F;
         const double* hi = trans ? F + J0 : Bs;
@@ -2782,23 +2823,25 @@ gn_status trsm_small(gn_handle h, double* F, long long m, long long k, long long
 
 gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ldf, const double* R, long long ldr,
                   int trans, char* oz, size_t oz_bytes, int digits, const void* src, int src_f32, long long lds) {
-    const long long nb = (k + TW - 1) / TW;
-    const size_t wb = tw_bytes(k);
+    // wide blocks only where the scratch holds all rows (up to TRSM_ROWS) at once
+    const int tb = tw_wide(m, k) && oz_bytes + 256 >= trsm_oz_ws_bytes(m, k, digits) ? 2 * TW : TW;
+    const long long nb = (k + tb - 1) / tb;
+    const size_t wb = tw_bytes(k, tb);
     double* W = reinterpret_cast<double*>(oz);
     int* e = reinterpret_cast<int*>(oz + wb - ((sizeof(int) * k + 255) & ~static_cast<size_t>(255)));
     oz += wb;
     oz_bytes -= wb;
-    const bool few = small_gemm(m, std::min<long long>(k, TW), k) &&
+    const bool few = tb == TW && small_gemm(m, std::min<long long>(k, TW), k) &&
                      sizeof(double) * m * k <= oz_bytes;   // few rows: FP64 units
     // rows at a time: as many as the scratch holds
     long long rows = std::min(m, TRSM_ROWS);
-    while (oz_ws_bytes(rows, std::min<long long>(k, TW), k, 0, digits) > oz_bytes) rows = (rows + 1) / 2;
+    while (oz_ws_bytes(rows, std::min<long long>(k, tb), k, 0, digits) > oz_bytes) rows = (rows + 1) / 2;
     constexpr size_t smem = sizeof(double) * (TW * (TW + 1) + TW);
     static bool attr = false;
     if (!attr) {
-        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem)));
-        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<512>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem)));
         attr = true;
     }
@@ -2815,12 +2858,13 @@ gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ld
         tri_scale_copy_kernel<double><<<cgrid, 256, 0, h->stream>>>(static_cast<const double*>(src), lds, Fs, lds_f, m, ki, e);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
-    // 8 rows per CTA while one round of CTAs (one per SM: 133 KB) holds all rows
-    const long long w_rows = std::max(tw_base(nb - 1, k, trans) + tw_rows(nb - 1, k, trans), k);
-    const bool narrow = w_rows <= 8LL * h->sm_count;
-    const dim3 wgrid(static_cast<unsigned>((k + (narrow ? 7 : 31)) / (narrow ? 8 : 32)), static_cast<unsigned>(nb));
-    if (narrow) tri_w_kernel<128><<<wgrid, 128, smem, h->stream>>>(R, ldr, ki, trans, e, W);
-    else tri_w_kernel<512><<<wgrid, 512, smem, h->stream>>>(R, ldr, ki, trans, e, W);
+    // warps per CTA: one round of CTAs holds all rows
+    const long long w_rows = tw_base(nb - 1, k, tb, trans) + tw_rows(nb - 1, k, tb, trans);
+    const long long sms = std::max<long long>(1, h->sm_count - nb);   // a block's last CTA is not full
+    const int warps = static_cast<int>(std::min<long long>(16, std::max<long long>(4, (w_rows + TW_NR * sms - 1) / (TW_NR * sms))));
+    const dim3 wgrid(static_cast<unsigned>((k + TW_NR * warps - 1) / (TW_NR * warps)), static_cast<unsigned>(nb));
+    if (tb == TW) tri_w_kernel<1><<<wgrid, 32 * warps, smem, h->stream>>>(R, ldr, ki, trans, e, W);
+    else tri_w_kernel<2><<<wgrid, 32 * warps, smem, h->stream>>>(R, ldr, ki, trans, e, W);
     count_launch();
     GN_CUDA_TRY(cudaGetLastError());
     if (few) return trsm_small(h, F, m, k, ldf, R, ldr, trans, W, Fs);
@@ -2829,16 +2873,16 @@ gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ld
         const long long mm = std::min(rows, m - i0);
         double* Fi = F + i0 * ldf;
         for (long long b = 0; b < nb; ++b) {
-            const long long J = trans ? nb - 1 - b : b, J0 = J * TW, bw = std::min<long long>(TW, k - J0);
-            const long long K = tw_rows(J, k, trans), c0 = trans ? J0 : 0;   // operand columns [c0, c0 + K)
-            const double* Wj = W + tw_base(J, k, trans) * TW;
+            const long long J = trans ? nb - 1 - b : b, J0 = J * tb, bw = std::min<long long>(tb, k - J0);
+            const long long K = tw_rows(J, k, tb, trans), c0 = trans ? J0 : 0;   // operand columns [c0, c0 + K)
+            const double* Wj = W + tw_base(J, k, tb, trans) * tb;
             // the part of K that holds B_J first (in place), then the rest onto it
             const long long k0 = trans ? 0 : std::max<long long>(0, K - KG), k1 = trans ? std::min(K, KG) : K;
-            GN_TRY(oz_dgemm(h, mm, bw, k1 - k0, 1.0, Fi + c0 + k0, 0, ldf, 0, Wj + k0 * TW, TW, 0, 0.0, Fi + J0, ldf,
+            GN_TRY(oz_dgemm(h, mm, bw, k1 - k0, 1.0, Fi + c0 + k0, 0, ldf, 0, Wj + k0 * tb, tb, 0, 0.0, Fi + J0, ldf,
                             oz, oz_bytes, digits));
             const long long q0 = trans ? k1 : 0, q1 = trans ? K : k0;
             if (q1 > q0)
-                GN_TRY(oz_dgemm(h, mm, bw, q1 - q0, 1.0, Fi + c0 + q0, 0, ldf, 0, Wj + q0 * TW, TW, 0, 1.0, Fi + J0,
+                GN_TRY(oz_dgemm(h, mm, bw, q1 - q0, 1.0, Fi + c0 + q0, 0, ldf, 0, Wj + q0 * tb, tb, 0, 1.0, Fi + J0,
                                 ldf, oz, oz_bytes, digits));
         }
     }
@@ -2856,7 +2900,7 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
     }
     if (oz && k > TB) {   // (one 32-column block is one substitution launch)
         const size_t pad = (256 - (reinterpret_cast<uintptr_t>(oz) & 255)) & 255;
-        if (oz_bytes >= pad + tw_bytes(k) + oz_ws_bytes(std::min<long long>(m, 256), std::min<long long>(k, TW), k, 0, digits))
+        if (oz_bytes >= pad + tw_bytes(k, TW) + oz_ws_bytes(std::min<long long>(m, 256), std::min<long long>(k, TW), k, 0, digits))
             return trsm_oz(h, F, m, k, ldf, R, ldr, trans, static_cast<char*>(oz) + pad, oz_bytes - pad, digits,
                            src, src_f32, lds);
     }

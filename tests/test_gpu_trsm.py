@@ -122,3 +122,31 @@ def test_zero_pivot_leaves_the_columns_before_it(gn, H):
     ref = torch.linalg.solve_triangular(core.R[:150, :150], AX[:, :150], upper=True, left=False)
     assert close(F[:, :150], ref, 1e-12)
     assert not bool(F[:, 150].isfinite().any())
+
+
+# 256-column blocks: on both sides of the line where they begin (m >= 8192, m r^2 >= 4e9);
+# a last block of one column, of one half, of one half and a column, of both; more rows
+# than one pass takes (32768)
+@pytest.mark.parametrize("m,r", [(8191, 700), (8192, 698), (8192, 700), (8193, 768), (8200, 769), (8192, 770),
+                                 (8192, 896), (8195, 897), (8192, 898), (9000, 1000), (33000, 350)])
+@pytest.mark.parametrize("trans", [0, 1])
+def test_wide_blocks(gn, H, m, r, trans):
+    n, l = 40, 3
+    AX, YtA, core, rn = state(gn, m, n, r, l, torch.float32 if m % 2 else torch.float64)
+    ws = H.workspace(m, max(n, r + l + 1), r, l, gn.F64)
+    k = r
+    ref = AX.double()
+    if trans:   # F = AX Q_2 R_2^-T over the first k columns
+        k = r - 1
+        core.Q2.copy_(rn(r, r) / r ** 0.5)
+        core.R2.copy_(core.R)
+        core.k, core.sgn = k, 1
+        ref = torch.linalg.solve_triangular(core.R2[:k, :k].T, ref @ core.Q2[:, :k], upper=False, left=False)
+    else:
+        ref = torch.linalg.solve_triangular(core.R, ref, upper=True, left=False)
+    F = torch.empty(m, r, dtype=torch.float64, device="cuda")
+    G = torch.empty(r, n, dtype=torch.float64, device="cuda")
+    H.factors(AX, YtA, core, F, G, ws)
+    assert H.sync_status() == 0
+    # R's condition number is below 10 r^1/2: r u 10 r^1/2 stays under 1e-10 at r = 1000
+    assert close(F[:, :k], ref, 1e-12 if r < 1000 else 1e-10)
