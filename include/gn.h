@@ -574,7 +574,8 @@ gn_status gn_batched_tune(gn_handle h, int32_t count, const gn_problem* probs, v
  * four launches on the handle's stream: one grouped tensor-core launch for
  * all sketches AX, Y^T A (BF16, FP32 accumulation), one split of every Y^T A
  * into three BF16 slices, one grouped launch for the slice products of every
- * core C = (Y^T A) X, and one kernel with a CTA per problem (FP64 Householder
+ * core C = (Y^T A) X, and one kernel with a cluster of four CTAs per problem, or
+ * one CTA where the batch has enough problems to fill the SMs (FP64 Householder
  * QR and Q in shared memory, diag(R) >= 0, the Section 5.1.2 detector and
  * Section 5.1.1 truncation per `mode` / `eps` exactly as gn_core, second QR
  * into Q2, R2 when truncated).  No host synchronisation and no allocation;

@@ -331,8 +331,8 @@ class Handle:
         _check(lib.gn_set_fp64_accum(self._h, int(part_k)), "gn_set_fp64_accum")
 
     def set_fp64_tc(self, on: bool):
-        """The factors' large FP64 products (FP32 AX) on the tensor cores by exact
-        digit slicing (True, default) or on the FP64 units (False)."""
+        """Large FP64 products (the FP64 path's, the QR updates', the solves') on the
+        tensor cores by exact digit slicing (True, default) or on the FP64 units (False)."""
         _check(lib.gn_set_fp64_tc(self._h, 1 if on else 0), "gn_set_fp64_tc")
 
     def dgemm_tc(self, A: torch.Tensor, B: torch.Tensor, C: torch.Tensor = None, alpha: float = 1.0,

@@ -7,7 +7,8 @@
 //      still in L2 when the second product streams it);
 //   2. one launch splitting every Y^T A into three BF16 slices;
 //   3. one grouped tcgen05 launch for the three slice products of every core;
-//   4. one launch with a cluster of four CTAs per problem: C = sum of the slice
+//   4. one launch with a cluster of four CTAs per problem (large batches: one
+//      CTA, see bc_pays): C = sum of the slice
 //      products in FP64, Householder QR in shared memory, R and Q (formed in place), the
 //      detector / truncation, and the second QR when the core is truncated.
 //

@@ -1,12 +1,13 @@
 // FP64 kernels of the stable core of generalized Nystrom (Section 5.1) and of
 // the plain FP64 GN path:
-//   * a tiled FP64 GEMM (DFMA) with optional split-K, used for the FP64
-//     sketches, the core product C = (Y^T A) X, the WY updates of the QR and
-//     the factor products;
+//   * a tiled FP64 GEMM (DFMA) with optional split-K and a cluster split-K
+//     kernel for small products (larger FP64 products run as digit slices on the
+//     tensor cores where their scratch is there);
 //   * blocked Householder QR with compact-WY trailing updates (Algorithm 2
 //     step 2, "Y^T A X = QR"), diag(R) made non-negative;
 //   * blocked right triangular solves F R = B and F R^T = B (eq. 5.1's AX/R
-//     and Section 5.1.1's Q_2 R_2^{-T});
+//     and Section 5.1.1's Q_2 R_2^{-T}), a block as one product with the stacked
+//     rows [-R_{<J,J} R_JJ^{-1}; R_JJ^{-1}];
 //   * the truncation rank and the power-method estimate of ||R^{-1}||_2
 //     (Sections 5.1.1 and 5.1.2);
 //   * operand quantisation (FP64/FP32 -> BF16, split BF16) and the fused
