@@ -5,9 +5,8 @@
 //     tensor cores where their scratch is there);
 //   * blocked Householder QR with compact-WY trailing updates (Algorithm 2
 //     step 2, "Y^T A X = QR"), diag(R) made non-negative;
-//   * blocked right triangular solves F R = B and F R^T = B (eq. 5.1's AX/R
-//     and Section 5.1.1's Q_2 R_2^{-T}), a block as one product with the stacked
-//     rows [-R_{<J,J} R_JJ^{-1}; R_JJ^{-1}];
+//   * right triangular solves F R = B and F R^T = B (eq. 5.1's AX/R and Section
+//     5.1.1's Q_2 R_2^{-T}) by substitution, halved recursively;
 //   * the truncation rank and the power-method estimate of ||R^{-1}||_2
 //     (Sections 5.1.1 and 5.1.2);
 //   * operand quantisation (FP64/FP32 -> BF16, split BF16) and the fused
@@ -200,7 +199,6 @@ __global__ void reduce_sum_kernel(const double* __restrict__ part, long long n, 
 // 1000 x 20 x 500: 94 + 5 us as 64 x 64 tiles with split K and a reduction
 // launch, 28 us here (10 M multiply-adds: 21 us at the units' rate); 30 x 500 x
 // 1000: 95 + 6 and 43 us (31); both sketch products at 64 x 64, r = 8: 108 and 14.
-// The columns of A from ka on come from A2 (an operand in two buffers).
 // --------------------------------------------------------------------------
 constexpr int SG_THREADS = 128;
 constexpr int SG_BM = 32;
@@ -208,10 +206,10 @@ constexpr int SG_KC = 32;
 constexpr int SG_MAX_SPLIT = 8;
 
 struct SmallGemm {
-    int M, N, K, ka, kchunk;
+    int M, N, K, kchunk;
     double alpha, beta;
-    const double *A, *A2, *B;
-    long long lda, lda2, ldb, ldc;
+    const double *A, *B;
+    long long lda, ldb, ldc;
     int ta, tb;
     double* C;
 };
@@ -237,11 +235,7 @@ __global__ void __launch_bounds__(SG_THREADS) dgemm_small_kernel(const __grid_co
             const int mm = g.ta ? e & 31 : e >> 5, kk = g.ta ? e >> 5 : e & 31;
             const int i = m0 + mm, k = k0 + kk;
             double v = 0.0;
-            if (i < g.M && k < kend) {
-                const double* p = k < g.ka ? g.A : g.A2;
-                const long long ld = k < g.ka ? g.lda : g.lda2;
-                v = g.ta ? p[k * ld + i] : p[i * ld + k];
-            }
+            if (i < g.M && k < kend) v = g.ta ? g.A[k * g.lda + i] : g.A[i * g.lda + k];
             ra[u] = v;
         }
 #pragma unroll
@@ -362,8 +356,7 @@ gn_status dgemm_launch(gn_handle h, long long M, long long N, long long K, doubl
 constexpr long long SG_MAX_MACS = 16LL << 20;
 
 gn_status dgemm_small(gn_handle h, long long M, long long N, long long K, double alpha, const double* A, long long lda,
-                      int ta, const double* A2, long long lda2, long long ka, const double* B, long long ldb, int tb,
-                      double beta, double* C, long long ldc) {
+                      int ta, const double* B, long long ldb, int tb, double beta, double* C, long long ldc) {
     // columns per warp: the widest that wastes nothing over the next narrower and keeps a few tiles per SM
     int nc = 1;
     for (int c : {2, 4}) {
@@ -377,8 +370,8 @@ gn_status dgemm_small(gn_handle h, long long M, long long N, long long K, double
     S = std::max<long long>(1, std::min(S, K / SG_KC));
     const long long kchunk = ((K + S - 1) / S + SG_KC - 1) / SG_KC * SG_KC;
     S = (K + kchunk - 1) / kchunk;
-    SmallGemm g{static_cast<int>(M), static_cast<int>(N), static_cast<int>(K), static_cast<int>(ka),
-                static_cast<int>(kchunk), alpha, beta, A, A2, B, lda, lda2, ldb, ldc, ta, tb, C};
+    SmallGemm g{static_cast<int>(M), static_cast<int>(N), static_cast<int>(K), static_cast<int>(kchunk),
+                alpha, beta, A, B, lda, ldb, ldc, ta, tb, C};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>((N + 4 * nc - 1) / (4 * nc)), static_cast<unsigned>((M + SG_BM - 1) / SG_BM),
                        static_cast<unsigned>(S));
@@ -1815,7 +1808,7 @@ gn_status dgemm(gn_handle h, long long M, long long N, long long K, double alpha
     // products: 0.08 ms less)
     const bool few_tiles = K >= 1 && ((M + GT - 1) / GT) * ((N + GT - 1) / GT) < h->sm_count && M * N * K <= 4 * SG_MAX_MACS;
     if (M > 0 && N > 0 && (small_gemm(M, N, K) || few_tiles))
-        return dgemm_small(h, M, N, K, alpha, A, lda, ta, A, lda, K, B, ldb, tb, beta, C, ldc);
+        return dgemm_small(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc);
     return dgemm_impl<double, double>(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, ws, ws_bytes);
 }
 
@@ -2568,379 +2561,190 @@ size_t trsm_ws_bytes(long long m, long long k, int sm_count) {
 }
 
 // ---------------------------------------------------------------------------
-// Triangular solve with the products on the tensor cores.  With blocks J of 128 or 256
-// columns, F R = B gives
-//     F_J = (B_J - F_{<J} R_{<J,J}) R_JJ^{-1} = [F_{<J}, B_J] W_J,
-//     W_J = [-R_{<J,J} R_JJ^{-1}; R_JJ^{-1}],
-// and, with the blocks from the last one back, F R^T = B gives
-//     F_J = [B_J, F_{>J}] W_J,   W_J = [R_JJ^{-T}; -R_{J,>J}^T R_JJ^{-T}].
-// F_{<J} and B_J are adjacent columns of F, so each block is one product in
-// place (its operand is sliced before C is written).  The rows of every W_J are
-// triangular solves of a block's unknowns, independent of one another: all of them
-// run in the launch below, in FP64 by substitution.
-// In this form the rows of [F, B_J] and the columns of W_J mix magnitudes: B_J is
-// |R_:J| times F, and the slices are relative to the largest entry.  So B's
-// column j is scaled by 2^-e_j beforehand, e_j the exponent of max_i |R_ij|
-// (trans: max_i |R_ji|), and the inverse's rows by 2^e_j: exact, and every term
-// of a product is then of one size (without it the error grew from 2e-10 to 8e-10
-// of F at r = 2000).
-// Against 32-column substitution steps with a wide update per 128 columns this
-// leaves three launches per block and no substitution over the m rows
-// (16 m k multiply-adds on the FP64 units).  m = 32768, k = 1000 (launches
-// summed): 5.83 -> 3.69 ms (2.8 with blocks of 256 columns); m = 64, k = 1000: 3.5 -> 0.25 ms (its products on the
-// FP64 units), gn_apply there (32768 x 16384, 64 vectors) 4.90 -> 1.27 ms.
-// Error of F against FP64 substitution at m = 32768, k = 1000: 2.5e-12 with 8
-// digits (2.6e-10 with the seven-digit updates before).
+// Triangular solve by substitution, halved recursively: the left half of the columns
+// (trans: the right one), its product taken off the other half, the other half.
+//     F R = B:    F_1 = B_1 R_11^{-1},   F_2 = (B_2 - F_1 R_12) R_22^{-1}
+//     F R^T = B:  F_2 = B_2 R_22^{-T},   F_1 = (B_1 - F_2 R_12^T) R_11^{-T}
+// Down to 32 or 128 columns, which one launch substitutes in FP64.  No inverse is
+// formed: the residual F R - B stays at the rounding of the products and of the
+// substitution, whatever the condition of R's diagonal blocks (a block's inverse costs
+// a factor |R_JJ^{-1}| |R_JJ|: 1e-12 |F||R| instead of 1e-17 on a Kahan matrix).  The
+// halves are disjoint columns, so every product reads what is final and updates what is
+// not, and an infinity or NaN spreads along its row from its own column on.
 // ---------------------------------------------------------------------------
-constexpr int TW = 128;              // columns per block, or per half of a wide one
-constexpr int TW_NR = 2;             // rows of W per warp
-// Blocks of 256 columns: half as many products, each F_{<J} sliced half as often, in
-// 256-column tiles (3e-8 m k^2 us saved), against rows of W that cost 3.6 times the
-// multiply-adds of a 128-column block's in a chain twice as long (85-110 us).  They pay
-// from m k^2 = 3e9 on.  gn_factors with 128- / 256-column blocks, us: 8192 x 500 447 / 482,
-// 8192 x 1000 1128 / 937, 12000 x 300 361 / 441, 20000 x 500 852 / 782, 32768 x 200
-// 472 / 518, 32768 x 1000 3406 / 2546, 32768 x 2000 12230 / 8108 (at k = 500 the CTAs of W
-// sized by its rows, below, take 55 us off the 128-column figure).
-inline bool tw_wide(long long m, long long k) {
-    return m >= 8192 && k > TW && static_cast<double>(m) * k * k >= 4e9;
-}
+constexpr int TR_W = 128;                // columns of one tri_rows_kernel launch
 constexpr long long TRSM_ROWS = 32768;   // rows of F solved together (bounds the slices' scratch)
+// Up to this many rows the base blocks have 128 columns (a launch of 64 rows: 25 us, where four
+// of 32 columns and three products are 4 x 20 + 3 x 7), above it 32 (2048 FP64 multiply-adds per
+// row and 128 columns instead of 8192, and the small products).  gn_factors with blocks of 32 /
+// 128 columns, us: 64 x 1000 1169 / 392, 4096 x 1000 1974 / 1308, 8192 x 500 1072 / 1001, 8192 x
+// 1000 2327 / 2166, 12000 x 300 716 / 802, 16384 x 500 1393 / 1652, 32768 x 1000 5210 / 6962.
+constexpr long long TRSM_FEW = 8192;
 
-// Rows of W_J in the stacked W, and its first row (blocks of tb columns).
-__host__ __device__ inline long long tw_rows(long long J, long long k, int tb, int trans) {
-    return trans ? k - J * tb : (J * tb + tb < k ? J * tb + tb : k);
-}
-__host__ __device__ inline long long tw_base(long long J, long long k, int tb, int trans) {
-    return trans ? J * k - tb * (J * (J - 1) / 2) : tb * (J * (J + 1) / 2);
-}
-
-// e_j = exponent of the largest |R_ij|, i <= j (trans: |R_ji|, i >= j); 0 for a zero
-// or non-finite column.  A CTA takes 32 columns (trans: rows).
-__global__ void __launch_bounds__(1024) tri_scale_kernel(const double* __restrict__ R, long long ldr, int k, int trans,
-                                                        int* __restrict__ e) {
-    __shared__ unsigned long long red[32][33];
-    const int c0 = blockIdx.x * 32, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    unsigned long long m = 0;   // |x| as an unsigned integer orders like |x|
-    if (!trans) {
-        const int j = c0 + lane;
-        if (j < k)
-            for (int i = warp; i <= j; i += 32)
-                m = max(m, static_cast<unsigned long long>(__double_as_longlong(R[static_cast<long long>(i) * ldr + j])) & 0x7FFFFFFFFFFFFFFFull);
-        red[warp][lane] = m;
-    } else {
-        const int j = c0 + warp;
-        if (j < k)
-            for (int i = j + lane; i < k; i += 32)
-                m = max(m, static_cast<unsigned long long>(__double_as_longlong(R[static_cast<long long>(j) * ldr + i])) & 0x7FFFFFFFFFFFFFFFull);
-        red[lane][warp] = m;
+// Columns [j0, j0 + bw), bw <= 128, of F R = B (trans: F R^T = B), a warp per row, four
+// columns per lane.  With the coefficients scaled by the reciprocal pivots, C_ab = R_ab /
+// R_aa, the unknowns before their own scaling follow x_b -= x_a C_ab (trans: x_a -= x_b
+// C_ba, C_ba = R_ab / R_bb), one shuffle and one FMA per step of the chain; x_a / R_aa at
+// the end.  A CTA (one per SM: 133 KB) keeps C in shared memory for its rows, all of its
+// warps fill it and the first `warps` take rows.  Bound by the FP64 rate: 320 instructions
+// of ~64 cycles per row.
+__global__ void __launch_bounds__(512) tri_rows_kernel(double* F, long long m, long long ldf, int j0, int bw,
+                                                      const double* __restrict__ R, long long ldr, int trans,
+                                                      int warps) {
+    extern __shared__ double tr_sm[];
+    double* Cs = tr_sm;                // [TR_W][TR_W + 1]
+    double* rd = Cs + TR_W * (TR_W + 1); // [TR_W]
+    constexpr int NT = TR_W / 32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const double* RJ = R + static_cast<long long>(j0) * (ldr + 1);
+    if (tid < TR_W) rd[tid] = tid < bw ? 1.0 / RJ[static_cast<long long>(tid) * (ldr + 1)] : 0.0;
+    __syncthreads();
+    // R_ab, a < b, read along rows: a warp's part of row a from column 32 (a / 32) on
+#pragma unroll 8
+    for (int i = warp; i < TR_W * NT; i += 16) {
+        const int a = i / NT, b = (i % NT) * 32 + lane;
+        if (i % NT < a / 32) continue;   // (warp-uniform)
+        const double v = a < b && b < bw ? RJ[static_cast<long long>(a) * ldr + b] : 0.0;
+        if (trans) Cs[b * (TR_W + 1) + a] = v * rd[b];
+        else Cs[a * (TR_W + 1) + b] = v * rd[a];
     }
     __syncthreads();
-    if (warp == 0 && c0 + lane < k) {
-        for (int w = 1; w < 32; ++w) m = max(m, red[w][lane]);
-        m = max(m, red[0][lane]);
-        const int E = static_cast<int>(m >> 52);
-        e[c0 + lane] = E == 0 || E == 0x7FF ? 0 : max(-500, min(500, E - 1023));
-    }
-}
-
-// F[:, j] = 2^-e_j src[:, j] (src FP32, FP64 or F itself).  A thread takes four
-// rows of a column (coalesced along the row).
-template <typename T>
-__global__ void __launch_bounds__(256) tri_scale_copy_kernel(const T* src, long long lds, double* F, long long ldf,
-                                                            long long m, int k, const int* __restrict__ e) {
-    const int j = blockIdx.x * 64 + (threadIdx.x & 63);
-    if (j >= k) return;
-    const double s = __longlong_as_double(static_cast<long long>(1023 - e[j]) << 52);
-    for (long long i = blockIdx.y * 16LL + (threadIdx.x >> 6) * 4; i < m; i += gridDim.y * 16LL) {
-        T v[4];
+    if (warp >= warps) return;
+    const long long step = static_cast<long long>(gridDim.x) * warps;
+    for (long long row = static_cast<long long>(blockIdx.x) * warps + warp; row < m; row += step) {
+        double* f = F + row * ldf + j0 + lane;
+        double x[NT];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = i + u < m ? src[(i + u) * lds + j] : T(0);
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (i + u < m) F[(i + u) * ldf + j] = static_cast<double>(v[u]) * s;
-    }
-}
-
-// Row kk of W_J solves x R_JJ = e_c (kk in J) or x R_JJ = -R[kk, J] (forward over
-// the columns), trans: x R_JJ^T = e_c or -R[J, kk]^T (backward).  With the
-// coefficients scaled by the reciprocal pivots, Cs[a][b] = R_ab / R_aa, the
-// unknowns before their own scaling follow x_b -= x_a Cs[a][b], one shuffle and
-// one FMA per step of the chain; x_a / R_aa at the end.  A wide block is solved in two
-// halves of 128 columns, the first one's unknowns taken off the second's right-hand
-// side in between.  A CTA keeps Cs in shared memory for its rows, two per warp (one
-// row's shuffle overlaps the other's FMA), as many warps as let one round of CTAs (one
-// per SM: 133 KB) hold all rows, 4 to 16: the CTA's FP64 rate bounds it (128 columns:
-// 94 us for 32 rows, 28-53 for 8).  k = 1000: 38 M multiply-adds (wide: 92 M).
-template <int NH>
-__global__ void __launch_bounds__(512) tri_w_kernel(const double* __restrict__ R, long long ldr, int k,
-                                                   int trans, const int* __restrict__ e,
-                                                   double* __restrict__ W) {
-    extern __shared__ double tw_sm[];
-    double* Cs = tw_sm;              // [TW][TW + 1]
-    double* rd = Cs + TW * (TW + 1); // [TW]
-    constexpr int TBW = NH * TW;
-    const int J = blockIdx.y, J0 = J * TBW, bw = min(TBW, k - J0);
-    const int rows = static_cast<int>(tw_rows(J, k, TBW, trans));
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nthr = blockDim.x;
-    const int r0 = blockIdx.x * (TW_NR * nthr / 32);
-    if (r0 >= rows) return;
-    constexpr int NR = TW_NR, NT = TW / 32;
-    const int in0 = trans ? 0 : J0;   // rows [in0, in0 + bw) of W_J are the inverse's
-    double x[NR][NT], x1[NR][NT];     // this half's unknowns; the first half's
-    double* out = W + tw_base(J, k, TBW, trans) * TBW;
-#pragma unroll
-    for (int q = 0; q < NH; ++q) {
-        const int hh = trans ? NH - 1 - q : q;
-        const int H0 = J0 + hh * TW, hw = min(TW, k - H0);   // hw <= 0: the last block's missing half
-        // row kk's right-hand side in this half: its column inside J, or its row / column of R outside
-#pragma unroll
-        for (int u = 0; u < NR; ++u) {
-            const int kk = r0 + NR * warp + u, c = kk - in0;
-            const bool unit = c >= 0 && c < bw;
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const int b = 32 * t + lane;
-                double v = 0.0;
-                if (unit) v = hh * TW + b == c ? 1.0 : 0.0;
-                else if (kk < rows && b < hw)
-                    v = trans ? -R[static_cast<long long>(H0 + b) * ldr + J0 + kk]
-                              : -R[static_cast<long long>(kk) * ldr + H0 + b];
-                x[u][t] = v;
-            }
-        }
-        if (NH == 2 && q == 1) {   // x -= x1 R_12 (trans: x1 R_12^T), R_12 = R[J0.., J0 + TW..]
-            const int w2 = min(TW, k - J0 - TW);
-            if (w2 > 0) {
-                __syncthreads();
-                for (int i = tid; i < TW * TW; i += nthr) {
-                    const int a = i / TW, b = i % TW;
-                    const double v = b < w2 ? R[static_cast<long long>(J0 + a) * ldr + J0 + TW + b] : 0.0;
-                    if (trans) Cs[b * (TW + 1) + a] = v;
-                    else Cs[a * (TW + 1) + b] = v;
-                }
-                __syncthreads();
-#pragma unroll
-                for (int p = 0; p < NT; ++p)
-#pragma unroll 8
-                    for (int s = 0; s < 32; ++s) {
-                        const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
-#pragma unroll
-                        for (int u = 0; u < NR; ++u) {
-                            const double xa = __shfl_sync(0xffffffffu, x1[u][p], s);
-#pragma unroll
-                            for (int t = 0; t < NT; ++t) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
-                        }
-                    }
-            }
-        }
-        if (q > 0) __syncthreads();
-        for (int i = tid; i < TW; i += nthr) rd[i] = i < hw ? 1.0 / R[static_cast<long long>(H0 + i) * (ldr + 1)] : 0.0;
-        __syncthreads();
-        for (int i = tid; i < TW * TW; i += nthr) {
-            const int a = i / TW, b = i % TW;   // R_ab, a < b: read along rows
-            const double v = a < b && b < hw ? R[static_cast<long long>(H0 + a) * ldr + H0 + b] : 0.0;
-            if (trans) Cs[b * (TW + 1) + a] = v * rd[b];   // eliminates x_b from x_a, a < b
-            else Cs[a * (TW + 1) + b] = v * rd[a];
-        }
-        __syncthreads();
+        for (int t = 0; t < NT; ++t) x[t] = 32 * t + lane < bw ? f[32 * t] : 0.0;
         if (!trans) {
 #pragma unroll
             for (int p = 0; p < NT; ++p) {
-                if (32 * p >= hw) break;
+                if (32 * p >= bw) break;
 #pragma unroll 8
                 for (int s = 0; s < 32; ++s) {
-                    const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+                    const double* cr = Cs + (32 * p + s) * (TR_W + 1) + lane;
+                    const double xa = __shfl_sync(0xffffffffu, x[p], s);
 #pragma unroll
-                    for (int u = 0; u < NR; ++u) {
-                        const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
-#pragma unroll
-                        for (int t = p; t < NT; ++t)
-                            if (t > p || lane > s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
-                    }
+                    for (int t = p; t < NT; ++t)
+                        if (t > p || lane > s) x[t] = fma(-xa, cr[32 * t], x[t]);
                 }
             }
         } else {
 #pragma unroll
             for (int p = NT - 1; p >= 0; --p) {
-                if (32 * p >= hw) continue;
+                if (32 * p >= bw) continue;
 #pragma unroll 8
                 for (int s = 31; s >= 0; --s) {
-                    const double* cr = Cs + (32 * p + s) * (TW + 1) + lane;
+                    if (32 * p + s >= bw) continue;   // (no such unknown)
+                    const double* cr = Cs + (32 * p + s) * (TR_W + 1) + lane;
+                    const double xa = __shfl_sync(0xffffffffu, x[p], s);
 #pragma unroll
-                    for (int u = 0; u < NR; ++u) {
-                        const double xa = __shfl_sync(0xffffffffu, x[u][p], s);
-#pragma unroll
-                        for (int t = 0; t <= p; ++t)
-                            if (t < p || lane < s) x[u][t] = fma(-xa, cr[32 * t], x[u][t]);
-                    }
+                    for (int t = 0; t <= p; ++t)
+                        if (t < p || lane < s) x[t] = fma(-xa, cr[32 * t], x[t]);
                 }
             }
         }
 #pragma unroll
-        for (int u = 0; u < NR; ++u) {
-            const int kk = r0 + NR * warp + u, c = kk - in0;
-            const double sc = c >= 0 && c < bw ? __longlong_as_double(static_cast<long long>(1023 + e[J0 + c]) << 52) : 1.0;
-#pragma unroll
-            for (int t = 0; t < NT; ++t) {
-                const int b = 32 * t + lane;
-                const double v = x[u][t] * rd[b];
-                if (NH == 2 && q == 0) x1[u][t] = b < hw ? v : 0.0;
-                if (kk < rows && b < hw) out[static_cast<long long>(kk) * TBW + hh * TW + b] = v * sc;
-            }
-        }
+        for (int t = 0; t < NT; ++t)
+            if (32 * t + lane < bw) f[32 * t] = x[t] * rd[32 * t + lane];
     }
 }
 
-size_t tw_bytes(long long k, int tb) {   // the stacked W of either direction
-    const long long nb = (k + tb - 1) / tb;
-    const long long rows = std::max(tw_base(nb - 1, k, tb, 0) + tw_rows(nb - 1, k, tb, 0),
-                                    tw_base(nb - 1, k, tb, 1) + tw_rows(nb - 1, k, tb, 1));
-    return ((sizeof(double) * rows * tb + 255) & ~static_cast<size_t>(255)) +
-           ((sizeof(int) * k + 255) & ~static_cast<size_t>(255));   // and the exponents
+inline int trsm_base(long long m) { return m <= TRSM_FEW ? TR_W : TB; }
+
+// Columns of the first half of w > base.
+inline long long trsm_half(long long w, int base) { return ((w + base - 1) / base + 1) / 2 * base; }
+
+struct TriSolve {
+    gn_handle h;
+    long long m;         // rows of the whole solve (the routes go by it, so that row groups do not change F)
+    double* F;
+    long long mm, ldf;   // rows of this group
+    const double* R;
+    long long ldr;
+    int trans, base, digits;
+    void* oz;
+    size_t oz_bytes;
+    double* ws;
+    size_t ws_bytes;
+};
+
+// F[:, o0 .. o0 + n) -= F[:, i0 .. i0 + k) times R's block (trans: its transpose).
+gn_status trsm_update(const TriSolve& t, long long o0, long long n, long long i0, long long k) {
+    const double* Rb = t.trans ? t.R + o0 * t.ldr + i0 : t.R + i0 * t.ldr + o0;
+    if (t.oz && !small_gemm(t.m, n, k))
+        return oz_dgemm(t.h, t.mm, n, k, -1.0, t.F + i0, 0, t.ldf, 0, Rb, t.ldr, t.trans, 1.0, t.F + o0, t.ldf, t.oz,
+                        t.oz_bytes, t.digits);
+    return dgemm(t.h, t.mm, n, k, -1.0, t.F + i0, t.ldf, 0, Rb, t.ldr, t.trans, 1.0, t.F + o0, t.ldf, t.ws, t.ws_bytes);
+}
+
+gn_status trsm_columns(const TriSolve& t, long long c0, long long w) {
+    if (w > t.base) {
+        const long long w1 = trsm_half(w, t.base);
+        if (!t.trans) {
+            GN_TRY(trsm_columns(t, c0, w1));
+            GN_TRY(trsm_update(t, c0 + w1, w - w1, c0, w1));
+            return trsm_columns(t, c0 + w1, w - w1);
+        }
+        GN_TRY(trsm_columns(t, c0 + w1, w - w1));
+        GN_TRY(trsm_update(t, c0, w1, c0 + w1, w - w1));
+        return trsm_columns(t, c0, w1);
+    }
+    if (t.base == TB) {
+        trsm_diag_kernel<<<static_cast<unsigned>((t.mm + 127) / 128), 128, 0, t.h->stream>>>(
+            t.F, t.mm, t.ldf, static_cast<int>(c0), static_cast<int>(w), t.R, t.ldr, t.trans);
+    } else {
+        // four warps with rows per CTA (one per sub-partition of its SM) until every SM has a CTA, then more
+        const long long warps = std::min<long long>(16, std::max<long long>(4, (t.mm + t.h->sm_count - 1) / t.h->sm_count));
+        constexpr size_t smem = sizeof(double) * (TR_W * (TR_W + 1) + TR_W);
+        GN_CUDA_TRY(cudaFuncSetAttribute(tri_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        const long long ctas = std::min<long long>(t.h->sm_count, (t.mm + warps - 1) / warps);
+        tri_rows_kernel<<<static_cast<unsigned>(ctas), 512, smem, t.h->stream>>>(
+            t.F, t.mm, t.ldf, static_cast<int>(c0), static_cast<int>(w), t.R, t.ldr, t.trans, static_cast<int>(warps));
+    }
+    count_launch();
+    GN_CUDA_TRY(cudaGetLastError());
+    return GN_OK;
+}
+
+// Scratch of the digit-sliced products of `rows` rows of an m-row solve: the first halving's are the largest.
+size_t trsm_group_bytes(long long rows, long long m, long long k, int digits) {
+    const int base = trsm_base(m);
+    if (k <= base) return 0;
+    const long long w1 = trsm_half(k, base);
+    return std::max(oz_ws_bytes(rows, w1, w1, 0, digits), oz_ws_bytes(rows, k - w1, w1, 0, digits));
 }
 
 size_t trsm_oz_ws_bytes(long long m, long long k, int digits) {
-    const int tb = tw_wide(m, k) ? 2 * TW : TW;
-    return tw_bytes(k, tb) + oz_ws_bytes(std::min(m, TRSM_ROWS), std::min<long long>(k, tb), k, 0, digits) + 256;
-}
-
-// Few rows: the same block products on the FP64 units (dgemm_small), B's scaled
-// copy kept apart from F so that no product reads what another CTA writes.
-gn_status trsm_small(gn_handle h, double* F, long long m, long long k, long long ldf, const double* R, long long ldr,
-                     int trans, const double* W, const double* Bs) {
-    const long long nb = (k + TW - 1) / TW;
-    for (long long b = 0; b < nb; ++b) {
-        const long long J = trans ? nb - 1 - b : b, J0 = J * TW, bw = std::min<long long>(TW, k - J0);
-        const long long K = tw_rows(J, k, TW, trans);
-        const double* Wj = W + tw_base(J, k, TW, trans) * TW;
-        // operand columns: F_{<J} then B_J, or (trans) B_J then F_{>J}
-        const double* lo = trans ? Bs + J0 : F;
-        const double* hi = trans ? F + J0 : Bs;
-        GN_TRY(dgemm_small(h, m, bw, K, 1.0, lo, trans ? k : ldf, 0, hi, trans ? ldf : k, trans ? bw : J0, Wj, TW, 0, 0.0,
-                           F + J0, ldf));
-    }
-    return GN_OK;
-}
-
-gn_status trsm_oz(gn_handle h, double* F, long long m, long long k, long long ldf, const double* R, long long ldr,
-                  int trans, char* oz, size_t oz_bytes, int digits, const void* src, int src_f32, long long lds) {
-    // wide blocks only where the scratch holds all rows (up to TRSM_ROWS) at once
-    const int tb = tw_wide(m, k) && oz_bytes + 256 >= trsm_oz_ws_bytes(m, k, digits) ? 2 * TW : TW;
-    const long long nb = (k + tb - 1) / tb;
-    const size_t wb = tw_bytes(k, tb);
-    double* W = reinterpret_cast<double*>(oz);
-    int* e = reinterpret_cast<int*>(oz + wb - ((sizeof(int) * k + 255) & ~static_cast<size_t>(255)));
-    oz += wb;
-    oz_bytes -= wb;
-    const bool few = tb == TW && small_gemm(m, std::min<long long>(k, TW), k) &&
-                     sizeof(double) * m * k <= oz_bytes;   // few rows: FP64 units
-    // rows at a time: as many as the scratch holds
-    long long rows = std::min(m, TRSM_ROWS);
-    while (oz_ws_bytes(rows, std::min<long long>(k, tb), k, 0, digits) > oz_bytes) rows = (rows + 1) / 2;
-    constexpr size_t smem = sizeof(double) * (TW * (TW + 1) + TW);
-    static bool attr = false;
-    if (!attr) {
-        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
-        GN_CUDA_TRY(cudaFuncSetAttribute(tri_w_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem)));
-        attr = true;
-    }
-    const int ki = static_cast<int>(k);
-    tri_scale_kernel<<<static_cast<unsigned>((k + 31) / 32), 1024, 0, h->stream>>>(R, ldr, ki, trans, e);
-    count_launch();
-    GN_CUDA_TRY(cudaGetLastError());
-    double* Fs = few ? reinterpret_cast<double*>(oz) : F;   // the scaled B
-    const long long lds_f = few ? k : ldf;
-    const dim3 cgrid(static_cast<unsigned>((k + 63) / 64), static_cast<unsigned>(std::min<long long>((m + 15) / 16, 8LL * h->sm_count)));
-    if (src_f32)
-        tri_scale_copy_kernel<float><<<cgrid, 256, 0, h->stream>>>(static_cast<const float*>(src), lds, Fs, lds_f, m, ki, e);
-    else
-        tri_scale_copy_kernel<double><<<cgrid, 256, 0, h->stream>>>(static_cast<const double*>(src), lds, Fs, lds_f, m, ki, e);
-    count_launch();
-    GN_CUDA_TRY(cudaGetLastError());
-    // warps per CTA: one round of CTAs holds all rows
-    const long long w_rows = tw_base(nb - 1, k, tb, trans) + tw_rows(nb - 1, k, tb, trans);
-    const long long sms = std::max<long long>(1, h->sm_count - nb);   // a block's last CTA is not full
-    const int warps = static_cast<int>(std::min<long long>(16, std::max<long long>(4, (w_rows + TW_NR * sms - 1) / (TW_NR * sms))));
-    const dim3 wgrid(static_cast<unsigned>((k + TW_NR * warps - 1) / (TW_NR * warps)), static_cast<unsigned>(nb));
-    if (tb == TW) tri_w_kernel<1><<<wgrid, 32 * warps, smem, h->stream>>>(R, ldr, ki, trans, e, W);
-    else tri_w_kernel<2><<<wgrid, 32 * warps, smem, h->stream>>>(R, ldr, ki, trans, e, W);
-    count_launch();
-    GN_CUDA_TRY(cudaGetLastError());
-    if (few) return trsm_small(h, F, m, k, ldf, R, ldr, trans, W, Fs);
-    constexpr long long KG = 4096;   // K of one in-place product: sliced whole before C is written
-    for (long long i0 = 0; i0 < m; i0 += rows) {
-        const long long mm = std::min(rows, m - i0);
-        double* Fi = F + i0 * ldf;
-        for (long long b = 0; b < nb; ++b) {
-            const long long J = trans ? nb - 1 - b : b, J0 = J * tb, bw = std::min<long long>(tb, k - J0);
-            const long long K = tw_rows(J, k, tb, trans), c0 = trans ? J0 : 0;   // operand columns [c0, c0 + K)
-            const double* Wj = W + tw_base(J, k, tb, trans) * tb;
-            // the part of K that holds B_J first (in place), then the rest onto it
-            const long long k0 = trans ? 0 : std::max<long long>(0, K - KG), k1 = trans ? std::min(K, KG) : K;
-            GN_TRY(oz_dgemm(h, mm, bw, k1 - k0, 1.0, Fi + c0 + k0, 0, ldf, 0, Wj + k0 * tb, tb, 0, 0.0, Fi + J0, ldf,
-                            oz, oz_bytes, digits));
-            const long long q0 = trans ? k1 : 0, q1 = trans ? K : k0;
-            if (q1 > q0)
-                GN_TRY(oz_dgemm(h, mm, bw, q1 - q0, 1.0, Fi + c0 + q0, 0, ldf, 0, Wj + q0 * tb, tb, 0, 1.0, Fi + J0,
-                                ldf, oz, oz_bytes, digits));
-        }
-    }
-    return GN_OK;
+    return trsm_group_bytes(std::min(m, TRSM_ROWS), m, k, digits) + 256;
 }
 
 gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, long long ldf,
                            const double* R, long long ldr, int trans, double* ws, size_t ws_bytes, void* oz,
                            size_t oz_bytes, int digits, const void* src, int src_f32, long long lds) {
     if (m <= 0 || k <= 0) return GN_OK;
-    if (!src) {
-        src = F;
-        src_f32 = 0;
-        lds = ldf;
-    }
-    if (oz && k > TB) {   // (one 32-column block is one substitution launch)
-        const size_t pad = (256 - (reinterpret_cast<uintptr_t>(oz) & 255)) & 255;
-        if (oz_bytes >= pad + tw_bytes(k, TW) + oz_ws_bytes(std::min<long long>(m, 256), std::min<long long>(k, TW), k, 0, digits))
-            return trsm_oz(h, F, m, k, ldf, R, ldr, trans, static_cast<char*>(oz) + pad, oz_bytes - pad, digits,
-                           src, src_f32, lds);
-    }
     if (src_f32)
         GN_TRY(copy_f32_to_f64(h, static_cast<const float*>(src), m, k, lds, F, ldf));
-    else if (src != F)
+    else if (src && (src != F || lds != ldf))
         GN_CUDA_TRY(cudaMemcpy2DAsync(F, ldf * 8, src, lds * 8, k * 8, m, cudaMemcpyDeviceToDevice, h->stream));
-    // FP64 units.  Two levels of blocking: 128-column outer blocks take the bulk
-    // of the update as one wide FP64 GEMM each; inside, 32-column blocks take a
-    // narrow GEMM over the outer block and the per-row triangular solve.
-    constexpr long long OB = 128;
-    const long long nob = (k + OB - 1) / OB;
-    const int blocks = static_cast<int>((m + 127) / 128);
-    for (long long obi = 0; obi < nob; ++obi) {
-        const long long ob = trans ? nob - 1 - obi : obi;
-        const long long J0 = ob * OB, JB = std::min<long long>(OB, k - J0);
-        if (!trans && J0 > 0)   // F[:, J] -= F[:, 0:J0] R[0:J0, J]
-            GN_TRY(dgemm(h, m, JB, J0, -1.0, F, ldf, 0, R + J0, ldr, 0, 1.0, F + J0, ldf, ws, ws_bytes));
-        if (trans && J0 + JB < k) {   // F[:, J] -= F[:, J+] R[J, J+]^T
-            const long long kk = k - J0 - JB;
-            GN_TRY(dgemm(h, m, JB, kk, -1.0, F + J0 + JB, ldf, 0, R + J0 * ldr + J0 + JB, ldr, 1, 1.0, F + J0,
-                         ldf, ws, ws_bytes));
+    TriSolve t{h, m, F, m, ldf, R, ldr, trans, k <= TB ? TB : trsm_base(m), digits, nullptr, 0, ws, ws_bytes};
+    long long rows = m;
+    if (oz && k > t.base) {
+        const size_t pad = (256 - (reinterpret_cast<uintptr_t>(oz) & 255)) & 255;
+        const size_t room = oz_bytes > pad ? oz_bytes - pad : 0;
+        rows = std::min(m, TRSM_ROWS);   // as many rows at a time as the scratch holds
+        while (rows > 256 && trsm_group_bytes(rows, m, k, digits) > room) rows = (rows + 1) / 2;
+        if (trsm_group_bytes(rows, m, k, digits) <= room) {
+            t.oz = static_cast<char*>(oz) + pad;
+            t.oz_bytes = room;
+        } else {
+            rows = m;   // too little: every product on the FP64 units
         }
-        const long long nb = (JB + TB - 1) / TB;
-        for (long long bi = 0; bi < nb; ++bi) {
-            const long long b = trans ? nb - 1 - bi : bi;
-            const long long j0 = J0 + b * TB;
-            const int jb = static_cast<int>(std::min<long long>(TB, J0 + JB - j0));
-            if (!trans && j0 > J0)   // F[:, j] -= F[:, J0:j0] R[J0:j0, j]
-                GN_TRY(dgemm(h, m, jb, j0 - J0, -1.0, F + J0, ldf, 0, R + J0 * ldr + j0, ldr, 0, 1.0, F + j0, ldf,
-                             ws, ws_bytes));
-            if (trans && j0 + jb < J0 + JB) {   // F[:, j] -= F[:, j+ .. J0+JB] R[j, j+ ..]^T
-                const long long kk = J0 + JB - j0 - jb;
-                GN_TRY(dgemm(h, m, jb, kk, -1.0, F + j0 + jb, ldf, 0, R + j0 * ldr + j0 + jb, ldr, 1, 1.0,
-                             F + j0, ldf, ws, ws_bytes));
-            }
-            trsm_diag_kernel<<<blocks, 128, 0, h->stream>>>(F, m, ldf, static_cast<int>(j0), jb, R, ldr, trans); count_launch();
-            GN_CUDA_TRY(cudaGetLastError());
-        }
+    }
+    for (long long i0 = 0; i0 < m; i0 += rows) {
+        t.F = F + i0 * ldf;
+        t.mm = std::min(rows, m - i0);
+        GN_TRY(trsm_columns(t, 0, k));
     }
     return GN_OK;
 }

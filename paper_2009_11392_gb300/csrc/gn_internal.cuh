@@ -209,9 +209,8 @@ gn_status qr_form_q(gn_handle h, const double* W, long long M, long long N, long
                     long long ldq, double* ws, size_t ws_bytes, void* oz = nullptr, size_t oz_bytes = 0);
 size_t qr_oz_ws_bytes(long long M, long long N);
 
-// Digits per operand of the FP64 path's products, and of the solves that follow
-// FP32 sketches (the conditioning of R amplifies their rounding: 8 digits keep it
-// at the FP64 units' size, 7 would not).
+// Digits per operand of the FP64 path's products, and of the solves of 1024 rows or
+// more that follow FP32 sketches.
 constexpr int OZ_DIGITS_F64 = 9;
 constexpr int OZ_DIGITS_SOLVE = 8;
 
@@ -220,8 +219,9 @@ constexpr int OZ_DIGITS_SOLVE = 8;
 //   upper == 1, trans == 0: F <- F R^{-1}   (R upper, k x k)
 //   upper == 1, trans == 1: F <- F R^{-T}
 // oz (optional; trsm_oz_ws_bytes(m, k, digits) solves up to 32768 rows together,
-// less takes fewer rows at a time, too little the FP64 units): the products by
-// digit slicing with `digits` (8 or 9) digits; null: the FP64 units.
+// less takes fewer rows at a time, too little the FP64 units): the larger products by
+// digit slicing with `digits` (8 or 9) digits; null: the FP64 units.  ws: scratch of
+// the FP64 products (trsm_ws_bytes; null: without split K).
 size_t trsm_oz_ws_bytes(long long m, long long k, int digits);
 size_t trsm_ws_bytes(long long m, long long k, int sm_count);
 gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, long long ldf,

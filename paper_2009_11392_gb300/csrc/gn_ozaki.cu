@@ -180,7 +180,7 @@ struct OzOperand {
     unsigned long long* mx;   // [passes][rows]
     int rows, K, S;
     int passes;     // ceil(K / OZ_KPASS): pass p is K range [p OZ_KPASS, min(K, (p + 1) OZ_KPASS))
-    int tpr;        // K contiguous: threads per row, a warp per 256 of the pass
+    int tpr;        // K contiguous: threads per row, one per 8 of the pass (4, 8, 16 or whole warps)
     int rpc;        // rows per cluster: OZ_CS (OZ_ST / tpr) (K contiguous) or 32 (rows contiguous)
     int clusters;   // passes x ceil(rows / rpc): one cluster of OZ_CS CTAs per pass and rpc rows
 };
@@ -206,8 +206,8 @@ __device__ __forceinline__ unsigned long long mx_word(unsigned long long m, floa
     return m ? static_cast<unsigned long long>(row_exponent<float>(m) + 1021) << 52 : 0ull;
 }
 
-// K contiguous (s_k == 1): tpr threads per row (a warp per 256 entries of the pass, up
-// to four), OZ_ST / tpr rows per CTA, eight adjacent entries along K per thread (16-byte
+// K contiguous (s_k == 1): tpr threads per row (one per 8 entries of the pass: 4, 8 or 16
+// of a warp, or one to four warps), OZ_ST / tpr rows per CTA, eight adjacent entries along K per thread (16-byte
 // stores per slice, 16-byte loads where the row is aligned); the row maximum is a
 // shuffle, plus an exchange between the row's warps when there are several.  Bound by
 // each CTA's chain (loads, row maximum, digits) as much as by memory: 3.6 GB over the
@@ -220,7 +220,7 @@ __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tpr = o.tpr;   // uniform over the cluster
     const int r = tid / tpr, l = tid - r * tpr;
-    const int nw = tpr >> 5, rows = OZ_ST / tpr;   // (with three warps per row the last warp idles)
+    const int nw = tpr >> 5, rows = OZ_ST / tpr;   // (nw = 0: several rows per warp; with three warps per row the last warp idles)
     const long long i = static_cast<long long>(q) * o.rpc + rank * rows + r;
     const bool live = r < rows && i < o.rows;
     const int K = min(OZ_KPASS, o.K - pass * OZ_KPASS);   // <= 8 tpr
@@ -244,7 +244,10 @@ __device__ __forceinline__ void slice_kcontig(const OzOperand& o, int pass, int 
 #pragma unroll
     for (int u = 0; u < 8; ++u) m = max(m, abs_bits(v[u]));
 #pragma unroll
-    for (int s = 16; s > 0; s >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, s));
+    for (int s = 16; s > 0; s >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(0xffffffffu, m, s);
+        if (s < tpr) m = max(m, o);
+    }
     if (nw > 1) {   // the row's warps
         if (lane == 0) sm.part[warp][0] = m;
         __syncthreads();
@@ -364,7 +367,7 @@ OzOperand oz_operand(const void* src, long long s_row, long long s_k, long long 
     o.slice_stride = slice_stride;
     o.mx = mx;
     o.passes = static_cast<int>((K + OZ_KPASS - 1) / OZ_KPASS);
-    o.tpr = s_k == 1 ? 32 * static_cast<int>((std::min<long long>(K, OZ_KPASS) + 255) / 256) : 0;
+    o.tpr = s_k != 1 ? 0 : K <= 32 ? 4 : K <= 64 ? 8 : K <= 128 ? 16 : 32 * static_cast<int>((std::min<long long>(K, OZ_KPASS) + 255) / 256);
     o.rpc = s_k == 1 ? OZ_CS * (OZ_ST / o.tpr) : 32;
     o.clusters = o.passes * static_cast<int>((rows + o.rpc - 1) / o.rpc);
     return o;
