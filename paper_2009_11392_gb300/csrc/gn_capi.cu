@@ -1069,8 +1069,9 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
     const long long rl = r + l, lds = round8(n), ldq = round8(k);
     __nv_bfloat16 *sl[3] = {nullptr, nullptr, nullptr}, *ql[3] = {nullptr, nullptr, nullptr};
     float* g32 = nullptr;
-    // FP32 AX: the solve's products on the tensor cores (digit slicing)
-    const bool oz_on = AX->dtype == GN_F32 && h->fp64_tc;
+    // FP32 AX of 1024 rows or more: the solve's products and AX Q_2 on the tensor cores (digit
+    // slicing); shorter ones stay on the FP64 units
+    const bool oz_on = AX->dtype == GN_F32 && h->fp64_tc && m >= 1024;
     void* oz = nullptr;
     // at least what the check above asks for, and what ws holds beyond it up to the whole solve
     const size_t oz_spare = ws_bytes - factors_ws(m, n, r, l, mixed, h->sm_count);

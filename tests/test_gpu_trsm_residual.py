@@ -101,3 +101,27 @@ def test_apply_solves_by_substitution(gn, H, kind, side):
         F, T, B = H.apply(AX, YtA, core, W, side=1)[:, :k], core.R, W
     assert H.sync_status() == 0
     assert backward(F, T, B, torch.arange(kw, device="cuda")) <= (k + 4) * 2.0 ** -53
+
+
+@pytest.mark.parametrize("m", [1, 700, 1023])
+def test_short_fp32_sketches_stay_on_the_fp64_units(gn, H, m):
+    """F = (AX Q_2) R_2^-T with R_2 the identity: AX Q_2 entry by entry, with a column of AX
+    1e10 times the others that Q_2 leaves out."""
+    n, l, r, k = 40, 3, 300, 200
+    g = torch.Generator(device="cuda").manual_seed(m)
+    rn = lambda a, b: torch.randn(a, b, generator=g, device="cuda", dtype=torch.float64)
+    core = gn.Core.empty(r, l, "cuda")
+    core.Q.copy_(rn(r + l, r))
+    core.Q2.copy_(rn(r, r))
+    core.Q2[0] = 0.0
+    core.R2.copy_(torch.eye(r, dtype=torch.float64, device="cuda"))
+    core.k, core.sgn = k, 1
+    AX = rn(m, r).float()
+    AX[:, 0] = 1e10
+    F = torch.empty(m, r, dtype=torch.float64, device="cuda")
+    G = torch.empty(r, n, dtype=torch.float64, device="cuda")
+    H.factors(AX, rn(r + l, n).float(), core, F, G, H.workspace(max(m, r), 2 * r, r, l, gn.BF16))
+    assert H.sync_status() == 0
+    a, q = AX.cpu().numpy().astype(np.longdouble), core.Q2[:, :k].cpu().numpy().astype(np.longdouble)
+    err = np.abs(F[:, :k].cpu().numpy() - a[:, 1:] @ q[1:])
+    assert np.all(err <= (r + 4) * 2.0 ** -53 * (np.abs(a[:, 1:]) @ np.abs(q[1:])))   # r u |AX||Q_2|
