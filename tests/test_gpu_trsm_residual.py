@@ -120,7 +120,7 @@ def test_short_fp32_sketches_stay_on_the_fp64_units(gn, H, m):
     AX[:, 0] = 1e10
     F = torch.empty(m, r, dtype=torch.float64, device="cuda")
     G = torch.empty(r, n, dtype=torch.float64, device="cuda")
-    H.factors(AX, rn(r + l, n).float(), core, F, G, H.workspace(max(m, r), 2 * r, r, l, gn.BF16))
+    H.factors(AX, rn(r + l, n).float(), core, F, G, H.workspace(max(m, 2 * r), 2 * r, r, l, gn.BF16))
     assert H.sync_status() == 0
     a, q = AX.cpu().numpy().astype(np.longdouble), core.Q2[:, :k].cpu().numpy().astype(np.longdouble)
     err = np.abs(F[:, :k].cpu().numpy() - a[:, 1:] @ q[1:])
