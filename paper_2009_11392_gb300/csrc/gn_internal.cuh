@@ -233,8 +233,8 @@ gn_status trsm_right_upper(gn_handle h, double* F, long long m, long long k, lon
 // same operand conventions as dgemm, A FP64 or (a_f32) FP32.  digits: BF16
 // digits per operand row / column (7: FP64 accuracy; d < 7: every term carries
 // an error of about 2^(1 - 7d) max|a_i.| max|b_.j|).  8 or 9 digits (FP64 A): a
-// 63-bit window, and infinities and NaN propagate.  C may overlap A or B when
-// K <= 4096 (both are sliced before C is written).
+// 63-bit window, and infinities and NaN propagate.  C shares no element with A or B
+// (it may be other columns of the same matrix).
 size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32, int digits = 7);
 gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double alpha, const void* A, int a_f32,
                    long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,

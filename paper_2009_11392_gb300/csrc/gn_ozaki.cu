@@ -405,8 +405,7 @@ gn_status slice_pair(gn_handle h, const OzOperand& a, int a_f32, const OzOperand
 
 // The operands of a product whose rows may hold infinities or NaN (FP64 paths
 // that must propagate them): an entry of C whose row of A or column of B is not
-// finite in a part is formed from the operands themselves; it is NaN when K = 0
-// (C overlaps A, so the operands are gone).  A null: not checked.
+// finite in a part is formed from the operands themselves.  A null: not checked.
 struct OzDirect {
     const double *A, *B;
     long long a_row, a_k, b_row, b_k;
@@ -415,7 +414,7 @@ struct OzDirect {
 
 __device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, int j) {
     const int k1 = min(x.K, (q + 1) * OZ_KPASS);
-    double s = x.K ? 0.0 : __longlong_as_double(0x7ff8000000000000LL);
+    double s = 0.0;
     for (int k = q * OZ_KPASS; k < k1; ++k) {
         s = fma(x.A[i * x.a_row + k * x.a_k], x.B[j * x.b_row + k * x.b_k], s);
         if (isnan(s)) break;
@@ -562,9 +561,6 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
     if (M > (1LL << 30) || N > (1LL << 30)) return GN_ERR_SHAPE;
     OzWs o;
     if (!oz_carve(M, N, K, sa, sb, ws, ws_bytes, &o)) return GN_ERR_WORKSPACE;
-    const double* A64 = static_cast<const double*>(A);
-    const bool in_place = digits > 7 && C < A64 + (ta ? K : M) * lda && C + M * ldc > A64;
-    if (in_place && K > OZ_PGRP * OZ_KPASS && beta == 0.0) return GN_ERR_INVALID_ARG;
     const int omax = std::max(sa, sb) - 1;   // kept orders 0 .. omax
     int norders = 0, pairs[OZ_MAX_DIGITS][2 * OZ_MAX_DIGITS][2], npairs[OZ_MAX_DIGITS];
     for (int ord = 0; ord <= omax; ++ord) {
@@ -654,7 +650,7 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
             OzDirect dd{};
             if (digits > 7)
                 dd = OzDirect{static_cast<const double*>(A) + a_off, B + b_off, a_row, a_k, b_row, b_k,
-                              in_place ? 0 : static_cast<int>(kc)};
+                              static_cast<int>(kc)};
             auto combine = [&]() {
                 switch (norders) {
                     case 2: return oz_combine_kernel<2>;
