@@ -75,7 +75,7 @@ unsigned long long launch_count();
 void count_launch();
 
 constexpr int TC_MAX_MAPS = 18;
-constexpr int TC_MAX_GEMMS = 9;
+constexpr int TC_MAX_GEMMS = 11;
 constexpr int TC_MAX_SRC = 12;
 
 constexpr int TC_BK = 64;   // K elements per stage of the BF16 multi-GEMM (one K block)

@@ -12,14 +12,14 @@
 //   * the slice products of one order o = s + t carry the unit 2^{-7(o+2)}; each
 //     term is at most 2^12 units, so the FP32 accumulation of the (o+1) products
 //     of order o over K terms is exact while (o+1) K 2^12 <= 2^24.  A pass covers
-//     at most 1024 of K: orders 0..3 are exact; orders 4..6 are rounded, their
-//     rounding sits below 2^-52 of the leading term.
+//     at most 1024 of K: orders 0..3 are exact (with nine digits 0..5, see OZ_OUTS_F64);
+//     the orders above are rounded, with seven digits below 2^-52 of the leading term.
 //   * one launch of the multi-GEMM engine computes D_o = sum_{s+t=o} A_s B_t for
 //     every kept order and every pass of the group (the passes as K-aligned
-//     parts stored apart; the orders of 7, 6, ..., 1 slice products paired on
-//     the CTAs by the boustrophedon tile order); C = beta C + sum over the
+//     parts stored apart; longer and shorter outputs paired on the CTAs by the
+//     boustrophedon tile order); C = beta C + sum over the
 //     passes of alpha 2^{ea_i + eb_j} sum_o D_o in FP64, the passes in order.
-// Orders above 6 are dropped: with 7 digits per operand the error per element is
+// Orders above digits - 1 are dropped: with 7 digits per operand the error per element is
 // about 2^-46 K max_k|a_ik| max_k|b_kj|, the size of an FP64 product's own
 // worst-case rounding error.  FP32 operands take 7 digits too: the digits cover
 // a window below the row's largest entry, not each entry's own 24 bits.
@@ -43,6 +43,13 @@ constexpr int OZ_KPASS = 1024;   // K per pass (exactness of the orders <= 3)
 constexpr int OZ_NPANEL = 256;   // least N per GEMM launch (oz_npanel bounds the FP32 outputs)
 constexpr int OZ_MAX_DIGITS = OZ_DIGITS_F64;
 constexpr int OZ_PGRP = 4;       // passes per group of launches (slicing, products, combination)
+
+// FP32 outputs of a product: one per order, and with nine digits a second one for the orders 4
+// and 5.  Their 5 and 6 slice products can pass 2^24 units over 1024 of K (digits all large and
+// of one sign), so they are cut after four: every output of the orders 0..5 is then exact.
+constexpr int OZ_OUTS_F64 = OZ_DIGITS_F64 + 2;
+constexpr int OZ_CUT = 4;        // slice products per output of the exact orders
+int oz_outputs(int digits) { return digits == OZ_DIGITS_F64 ? OZ_OUTS_F64 : digits; }
 
 size_t al256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 
@@ -426,11 +433,14 @@ __device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, in
 // the K parts q (passes, each with its own row exponents), added in part
 // order with one rounding each.  Within a part the first NEX orders are summed
 // as integers (one rounding), the orders below them in FP32.  NEX = 4 for up to
-// seven digits (units of 2^-35: the orders that are always exact); 6 for nine
-// (units of 2^-49, so that the FP32 sum of the last orders rounds below 2^-60
-// of the leading one).  A thread per column and row group (no division per
-// element; narrow products fill a block with more rows); each exact order is
-// an integer below 2^24 units, so it converts through a 32-bit integer.
+// seven digits (units of 2^-35: the orders that are always exact); 6 for eight and
+// nine (units of 2^-49, so that the FP32 sum of the last orders rounds below 2^-60
+// of the leading one).  With nine digits the orders 4 and 5 come as two outputs,
+// the second ones in slots 9 and 10, so that these are exact too; with eight they
+// are exact unless their sums pass 2^24 units.  A thread per column and row group
+// (no division per element; narrow products fill a block with more rows); each
+// output of an exact order is an integer of at most 2^24 units and converts
+// through a 32-bit integer.
 template <int NORD>
 __global__ void __launch_bounds__(256) oz_combine_kernel(
     const float* __restrict__ D, long long d_stride, long long part_stride, long long ldd, int nparts, int M, int N,
@@ -438,6 +448,7 @@ __global__ void __launch_bounds__(256) oz_combine_kernel(
     double alpha, double beta, double* __restrict__ C, long long ldc, int cw, const __grid_constant__ OzDirect direct,
     int j0) {
     constexpr int NEX = NORD > 7 ? 6 : 4, NEXACT = NORD < NEX ? NORD : NEX;
+    constexpr int NOUT = NORD == OZ_DIGITS_F64 ? OZ_OUTS_F64 : NORD;
     // a block is cw columns by blockDim.x / cw rows (cw: a power of two >= min(N, 256), >= 32)
     const int j = blockIdx.x * cw + static_cast<int>(threadIdx.x) % cw;
     const int rb = static_cast<int>(blockDim.x) / cw, step = gridDim.y * rb;
@@ -445,12 +456,15 @@ __global__ void __launch_bounds__(256) oz_combine_kernel(
     const bool unit = alpha == 1.0 || alpha == -1.0;
     const int flip = alpha == -1.0 ? static_cast<int>(0x80000000u) : 0;
     // one part of one entry from its orders
-    auto value = [&](const float (&d)[NORD], int q, int i) {
+    auto value = [&](const float (&d)[NOUT], int q, int i) {
         long long acc = 0;
 #pragma unroll
-        for (int o = 0; o < NEXACT; ++o)   // D_o is an integer number of units 2^{-7(o+2)}
-            acc += static_cast<long long>(__float2int_rn(d[o] * __int_as_float((127 + 7 * (o + 2)) << 23)))
-                   << (7 * (NEX - 1 - o));
+        for (int o = 0; o < NEXACT; ++o) {   // D_o is an integer number of units 2^{-7(o+2)}
+            const float unit_inv = __int_as_float((127 + 7 * (o + 2)) << 23);
+            int u = __float2int_rn(d[o] * unit_inv);
+            if (NOUT > NORD && o >= 4) u += __float2int_rn(d[NORD + o - 4] * unit_inv);
+            acc += static_cast<long long>(u) << (7 * (NEX - 1 - o));
+        }
         float low = 0.0f;
 #pragma unroll
         for (int o = NORD - 1; o >= NEX; --o) low += d[o];
@@ -481,9 +495,9 @@ __global__ void __launch_bounds__(256) oz_combine_kernel(
             double* c2 = c + step * ldc;
             const float* p = D + static_cast<long long>(i) * ldd + j;
             const float* p2 = p + step * ldd;
-            float d[NORD], e[NORD];
+            float d[NOUT], e[NOUT];
 #pragma unroll
-            for (int o = 0; o < NORD; ++o) {
+            for (int o = 0; o < NOUT; ++o) {
                 d[o] = p[o * d_stride];
                 e[o] = p2[o * d_stride];
             }
@@ -496,9 +510,9 @@ __global__ void __launch_bounds__(256) oz_combine_kernel(
         double out = 0.0;
         for (int q = 0; q < nparts; ++q) {   // K parts (passes) in order, as separate passes would add them
             const float* p = D + q * part_stride + static_cast<long long>(i) * ldd + j;
-            float d[NORD];
+            float d[NOUT];
 #pragma unroll
-            for (int o = 0; o < NORD; ++o) d[o] = p[o * d_stride];
+            for (int o = 0; o < NOUT; ++o) d[o] = p[o * d_stride];
             const double v = value(d, q, i);
             out = q ? out + v : (beta == 0.0 ? v : fma(beta, *c, v));
         }
@@ -518,7 +532,7 @@ long long oz_kgroup(long long K) { return std::min<long long>(std::max<long long
 long long oz_parts(long long kg) { return (kg + OZ_KPASS - 1) / OZ_KPASS; }
 
 bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, size_t ws_bytes, OzWs* o) {
-    const long long kg = oz_kgroup(K), S = oz_parts(kg), np = oz_npanel(M, N, S, sa);
+    const long long kg = oz_kgroup(K), S = oz_parts(kg), np = oz_npanel(M, N, S, oz_outputs(sa));
     o->ldk = r8(kg);
     o->ldd = r4(np);
     char* p = static_cast<char*>(ws);
@@ -530,7 +544,7 @@ bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, s
     };
     o->as = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * sa * M * o->ldk));
     o->bs = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * sb * N * o->ldk));
-    o->d = reinterpret_cast<float*>(take(sizeof(float) * S * sa * M * o->ldd));
+    o->d = reinterpret_cast<float*>(take(sizeof(float) * S * oz_outputs(sa) * M * o->ldd));
     o->mxa = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * S * M));
     o->mxb = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * S * N));
     return off <= ws_bytes;
@@ -540,13 +554,13 @@ bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, s
 
 size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32, int digits) {
     (void)a_f32;
-    const int sa = digits, sb = digits;
+    const int sa = digits, sb = digits, nout = oz_outputs(digits);
     const long long kg = oz_kgroup(K), S = oz_parts(kg);
     // the FP32 outputs of s parts at the panel for s parts, largest over s <= S:
     // the panel narrows as the parts grow, and the size must not shrink with K
     size_t d = 0;
     for (long long s = 1; s <= S; ++s)
-        d = std::max(d, al256(sizeof(float) * s * sa * M * r4(oz_npanel(M, std::max<long long>(N, 1), s, sa))));
+        d = std::max(d, al256(sizeof(float) * s * nout * M * r4(oz_npanel(M, std::max<long long>(N, 1), s, nout))));
     return al256(sizeof(__nv_bfloat16) * sa * M * r8(kg)) + al256(sizeof(__nv_bfloat16) * sb * N * r8(kg)) + d +
            al256(8 * S * M) + al256(8 * S * N) + 256;
 }
@@ -561,27 +575,36 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
     if (M > (1LL << 30) || N > (1LL << 30)) return GN_ERR_SHAPE;
     OzWs o;
     if (!oz_carve(M, N, K, sa, sb, ws, ws_bytes, &o)) return GN_ERR_WORKSPACE;
-    const int omax = std::max(sa, sb) - 1;   // kept orders 0 .. omax
-    int norders = 0, pairs[OZ_MAX_DIGITS][2 * OZ_MAX_DIGITS][2], npairs[OZ_MAX_DIGITS];
-    for (int ord = 0; ord <= omax; ++ord) {
-        npairs[ord] = 0;
-        for (int s = 0; s < sa; ++s) {
-            const int t = ord - s;
-            if (t < 0 || t >= sb) continue;
-            pairs[ord][npairs[ord]][0] = s;
-            pairs[ord][npairs[ord]][1] = t;
-            ++npairs[ord];
-        }
-        if (npairs[ord] > 0) norders = ord + 1;
+    // outputs: the slice products (s, ord - s) of every order 0 .. digits - 1, the orders 4 and 5 of
+    // nine digits cut after OZ_CUT of them (the rest in the slots after the orders')
+    struct Out {
+        int slot, ord, s0, n;   // slice products (s0 + q, ord - s0 - q), q < n
+    };
+    Out outs[OZ_OUTS_F64];
+    const int nout = oz_outputs(digits);
+    for (int ord = 0; ord < digits; ++ord) {
+        const bool cut = nout > digits && (ord == 4 || ord == 5);
+        outs[ord] = Out{ord, ord, 0, cut ? OZ_CUT : ord + 1};
+        if (cut) outs[digits + ord - 4] = Out{digits + ord - 4, ord, OZ_CUT, ord + 1 - OZ_CUT};
     }
-    // every order 0 .. omax has the pair (0, ord): no order is empty
-    if (norders > TC_MAX_GEMMS || sa + sb > TC_MAX_MAPS || npairs[omax] > TC_MAX_SRC) return GN_ERR_UNSUPPORTED;
+    if (nout > TC_MAX_GEMMS || sa + sb > TC_MAX_MAPS || digits > TC_MAX_SRC) return GN_ERR_UNSUPPORTED;
+    // launch order: lengths digits, digits - 1, ..., 1, which the boustrophedon order on
+    // (digits + 1) / 2 groups of CTAs pairs to equal loads (seven digits: 7; 6 + 1; 5 + 2; 4 + 3).
+    // Nine digits, 9, 8, 7, 4, 4, 4, 3, 2, 2, 1, 1 on 5 groups: 4 + 4 + 2, 4 + 3, 7 + 2, 8 + 1, 9 + 1.
+    if (nout > digits) {
+        const int by[OZ_OUTS_F64] = {5, 4, 6, 7, 8, 0, 9, 1, 2, 3, 10};
+        Out t[OZ_OUTS_F64];
+        for (int i = 0; i < nout; ++i) t[i] = outs[by[i]];
+        std::copy(t, t + nout, outs);
+    } else {
+        std::reverse(outs, outs + nout);
+    }
     const long long as_stride = M * o.ldk, bs_stride = N * o.ldk, d_stride = M * o.ldd;
     // groups of at most OZ_PGRP passes: one slicing launch for all of them, the
     // passes as K-aligned parts of one multi-GEMM launch (stored apart), one
     // combination adding them in order
-    const long long part_stride = sa * d_stride;
-    const long long npanel = oz_npanel(M, N, oz_parts(oz_kgroup(K)), sa);   // the carve's panel (largest group)
+    const long long part_stride = nout * d_stride;
+    const long long npanel = oz_npanel(M, N, oz_parts(oz_kgroup(K)), nout);   // the carve's panel (largest group)
     for (long long k0 = 0; k0 < K; k0 += OZ_PGRP * OZ_KPASS) {
         const long long kc = std::min<long long>(OZ_PGRP * OZ_KPASS, K - k0);
         const int S = static_cast<int>(oz_parts(kc));
@@ -601,7 +624,7 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
             // N tile: the widest of 256 / 128 / 64 that still gives the GPU about
             // two work items per SM over the orders and parts (small products are latency-bound)
             int bn = static_cast<int>(std::min<long long>(256, (nb + 31) / 32 * 32));
-            while (bn > 64 && ((M + 127) / 128) * ((nb + bn - 1) / bn) * norders * S < 2LL * h->sm_count)
+            while (bn > 64 && ((M + 127) / 128) * ((nb + bn - 1) / bn) * nout * S < 2LL * h->sm_count)
                 bn = (bn / 2 + 31) / 32 * 32;
             TcParams p;
             memset(&p, 0, sizeof(p));
@@ -609,12 +632,8 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                 GN_TRY(tc_make_map_bf16(&p.maps[s], o.as + s * as_stride, M, kc, o.ldk, 64, 128));
             for (int t = 0; t < sb; ++t)
                 GN_TRY(tc_make_map_bf16(&p.maps[sa + t], o.bs + t * bs_stride + j0 * o.ldk, nb, kc, o.ldk, 64, bn));
-            // the orders with the most slice products first (the longest tiles)
-            int order_of[OZ_MAX_DIGITS];
-            for (int i = 0; i < norders; ++i) order_of[i] = i;
-            std::stable_sort(order_of, order_of + norders, [&](int a, int b) { return npairs[a] > npairs[b]; });
-            for (int gi = 0; gi < norders; ++gi) {
-                const int ord = order_of[gi];
+            for (int gi = 0; gi < nout; ++gi) {
+                const Out& out = outs[gi];
                 TcGemm& g = p.g[gi];
                 g.M = static_cast<int>(M);
                 g.N = static_cast<int>(nb);
@@ -622,12 +641,12 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                 g.bn = bn;
                 g.a_mn = 0;
                 g.b_mn = 0;
-                g.nsrc = npairs[ord];
-                for (int q = 0; q < npairs[ord]; ++q) {
-                    g.a_map[q] = pairs[ord][q][0];
-                    g.b_map[q] = sa + pairs[ord][q][1];
+                g.nsrc = out.n;
+                for (int q = 0; q < out.n; ++q) {
+                    g.a_map[q] = static_cast<signed char>(out.s0 + q);
+                    g.b_map[q] = static_cast<signed char>(sa + out.ord - out.s0 - q);
                 }
-                g.D = o.d + ord * d_stride;
+                g.D = o.d + out.slot * d_stride;
                 g.ldd = o.ldd;
                 if (S >= 2) {   // pass q of the group: its own row scaling, stored at D + q part_stride
                     g.ksplit = S;
@@ -635,10 +654,8 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                     g.kpart = OZ_KPASS / TC_BK;
                 }
             }
-            p.ngemm = norders;
-            // orders of 7, 6, ..., 1 slice products: the boustrophedon order on
-            // 4 groups of CTAs gives every CTA 7 (order 6; 5 + 0; 4 + 1; 3 + 2)
-            p.snake_groups = (norders + 1) / 2;
+            p.ngemm = nout;
+            p.snake_groups = (digits + 1) / 2;
             GN_TRY(tc_launch(h, &p));
             int cw = 32;   // a power of two, so that it divides the block's 256 threads
             while (cw < nb && cw < 256) cw *= 2;
@@ -652,7 +669,7 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                 dd = OzDirect{static_cast<const double*>(A) + a_off, B + b_off, a_row, a_k, b_row, b_k,
                               static_cast<int>(kc)};
             auto combine = [&]() {
-                switch (norders) {
+                switch (digits) {
                     case 2: return oz_combine_kernel<2>;
                     case 3: return oz_combine_kernel<3>;
                     case 4: return oz_combine_kernel<4>;
