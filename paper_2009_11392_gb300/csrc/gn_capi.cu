@@ -430,9 +430,8 @@ gn_status launch_sketch_tc(gn_handle h, const gn_mat* A, const gn_mat* X, const 
     }
     // Order: the longer-K GEMM first (its tiles are the expensive ones).
     if (m >= n) {
-        TcGemm t = p.g[0];
-        p.g[0] = p.g[1];
-        p.g[1] = t;
+        std::swap(p.g[0], p.g[1]);
+        std::swap(p.sf[0], p.sf[1]);
     }
     p.ngemm = 2;
     GN_TRY(tc_launch(h, &p));
@@ -474,14 +473,15 @@ gn_status launch_sketch_e4m3(gn_handle h, const gn_mat* A, const gn_mat* X, cons
     g0.b_map[0] = 1;
     g0.D = static_cast<float*>(AX->data);
     g0.ldd = AX->ld;
-    g0.sfa = imA;                               // A tile (rb, kb): image (rb, kb)
-    g0.sfa_ld = static_cast<int>(tiles128(n));
-    g0.sfa_tr = 0;
-    g0.sfa_rows = static_cast<int>(tiles128(m));
-    g0.sfb = imX;                               // X^T tile (rb, kb) is X tile (kb, rb)
-    g0.sfb_ld = static_cast<int>(tiles128(r));
-    g0.sfb_tr = 1;
-    g0.sfb_rows = static_cast<int>(tiles128(r));
+    TcScales& s0 = p.sf[0];
+    s0.sfa = imA;                               // A tile (rb, kb): image (rb, kb)
+    s0.sfa_ld = static_cast<int>(tiles128(n));
+    s0.sfa_tr = 0;
+    s0.sfa_rows = static_cast<int>(tiles128(m));
+    s0.sfb = imX;                               // X^T tile (rb, kb) is X tile (kb, rb)
+    s0.sfb_ld = static_cast<int>(tiles128(r));
+    s0.sfb_tr = 1;
+    s0.sfb_rows = static_cast<int>(tiles128(r));
     TcGemm& g1 = p.g[1];
     g1.M = static_cast<int>(rl);
     g1.N = static_cast<int>(n);
@@ -492,16 +492,20 @@ gn_status launch_sketch_e4m3(gn_handle h, const gn_mat* A, const gn_mat* X, cons
     g1.b_map[0] = 3;
     g1.D = static_cast<float*>(YtA->data);
     g1.ldd = YtA->ld;
-    g1.sfa = imY;                               // Y^T tile (rb, kb) is Y tile (kb, rb)
-    g1.sfa_ld = static_cast<int>(tiles128(rl));
-    g1.sfa_tr = 1;
-    g1.sfa_rows = static_cast<int>(tiles128(rl));
-    g1.sfb = imA;                               // A^T tile (rb, kb) is A tile (kb, rb)
-    g1.sfb_ld = static_cast<int>(tiles128(n));
-    g1.sfb_tr = 1;
-    g1.sfb_rows = static_cast<int>(tiles128(n));
+    TcScales& s1 = p.sf[1];
+    s1.sfa = imY;                               // Y^T tile (rb, kb) is Y tile (kb, rb)
+    s1.sfa_ld = static_cast<int>(tiles128(rl));
+    s1.sfa_tr = 1;
+    s1.sfa_rows = static_cast<int>(tiles128(rl));
+    s1.sfb = imA;                               // A^T tile (rb, kb) is A tile (kb, rb)
+    s1.sfb_ld = static_cast<int>(tiles128(n));
+    s1.sfb_tr = 1;
+    s1.sfb_rows = static_cast<int>(tiles128(n));
     if (r == 0 || rl == 0) {   // a block sketch that needs one product only
-        if (r == 0) p.g[0] = p.g[1];
+        if (r == 0) {
+            p.g[0] = p.g[1];
+            p.sf[0] = p.sf[1];
+        }
         p.ngemm = 1;
         p.f8 = 1;
         return tc_launch(h, &p);
@@ -514,9 +518,8 @@ gn_status launch_sketch_e4m3(gn_handle h, const gn_mat* A, const gn_mat* X, cons
     if (split.bytes() && ws_bytes >= cv.off + pad + split.bytes())
         sketch_split_apply(split, &g0, &g1, AX, YtA, rest + pad, &jobs, &njobs);
     if (m >= n) {   // the longer-K GEMM first
-        TcGemm t = p.g[0];
-        p.g[0] = p.g[1];
-        p.g[1] = t;
+        std::swap(p.g[0], p.g[1]);
+        std::swap(p.sf[0], p.sf[1]);
     }
     p.ngemm = 2;
     p.f8 = 1;

@@ -74,8 +74,8 @@ namespace gn {
 unsigned long long launch_count();
 void count_launch();
 
-constexpr int TC_MAX_MAPS = 18;
-constexpr int TC_MAX_GEMMS = 11;
+constexpr int TC_MAX_MAPS = 20;
+constexpr int TC_MAX_GEMMS = 12;
 constexpr int TC_MAX_SRC = 12;
 
 constexpr int TC_BK = 64;   // K elements per stage of the BF16 multi-GEMM (one K block)
@@ -99,8 +99,12 @@ struct TcGemm {
                              // (not added) at D + c * part_stride, to be summed by the caller
     int kpart;               // > 0 (stored parts only): part c covers K blocks [c kpart, (c + 1) kpart)
                              // of every source (K-aligned); 0: parts of the sources' joint K sequence
-    // e4m3 launches (TcParams::f8): scale-factor images, 512 bytes of the tile's
-    // UE8M0 byte per 128 x 128 tile of the original matrix, row-major over tiles.
+};
+
+// e4m3 launches (TcParams::f8): a GEMM's scale-factor images, 512 bytes of the tile's
+// UE8M0 byte per 128 x 128 tile of the original matrix, row-major over tiles.
+constexpr int TC_MAX_F8_GEMMS = 2;
+struct TcScales {
     const uint8_t* sfa;
     const uint8_t* sfb;
     int sfa_ld, sfb_ld;      // tiles per row of the image's tile grid
@@ -111,6 +115,7 @@ struct TcGemm {
 struct TcParams {
     CUtensorMap maps[TC_MAX_MAPS];
     TcGemm g[TC_MAX_GEMMS];
+    TcScales sf[TC_MAX_F8_GEMMS];   // of g[i] (f8 only)
     const TcGemm* gg;          // grouped mode: descriptors in device memory
     const CUtensorMap* gmaps;  // grouped mode: tensor maps in device memory (64-B aligned)
     int ngemm;

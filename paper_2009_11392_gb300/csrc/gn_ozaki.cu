@@ -47,9 +47,22 @@ constexpr int OZ_PGRP = 4;       // passes per group of launches (slicing, produ
 // FP32 outputs of a product: one per order, and with nine digits a second one for the orders 4
 // and 5.  Their 5 and 6 slice products can pass 2^24 units over 1024 of K (digits all large and
 // of one sign), so they are cut after four: every output of the orders 0..5 is then exact.
-constexpr int OZ_OUTS_F64 = OZ_DIGITS_F64 + 2;
+// The last output is the size of each entry, sum_k |a_ik| |b_kj| from the leading digits' absolute
+// values (a slice of its own): where that is small, the window below the row's and the column's
+// largest entries is not enough and the entry is formed from the operands (see OZ_SMALL).
+constexpr int OZ_OUTS_F64 = OZ_DIGITS_F64 + 3;
+constexpr int OZ_SLICES_F64 = OZ_DIGITS_F64 + 1;
 constexpr int OZ_CUT = 4;        // slice products per output of the exact orders
 int oz_outputs(int digits) { return digits == OZ_DIGITS_F64 ? OZ_OUTS_F64 : digits; }
+int oz_slices(int digits) { return digits == OZ_DIGITS_F64 ? OZ_SLICES_F64 : digits; }
+
+// An entry whose size S is below this (rows and columns scaled to maxima of 1/4 .. 1/2) in a part
+// is formed from the operands with FP64 FMA.  The digits' error in a part is at most K 2^-62
+// there (rounding of both operands to 2^-64, the orders dropped below 2^-62), typically
+// K^1/2 2^-65; the bound of an FP64 sum is K 2^-53 S.  The two meet at S = 2^-9, so that the
+// digits never exceed the bound that the FP64 units keep, entry by entry.  (Leading digits round:
+// S is at most twice too large where it is that small.)
+constexpr float OZ_SMALL = 1.0f / 256.0f;
 
 size_t al256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 
@@ -146,7 +159,7 @@ __device__ __forceinline__ float digit_value(unsigned long long U, int s) {
 }
 
 // Digits of two entries adjacent along K, stored as one bf16 pair per slice
-// (out 4-byte aligned, slice_stride even).
+// (out 4-byte aligned, slice_stride even); after nine digits the absolute values of the first.
 template <int W>
 __device__ __forceinline__ void write_digits2(long long Y0, long long Y1, int S, unsigned long long bias,
                                               __nv_bfloat16* out, long long slice_stride) {
@@ -155,8 +168,10 @@ __device__ __forceinline__ void write_digits2(long long Y0, long long Y1, int S,
 #pragma unroll
     for (int s = 0; s < W; ++s) {
         if (s >= S) break;
-        *reinterpret_cast<__nv_bfloat162*>(out + s * slice_stride) =
-            __floats2bfloat162_rn(digit_value<W>(U0, s), digit_value<W>(U1, s));
+        const __nv_bfloat162 w = __floats2bfloat162_rn(digit_value<W>(U0, s), digit_value<W>(U1, s));
+        *reinterpret_cast<__nv_bfloat162*>(out + s * slice_stride) = w;
+        if (W == OZ_DIGITS_F64 && s == 0 && S == W)
+            *reinterpret_cast<__nv_bfloat162*>(out + W * slice_stride) = __habs2(w);
     }
 }
 
@@ -171,6 +186,11 @@ __device__ __forceinline__ void write_digits8(const unsigned long long (&U)[8], 
 #pragma unroll
         for (int u = 0; u < 4; ++u) w[u] = __floats2bfloat162_rn(digit_value<W>(U[2 * u], s), digit_value<W>(U[2 * u + 1], s));
         *reinterpret_cast<uint4*>(out + s * slice_stride) = *reinterpret_cast<const uint4*>(w);
+        if (W == OZ_DIGITS_F64 && s == 0 && S == W) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) w[u] = __habs2(w[u]);
+            *reinterpret_cast<uint4*>(out + W * slice_stride) = *reinterpret_cast<const uint4*>(w);
+        }
     }
 }
 
@@ -410,21 +430,53 @@ gn_status slice_pair(gn_handle h, const OzOperand& a, int a_f32, const OzOperand
     return GN_OK;
 }
 
-// The operands of a product whose rows may hold infinities or NaN (FP64 paths
-// that must propagate them): an entry of C whose row of A or column of B is not
-// finite in a part is formed from the operands themselves.  A null: not checked.
+// The operands of a product with eight or nine digits: an entry of C whose row of A or
+// column of B is not finite in a part, or (nine) whose size is below OZ_SMALL, is formed
+// from the operands themselves.  A null: not checked.
 struct OzDirect {
     const double *A, *B;
     long long a_row, a_k, b_row, b_k;
     int K;
 };
 
-__device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, int j) {
-    const int k1 = min(x.K, (q + 1) * OZ_KPASS);
+// Part q of entry (i, j), j a lane's own column, for the lanes of `need` (a warp has one row
+// i and the columns of its first popc(live) lanes; all of these call).  A few entries: the
+// lanes share each one's sum.  Many: a lane each, eight terms loaded ahead.
+__device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, int j, unsigned need, unsigned live) {
+    const int lane = threadIdx.x & 31, k0 = q * OZ_KPASS, k1 = min(x.K, k0 + OZ_KPASS);
+    const double* a = x.A + i * x.a_row;
+    const double* b = x.B + j * x.b_row;
     double s = 0.0;
-    for (int k = q * OZ_KPASS; k < k1; ++k) {
-        s = fma(x.A[i * x.a_row + k * x.a_k], x.B[j * x.b_row + k * x.b_k], s);
-        if (isnan(s)) break;
+    if (__popc(need) > 8) {
+        if (need >> lane & 1) {
+            int k = k0;
+            for (; k + 8 <= k1; k += 8) {
+                double av[8], bv[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) {
+                    av[u] = a[(k + u) * x.a_k];
+                    bv[u] = b[(k + u) * x.b_k];
+                }
+#pragma unroll
+                for (int u = 0; u < 8; ++u) s = fma(av[u], bv[u], s);
+            }
+            for (; k < k1; ++k) s = fma(a[k * x.a_k], b[k * x.b_k], s);
+        }
+        return s;
+    }
+    const int cnt = __popc(live);
+    for (unsigned todo = need; todo; todo &= todo - 1) {
+        const int t = __ffs(todo) - 1;
+        const double* bt = x.B + (j - lane + t) * x.b_row;
+        double p = 0.0;
+        for (int k = k0 + lane; k < k1; k += cnt) p = fma(a[k * x.a_k], bt[k * x.b_k], p);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const double y = __shfl_down_sync(live, p, o);
+            if (lane + o < cnt) p += y;
+        }
+        p = __shfl_sync(live, p, 0);
+        if (lane == t) s = p;
     }
     return s;
 }
@@ -436,8 +488,8 @@ __device__ __noinline__ double oz_direct_dot(const OzDirect& x, int q, int i, in
 // seven digits (units of 2^-35: the orders that are always exact); 6 for eight and
 // nine (units of 2^-49, so that the FP32 sum of the last orders rounds below 2^-60
 // of the leading one).  With nine digits the orders 4 and 5 come as two outputs,
-// the second ones in slots 9 and 10, so that these are exact too; with eight they
-// are exact unless their sums pass 2^24 units.  A thread per column and row group
+// the second ones in slots 9 and 10, so that these are exact too (slot 11 is the
+// entry's size); with eight they are exact unless their sums pass 2^24 units.  A thread per column and row group
 // (no division per element; narrow products fill a block with more rows); each
 // output of an exact order is an integer of at most 2^24 units and converts
 // through a 32-bit integer.
@@ -452,6 +504,7 @@ __global__ void __launch_bounds__(256) oz_combine_kernel(
     // a block is cw columns by blockDim.x / cw rows (cw: a power of two >= min(N, 256), >= 32)
     const int j = blockIdx.x * cw + static_cast<int>(threadIdx.x) % cw;
     const int rb = static_cast<int>(blockDim.x) / cw, step = gridDim.y * rb;
+    const unsigned live = __ballot_sync(0xffffffffu, j < N);   // (a warp's columns are consecutive)
     if (j >= N) return;
     const bool unit = alpha == 1.0 || alpha == -1.0;
     const int flip = alpha == -1.0 ? static_cast<int>(0x80000000u) : 0;
@@ -483,7 +536,15 @@ __global__ void __launch_bounds__(256) oz_combine_kernel(
         } else if ((__double2hiint(x) << 1 | __double2loint(x)) != 0) {
             v = alpha * ldexp(x, p);
         }
-        if (NEX == 6 && direct.A && max(ma, mb) >= 0x7FF0000000000000ull) v = alpha * oz_direct_dot(direct, q, i, j0 + j);
+        if (NEX == 6) {
+            const bool need = direct.A && (max(ma, mb) >= 0x7FF0000000000000ull ||
+                                           (NOUT > NORD && ma && mb && d[NOUT - 1] < OZ_SMALL));
+            const unsigned any = __ballot_sync(live, need);
+            if (any) {
+                const double x = oz_direct_dot(direct, q, i, j0 + j, any, live);
+                if (need) v = alpha * x;
+            }
+        }
         return v;
     };
     int i = blockIdx.y * rb + static_cast<int>(threadIdx.x) / cw;
@@ -542,8 +603,8 @@ bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, s
         off += al256(bytes);
         return q;
     };
-    o->as = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * sa * M * o->ldk));
-    o->bs = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * sb * N * o->ldk));
+    o->as = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * oz_slices(sa) * M * o->ldk));
+    o->bs = reinterpret_cast<__nv_bfloat16*>(take(sizeof(__nv_bfloat16) * oz_slices(sb) * N * o->ldk));
     o->d = reinterpret_cast<float*>(take(sizeof(float) * S * oz_outputs(sa) * M * o->ldd));
     o->mxa = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * S * M));
     o->mxb = reinterpret_cast<unsigned long long*>(take(sizeof(unsigned long long) * S * N));
@@ -554,14 +615,14 @@ bool oz_carve(long long M, long long N, long long K, int sa, int sb, void* ws, s
 
 size_t oz_ws_bytes(long long M, long long N, long long K, int a_f32, int digits) {
     (void)a_f32;
-    const int sa = digits, sb = digits, nout = oz_outputs(digits);
+    const int slices = oz_slices(digits), nout = oz_outputs(digits);
     const long long kg = oz_kgroup(K), S = oz_parts(kg);
     // the FP32 outputs of s parts at the panel for s parts, largest over s <= S:
     // the panel narrows as the parts grow, and the size must not shrink with K
     size_t d = 0;
     for (long long s = 1; s <= S; ++s)
         d = std::max(d, al256(sizeof(float) * s * nout * M * r4(oz_npanel(M, std::max<long long>(N, 1), s, nout))));
-    return al256(sizeof(__nv_bfloat16) * sa * M * r8(kg)) + al256(sizeof(__nv_bfloat16) * sb * N * r8(kg)) + d +
+    return al256(sizeof(__nv_bfloat16) * slices * M * r8(kg)) + al256(sizeof(__nv_bfloat16) * slices * N * r8(kg)) + d +
            al256(8 * S * M) + al256(8 * S * N) + 256;
 }
 
@@ -576,7 +637,8 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
     OzWs o;
     if (!oz_carve(M, N, K, sa, sb, ws, ws_bytes, &o)) return GN_ERR_WORKSPACE;
     // outputs: the slice products (s, ord - s) of every order 0 .. digits - 1, the orders 4 and 5 of
-    // nine digits cut after OZ_CUT of them (the rest in the slots after the orders')
+    // nine digits cut after OZ_CUT of them (the rest in the slots after the orders'), the size last
+    const int ns = oz_slices(digits);
     struct Out {
         int slot, ord, s0, n;   // slice products (s0 + q, ord - s0 - q), q < n
     };
@@ -587,12 +649,13 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
         outs[ord] = Out{ord, ord, 0, cut ? OZ_CUT : ord + 1};
         if (cut) outs[digits + ord - 4] = Out{digits + ord - 4, ord, OZ_CUT, ord + 1 - OZ_CUT};
     }
-    if (nout > TC_MAX_GEMMS || sa + sb > TC_MAX_MAPS || digits > TC_MAX_SRC) return GN_ERR_UNSUPPORTED;
+    if (nout > digits) outs[nout - 1] = Out{nout - 1, 2 * digits, digits, 1};   // slice `digits` of both
+    if (nout > TC_MAX_GEMMS || 2 * ns > TC_MAX_MAPS || digits > TC_MAX_SRC) return GN_ERR_UNSUPPORTED;
     // launch order: lengths digits, digits - 1, ..., 1, which the boustrophedon order on
     // (digits + 1) / 2 groups of CTAs pairs to equal loads (seven digits: 7; 6 + 1; 5 + 2; 4 + 3).
-    // Nine digits, 9, 8, 7, 4, 4, 4, 3, 2, 2, 1, 1 on 5 groups: 4 + 4 + 2, 4 + 3, 7 + 2, 8 + 1, 9 + 1.
+    // Nine digits, 9, 8, 7, 4, 4, 4, 3, 2, 2, 1, 1, 1 on 5 groups: 4 + 4 + 1, 4 + 3 + 2, 7 + 2, 8 + 1, 9 + 1.
     if (nout > digits) {
-        const int by[OZ_OUTS_F64] = {5, 4, 6, 7, 8, 0, 9, 1, 2, 3, 10};
+        const int by[OZ_OUTS_F64] = {5, 4, 6, 7, 8, 0, 9, 1, 2, 3, 11, 10};
         Out t[OZ_OUTS_F64];
         for (int i = 0; i < nout; ++i) t[i] = outs[by[i]];
         std::copy(t, t + nout, outs);
@@ -628,10 +691,10 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                 bn = (bn / 2 + 31) / 32 * 32;
             TcParams p;
             memset(&p, 0, sizeof(p));
-            for (int s = 0; s < sa; ++s)
+            for (int s = 0; s < ns; ++s)
                 GN_TRY(tc_make_map_bf16(&p.maps[s], o.as + s * as_stride, M, kc, o.ldk, 64, 128));
-            for (int t = 0; t < sb; ++t)
-                GN_TRY(tc_make_map_bf16(&p.maps[sa + t], o.bs + t * bs_stride + j0 * o.ldk, nb, kc, o.ldk, 64, bn));
+            for (int t = 0; t < ns; ++t)
+                GN_TRY(tc_make_map_bf16(&p.maps[ns + t], o.bs + t * bs_stride + j0 * o.ldk, nb, kc, o.ldk, 64, bn));
             for (int gi = 0; gi < nout; ++gi) {
                 const Out& out = outs[gi];
                 TcGemm& g = p.g[gi];
@@ -644,7 +707,7 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                 g.nsrc = out.n;
                 for (int q = 0; q < out.n; ++q) {
                     g.a_map[q] = static_cast<signed char>(out.s0 + q);
-                    g.b_map[q] = static_cast<signed char>(sa + out.ord - out.s0 - q);
+                    g.b_map[q] = static_cast<signed char>(ns + out.ord - out.s0 - q);
                 }
                 g.D = o.d + out.slot * d_stride;
                 g.ldd = o.ldd;

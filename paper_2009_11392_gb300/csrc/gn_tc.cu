@@ -450,15 +450,16 @@ __global__ void __launch_bounds__(NUM_THREADS, 1) tc_multigemm_kernel(const __gr
                 const uint8_t *sf_a[MT], *sf_b = nullptr;   // scale-factor images: K block 0, then a step per block
                 long long sf_astep = 0, sf_bstep = 0;
                 if (F8) {
-                    sf_astep = 512LL * (G.sfa_tr ? G.sfa_ld : 1);
-                    sf_bstep = 512LL * (G.sfb_tr ? G.sfb_ld : 1);
+                    const TcScales& f = p.sf[c.g];
+                    sf_astep = 512LL * (f.sfa_tr ? f.sfa_ld : 1);
+                    sf_bstep = 512LL * (f.sfb_tr ? f.sfb_ld : 1);
 #pragma unroll
                     for (int hh = 0; hh < MT; ++hh) {
-                        const long long rb = min(m0 / BM + hh, G.sfa_rows - 1);
-                        sf_a[hh] = G.sfa + 512 * (G.sfa_tr ? rb : rb * G.sfa_ld);
+                        const long long rb = min(m0 / BM + hh, f.sfa_rows - 1);
+                        sf_a[hh] = f.sfa + 512 * (f.sfa_tr ? rb : rb * f.sfa_ld);
                     }
-                    const long long rb = min(n0 / BM, G.sfb_rows - 1);   // bn = 128: one tile
-                    sf_b = G.sfb + 512 * (G.sfb_tr ? rb : rb * G.sfb_ld);
+                    const long long rb = min(n0 / BM, f.sfb_rows - 1);   // bn = 128: one tile
+                    sf_b = f.sfb + 512 * (f.sfb_tr ? rb : rb * f.sfb_ld);
                 }
                 int src = kr.kb0 / nk, kk = kr.kb0 - src * nk;   // source and K block inside its range
                 const CUtensorMap* ma = map_of<GROUPED>(p, G.map_base + G.a_map[src]);
@@ -827,8 +828,8 @@ int pick_mt(const TcGemm* g, int ngemm, int f8, int sm_count) {
 gn_status tc_launch(gn_handle h, TcParams* p) {
     const int MT = pick_mt(p->g, p->ngemm, p->f8, h->sm_count);
     for (int i = 0; i < p->ngemm; ++i) {
-        if (p->f8 && (p->g[i].a_mn || p->g[i].b_mn || p->g[i].bn != 128 || p->g[i].nsrc != 1 || !p->g[i].sfa ||
-                      !p->g[i].sfb || p->g[i].sfa_rows < 1 || p->g[i].sfb_rows < 1))
+        if (p->f8 && (i >= TC_MAX_F8_GEMMS || p->g[i].a_mn || p->g[i].b_mn || p->g[i].bn != 128 || p->g[i].nsrc != 1 ||
+                      !p->sf[i].sfa || !p->sf[i].sfb || p->sf[i].sfa_rows < 1 || p->sf[i].sfb_rows < 1))
             return GN_ERR_INVALID_ARG;
         GN_TRY(tc_prepare_gemm(&p->g[i], 0, MT, p->f8));
     }

@@ -58,3 +58,52 @@ def test_large_digits_of_one_sign(gn, H, K):
             num, den = float(got[i, j]).as_integer_ratio()
             err = abs(num * 2 ** 124 // den - exact[i, j])
             assert err * 2 ** 53 <= 3 * ((K + 1023) // 1024) * abs(exact[i, j])
+
+
+def entrywise(got, left, right, rows, cols):
+    """max |got - left right| / (|left| |right|) over sampled entries, in units of K 2^-53: at
+    most 1 for an FP64 sum in any order."""
+    a, b = (t.cpu().numpy().astype(np.longdouble) for t in (left[rows], right[:, cols]))
+    size = np.abs(a) @ np.abs(b)
+    err = np.abs(got[rows][:, cols].cpu().numpy() - a @ b)
+    assert np.all(err[size == 0] == 0)
+    return float((err[size > 0] / size[size > 0]).max()) / (left.shape[1] * 2.0 ** -53)
+
+
+def scales(kind, m, n, r, l, rn):
+    A, X, Y = rn(m, n), rn(n, r), rn(m, r + l)
+    if kind == "hidden column":    # the largest entries meet zeros
+        A[:, 3] = 1e20
+        A[7] *= 1e18
+        X[3] = 0.0
+        Y[7] = 0.0
+    elif kind == "selection":      # X and Y pick columns and rows
+        X.zero_()
+        Y.zero_()
+        X[torch.randperm(n, device="cuda")[:r], torch.arange(r, device="cuda")] = 1.0
+        Y[torch.randperm(m, device="cuda")[:r + l], torch.arange(r + l, device="cuda")] = -1.0
+        A *= torch.exp2(torch.randint(-80, 80, (m, n), device="cuda").double())
+    elif kind == "graded":         # 1e-30 .. 1 along the contractions, in opposite directions
+        d = torch.logspace(0, -30, n, dtype=torch.float64, device="cuda")
+        A *= d
+        X *= d.flip(0)[:, None]
+        Y *= torch.logspace(-30, 0, m, dtype=torch.float64, device="cuda")[:, None]
+    elif kind == "sparse":         # 2 % of both operands
+        A *= torch.rand_like(A) < 0.02
+        X *= torch.rand_like(X) < 0.02
+        Y *= torch.rand_like(Y) < 0.02
+    return A, X, Y
+
+
+# one pass and several, a last pass of one, fewer columns than a warp and one more than two
+@pytest.mark.parametrize("kind", ["gaussian", "hidden column", "selection", "graded", "sparse"])
+@pytest.mark.parametrize("m,n,r,l", [(700, 900, 40, 8), (2500, 1025, 17, 9), (1300, 5000, 65, 3)])
+def test_entries_keep_the_bound_of_an_fp64_sum(gn, H, kind, m, n, r, l):
+    g = torch.Generator(device="cuda").manual_seed(m)
+    rn = lambda a, b: torch.randn(a, b, generator=g, device="cuda", dtype=torch.float64)
+    A, X, Y = scales(kind, m, n, r, l, rn)
+    AX, YtA = sketch(gn, H, A, X, Y)
+    assert m * n * r > 1 << 24
+    at = lambda k: torch.arange(0, k, max(1, k // 40), device="cuda")
+    assert entrywise(AX, A, X, at(m), at(r)) <= 1.0
+    assert entrywise(YtA, Y.T, A, at(r + l), at(n)) <= 1.0

@@ -47,7 +47,7 @@ SIZES = [(64, 256), (3000, 200), (2000, 257), (8192, 300), (8193, 300), (8300, 1
 
 
 @pytest.mark.parametrize("kind,m,k,trans", [(kind, m, k, 0) for kind in ("graded", "kahan", "unit") for m, k in SIZES] +
-                         [(kind, 64, 256, 1) for kind in ("graded", "kahan")] + [("unit", m, k, 1) for m, k in SIZES])
+                         [(kind, m, k, 1) for kind in ("graded", "kahan", "unit") for m, k in SIZES])
 def test_solve_is_backward_stable(gn, H, kind, m, k, trans):
     g = torch.Generator(device="cuda").manual_seed(k + m)
     rn = lambda a, b: torch.randn(a, b, generator=g, device="cuda", dtype=torch.float64)
