@@ -651,16 +651,23 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
     }
     if (nout > digits) outs[nout - 1] = Out{nout - 1, 2 * digits, digits, 1};   // slice `digits` of both
     if (nout > TC_MAX_GEMMS || 2 * ns > TC_MAX_MAPS || digits > TC_MAX_SRC) return GN_ERR_UNSUPPORTED;
-    // launch order: lengths digits, digits - 1, ..., 1, which the boustrophedon order on
-    // (digits + 1) / 2 groups of CTAs pairs to equal loads (seven digits: 7; 6 + 1; 5 + 2; 4 + 3).
-    // Nine digits, 9, 8, 7, 4, 4, 4, 3, 2, 2, 1, 1, 1 on 5 groups: 4 + 4 + 1, 4 + 3 + 2, 7 + 2, 8 + 1, 9 + 1.
+    // Launch order: the longest first.  Lengths digits, digits - 1, ..., 1 are paired to equal loads
+    // by the boustrophedon order on (digits + 1) / 2 groups of CTAs (seven digits: 7; 6 + 1; 5 + 2;
+    // 4 + 3).  Nine digits' 9, 8, 7, 4, 4, 4, 3, 2, 2, 1, 1, 1 are when the tiles fill the SMs several
+    // times; with a CTA group per tile they go 4 + 4 + 1, 4 + 3 + 2, 7 + 2, 8 + 1, 9 + 1 (at most 10
+    // slice products per CTA; 11 in decreasing order).
+    std::stable_sort(outs, outs + nout, [](const Out& a, const Out& b) { return a.n > b.n; });
+    Out few[OZ_OUTS_F64];
     if (nout > digits) {
-        const int by[OZ_OUTS_F64] = {5, 4, 6, 7, 8, 0, 9, 1, 2, 3, 11, 10};
-        Out t[OZ_OUTS_F64];
-        for (int i = 0; i < nout; ++i) t[i] = outs[by[i]];
-        std::copy(t, t + nout, outs);
-    } else {
-        std::reverse(outs, outs + nout);
+        const int by[OZ_OUTS_F64] = {4, 4, 7, 8, 9, 1, 1, 2, 3, 4, 1, 2};   // lengths
+        bool used[OZ_OUTS_F64] = {};
+        for (int i = 0; i < nout; ++i)
+            for (int q = 0; q < nout; ++q)
+                if (!used[q] && outs[q].n == by[i]) {
+                    used[q] = true;
+                    few[i] = outs[q];
+                    break;
+                }
     }
     const long long as_stride = M * o.ldk, bs_stride = N * o.ldk, d_stride = M * o.ldd;
     // groups of at most OZ_PGRP passes: one slicing launch for all of them, the
@@ -695,8 +702,9 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                 GN_TRY(tc_make_map_bf16(&p.maps[s], o.as + s * as_stride, M, kc, o.ldk, 64, 128));
             for (int t = 0; t < ns; ++t)
                 GN_TRY(tc_make_map_bf16(&p.maps[ns + t], o.bs + t * bs_stride + j0 * o.ldk, nb, kc, o.ldk, 64, bn));
+            const bool spread = nout > digits && (digits + 1) / 2 * ((M + 127) / 128) * ((nb + bn - 1) / bn) * S <= h->sm_count;
             for (int gi = 0; gi < nout; ++gi) {
-                const Out& out = outs[gi];
+                const Out& out = spread ? few[gi] : outs[gi];
                 TcGemm& g = p.g[gi];
                 g.M = static_cast<int>(M);
                 g.N = static_cast<int>(nb);
