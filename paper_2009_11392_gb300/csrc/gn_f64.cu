@@ -355,22 +355,57 @@ gn_status dgemm_launch(gn_handle h, long long M, long long N, long long K, doubl
 // sliced product (40-60 us) and below 64 x 64 tiles at any size that leaves SMs idle.
 constexpr long long SG_MAX_MACS = 16LL << 20;
 
+// Columns per warp, K parts and K per part of the small kernel.
+struct SmallPlan {
+    int nc;
+    long long tiles, splits, kchunk;
+};
+SmallPlan small_plan(long long M, long long N, long long K, int sms) {
+    SmallPlan p;
+    // columns per warp: the widest that wastes nothing over the next narrower and keeps two CTAs per SM
+    // with K split as far as it goes (48 x 32 x 8000: 128 CTAs of one column per warp, 32 of four)
+    p.nc = 1;
+    const long long most = std::max<long long>(1, std::min<long long>(SG_MAX_SPLIT, K / SG_KC));
+    for (int c : {2, 4}) {
+        const long long w0 = (N + 4 * p.nc - 1) / (4 * p.nc) * p.nc, w1 = (N + 4 * c - 1) / (4 * c) * c;
+        if (w1 <= w0 && (M + SG_BM - 1) / SG_BM * ((N + 4 * c - 1) / (4 * c)) * most >= 2LL * sms) p.nc = c;
+    }
+    p.tiles = (M + SG_BM - 1) / SG_BM * ((N + 4 * p.nc - 1) / (4 * p.nc));
+    // K parts: enough CTAs for four per SM (one per sub-partition's worth of warps), at least 32 of K each
+    p.splits = std::max<long long>(1, std::min<long long>(SG_MAX_SPLIT, (4LL * sms + p.tiles - 1) / p.tiles));
+    p.splits = std::max<long long>(1, std::min(p.splits, K / SG_KC));
+    p.kchunk = ((K + p.splits - 1) / p.splits + SG_KC - 1) / SG_KC * SG_KC;
+    p.splits = (K + p.kchunk - 1) / p.kchunk;
+    return p;
+}
+
+// Microseconds of a product on the FP64 units, two multiply-adds per cycle and SM at ~1.93 GHz:
+// by the small kernel (a CTA's warps take nc instructions per element of K) and by the tiled one.
+double small_us(long long M, long long N, long long K, int sms) {
+    const SmallPlan p = small_plan(M, N, K, sms);
+    return 5.0 + std::max(1.0, static_cast<double>(p.tiles * p.splits) / sms) * std::min(K, p.kchunk) * p.nc * 64.0 / 1930.0;
+}
+double tiled_us(long long M, long long N, long long K, int sms) {
+    const long long bm = tile_m(M), bn = bm < GT ? 128 : GT, splits = choose_splits(M, N, K, sms);
+    const long long ctas = (M + bm - 1) / bm * ((N + bn - 1) / bn) * splits;
+    return 5.0 + static_cast<double>((ctas + sms - 1) / sms) * ((K + splits - 1) / splits) * (bm * bn / 2) / 1930.0;
+}
+// Whether dgemm takes the small kernel: small products, larger ones whose 64 x 64 tiles leave SMs
+// idle (the adjoint's three 256 x 256 x 384 products: 0.08 ms less), and skinny ones, whose tiles
+// are mostly padding (12 x 8 x 400000: 1.7 ms against 3.5; 100 x 10 x 30000: 0.13 against 0.51).
+bool takes_small(long long M, long long N, long long K, int sms) {
+    if (K < 1 || (M + SG_BM - 1) / SG_BM > 65535 || K > 0x7FFFFFFF - 2 * SG_KC) return false;
+    if (M * N * K <= SG_MAX_MACS) return true;
+    if (((M + GT - 1) / GT) * ((N + GT - 1) / GT) < sms && M * N * K <= 4 * SG_MAX_MACS) return true;
+    return small_us(M, N, K, sms) < 0.7 * tiled_us(M, N, K, sms);
+}
+
 gn_status dgemm_small(gn_handle h, long long M, long long N, long long K, double alpha, const double* A, long long lda,
                       int ta, const double* B, long long ldb, int tb, double beta, double* C, long long ldc) {
-    // columns per warp: the widest that wastes nothing over the next narrower and keeps a few tiles per SM
-    int nc = 1;
-    for (int c : {2, 4}) {
-        const long long w0 = (N + 4 * nc - 1) / (4 * nc) * nc, w1 = (N + 4 * c - 1) / (4 * c) * c;
-        if (w1 <= w0 && (M + SG_BM - 1) / SG_BM * ((N + 4 * c - 1) / (4 * c)) * std::max<long long>(1, K / 64) >= 2LL * h->sm_count)
-            nc = c;
-    }
-    const long long tiles = (M + SG_BM - 1) / SG_BM * ((N + 4 * nc - 1) / (4 * nc));
-    // K parts: enough CTAs for four per SM (one per sub-partition's worth of warps), at least 32 of K each
-    long long S = std::max<long long>(1, std::min<long long>(SG_MAX_SPLIT, (4LL * h->sm_count + tiles - 1) / tiles));
-    S = std::max<long long>(1, std::min(S, K / SG_KC));
-    const long long kchunk = ((K + S - 1) / S + SG_KC - 1) / SG_KC * SG_KC;
-    S = (K + kchunk - 1) / kchunk;
-    SmallGemm g{static_cast<int>(M), static_cast<int>(N), static_cast<int>(K), static_cast<int>(kchunk),
+    const SmallPlan p = small_plan(M, N, K, h->sm_count);
+    const int nc = p.nc;
+    const long long S = p.splits;
+    SmallGemm g{static_cast<int>(M), static_cast<int>(N), static_cast<int>(K), static_cast<int>(p.kchunk),
                 alpha, beta, A, B, lda, ldb, ldc, ta, tb, C};
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>((N + 4 * nc - 1) / (4 * nc)), static_cast<unsigned>((M + SG_BM - 1) / SG_BM),
@@ -1801,13 +1836,14 @@ bool small_gemm(long long M, long long N, long long K) {
     return K >= 1 && M * N * K <= SG_MAX_MACS && (M + SG_BM - 1) / SG_BM <= 65535;
 }
 
+double f64_units_us(long long M, long long N, long long K, int sm_count) {
+    return takes_small(M, N, K, sm_count) ? small_us(M, N, K, sm_count) : tiled_us(M, N, K, sm_count);
+}
+
 gn_status dgemm(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
                 long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                 long long ldc, double* ws, size_t ws_bytes) {
-    // (also larger ones whose 64 x 64 tiles leave SMs idle: the adjoint's three 256 x 256 x 384
-    // products: 0.08 ms less)
-    const bool few_tiles = K >= 1 && ((M + GT - 1) / GT) * ((N + GT - 1) / GT) < h->sm_count && M * N * K <= 4 * SG_MAX_MACS;
-    if (M > 0 && N > 0 && (small_gemm(M, N, K) || few_tiles))
+    if (M > 0 && N > 0 && takes_small(M, N, K, h->sm_count))
         return dgemm_small(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc);
     return dgemm_impl<double, double>(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, ws, ws_bytes);
 }

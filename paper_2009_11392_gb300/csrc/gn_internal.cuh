@@ -245,11 +245,13 @@ gn_status oz_dgemm(gn_handle h, long long M, long long N, long long K, double al
                    long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                    long long ldc, void* ws, size_t ws_bytes, int digits = 7);
 
+// Whether dgemm takes its kernel for products of few multiply-adds whatever their shape (no
+// workspace), and about how long dgemm takes.
+bool small_gemm(long long M, long long N, long long K);
+double f64_units_us(long long M, long long N, long long K, int sm_count);
 // dgemm for FP64 operands through oz_dgemm with nine digits (63 bits below each
 // row's largest entry) where the product is large enough, ws holds
 // dgemm_fast_ws_bytes and gn_set_fp64_tc is on; dgemm otherwise.
-// Whether dgemm takes its kernel for products of few multiply-adds (no workspace).
-bool small_gemm(long long M, long long N, long long K);
 size_t dgemm_fast_ws_bytes(long long M, long long N, long long K, int sm_count);
 gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double alpha, const double* A,
                      long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,

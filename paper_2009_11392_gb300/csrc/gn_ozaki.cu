@@ -766,17 +766,31 @@ namespace {
 // Blocks of C per digit-sliced product: the scratch (the slices of up to 4096 of K)
 // stays near 2 GB however large the matrices are.
 constexpr long long OZ_MBLK = 8192, OZ_NBLK = 16384;
-// Digit slicing takes ~40 us of launches whatever the size; the FP64 units take
-// MNK / 485e9 s when the product spreads over the SMs (dgemm's small kernel), so
-// they keep products of up to 16 M multiply-adds.  Both products of a sketch at
-// m, n, r = 1000, 500, 20: 115 us in slices, 73 on the units; 4096, 2048, 100: 0.44 ms in slices and 5.25
-// on the units; 20000, 10000, 500: 28.0 and 428.5 ms.
-bool oz_f64_pays(long long M, long long N, long long K) { return M >= 1 && N >= 1 && K >= 1 && !small_gemm(M, N, K); }
+// Microseconds of a nine-digit product: per block of C and group of K, three launches, the longest
+// chain of slice products of one tile (10 per 64 of K, 0.28 us for 64 columns, 0.49 for 256) or
+// all of them over the SMs, the slices and the outputs through memory.
+double oz_us(long long M, long long N, long long K, int sms) {
+    const double m = static_cast<double>(std::min(M, OZ_MBLK)), n = static_cast<double>(std::min(N, OZ_NBLK));
+    const long long kc = std::min<long long>(K, OZ_PGRP * OZ_KPASS), parts = (kc + OZ_KPASS - 1) / OZ_KPASS;
+    const double bn = std::min(256.0, n), c = 0.21 + 0.0011 * bn, kb = static_cast<double>(std::min<long long>(16, (kc + 63) / 64));
+    const double tiles = static_cast<double>((std::min(M, OZ_MBLK) + 127) / 128) * std::max(1.0, n / bn) * parts;
+    const double one = 15.0 + kb * c * std::max(10.0, 46.0 * tiles / sms) + (m + n) * kc * 28.0 / 4e6 + m * n * parts * 100.0 / 4e6;
+    return one * std::max(1.0, M / m) * std::max(1.0, N / n) * std::max(1.0, static_cast<double>(K) / kc);
+}
+// Products of up to 16 M multiply-adds stay on the FP64 units (three launches and a tile's chain
+// take ~40 us whatever the size), and larger ones that the estimates put at half the time there: few rows and columns
+// over a long K, or few of them against many over a short one, where a tile of 128 rows and its
+// slices are mostly padding.  Both products of a sketch at m, n, r, l = 1000, 500, 20, 10: 115 us
+// in slices, 73 on the units; 4096, 2048, 100, 50: 0.44 ms and 5.25; 20000, 10000, 500, 250: 22.8
+// and 428.5; 100000, 40, 10, 5: 2.12 and 0.78; 40, 100000, 10, 5: 2.37 and 1.57.
+bool oz_f64_pays(long long M, long long N, long long K, int sms) {
+    return M >= 1 && N >= 1 && K >= 1 && !small_gemm(M, N, K) && 0.5 * oz_us(M, N, K, sms) < f64_units_us(M, N, K, sms);
+}
 }  // namespace
 
 size_t dgemm_fast_ws_bytes(long long M, long long N, long long K, int sm_count) {
     size_t b = dgemm_ws_bytes(M, N, K, sm_count);
-    if (!oz_f64_pays(M, N, K)) return b;
+    if (!oz_f64_pays(M, N, K, sm_count)) return b;
     for (long long mm : {std::min(M, OZ_MBLK), M % OZ_MBLK})
         for (long long nn : {std::min(N, OZ_NBLK), N % OZ_NBLK})
             if (mm > 0 && nn > 0) b = std::max(b, oz_ws_bytes(mm, nn, K, 0, OZ_DIGITS_F64) + 256);
@@ -787,7 +801,7 @@ gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double 
                      long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                      long long ldc, double* ws, size_t ws_bytes) {
     const size_t need = dgemm_fast_ws_bytes(M, N, K, h->sm_count);
-    if (!h->fp64_tc || !ws || ws_bytes < need || !oz_f64_pays(M, N, K))
+    if (!h->fp64_tc || !ws || ws_bytes < need || !oz_f64_pays(M, N, K, h->sm_count))
         return dgemm(h, M, N, K, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, ws, ws_bytes);
     const size_t pad = (256 - (reinterpret_cast<uintptr_t>(ws) & 255)) & 255;
     char* base = reinterpret_cast<char*>(ws) + pad;

@@ -107,3 +107,19 @@ def test_entries_keep_the_bound_of_an_fp64_sum(gn, H, kind, m, n, r, l):
     at = lambda k: torch.arange(0, k, max(1, k // 40), device="cuda")
     assert entrywise(AX, A, X, at(m), at(r)) <= 1.0
     assert entrywise(YtA, Y.T, A, at(r + l), at(n)) <= 1.0
+
+
+# few rows and columns over a long contraction, for AX and for Y^T A
+@pytest.mark.parametrize("m,n,r,l", [(40, 100000, 10, 5), (100, 30000, 10, 5), (60, 16000, 33, 1), (50000, 40, 12, 6)])
+def test_skinny_products_stay_on_the_fp64_units(gn, H, m, n, r, l):
+    """A tile of 128 rows would be mostly padding and its slices as long as the operands."""
+    g = torch.Generator(device="cuda").manual_seed(m)
+    rn = lambda a, b: torch.randn(a, b, generator=g, device="cuda", dtype=torch.float64)
+    A, X, Y = rn(m, n), rn(n, r), rn(m, r + l)
+    before = gn.kernel_launches()
+    AX, YtA = sketch(gn, H, A, X, Y)
+    # one launch for the skinny product, three per block of 8192 rows or 16384 columns for the other
+    assert gn.kernel_launches() - before <= 1 + 3 * (max(m, n) // 8192 + 1)
+    at = lambda k: torch.arange(0, k, max(1, k // 12), device="cuda")
+    assert entrywise(AX, A, X, at(m), at(r)) <= 1.0
+    assert entrywise(YtA, Y.T, A, at(r + l), at(n)) <= 1.0
