@@ -143,6 +143,11 @@ size_t factors_oz_ws(long long m, long long r) {
     return std::max(oz_ws_bytes(m, 128, r, 0), oz_ws_bytes(m, r, r, 1));
 }
 
+// ... and what lets the solve take all of its rows (up to 32768) together.
+size_t factors_oz_full(long long m, long long r) {
+    return std::max(factors_oz_ws(m, r), align256(trsm_oz_ws_bytes(m, r, OZ_DIGITS_SOLVE)));
+}
+
 // Factors: the FP64 solves' scratch, plus (FP32 Y^T A) the BF16 slices of Y^T A
 // and Q_1 and the FP32 product G.
 size_t factors_ws(long long m, long long n, long long r, long long l, int mixed, int sms) {
@@ -818,7 +823,7 @@ gn_status gn_workspace_size(int64_t m, int64_t n, int64_t r, int64_t l, int32_t 
                             sketch_split(m, n, r, r + l, op_dtype == GN_BF16X2 ? 2 : 1, op_dtype == GN_E4M3, sms).bytes());
     if (!mixed) b = std::max(b, f64_fast_ws(m, n, r, l, sms));
     // (the factors' own check asks for less: the solve then takes fewer rows at a time)
-    if (mixed) b = std::max(b, factors_ws(m, n, r, l, 1, sms) + trsm_oz_ws_bytes(m, r, OZ_DIGITS_SOLVE));
+    if (mixed) b = std::max(b, factors_ws(m, n, r, l, 1, sms) - factors_oz_ws(m, r) + factors_oz_full(m, r));
     *bytes = b;
     return GN_OK;
 }
@@ -1078,9 +1083,7 @@ gn_status gn_factors(gn_handle h, const gn_mat* AX, const gn_mat* YtA, const gn_
     void* oz = nullptr;
     // at least what the check above asks for, and what ws holds beyond it up to the whole solve
     const size_t oz_spare = ws_bytes - factors_ws(m, n, r, l, mixed, h->sm_count);
-    const size_t oz_bytes = oz_on ? (std::max(factors_oz_ws(m, r), std::min(factors_oz_ws(m, r) + oz_spare,
-                                                                            trsm_oz_ws_bytes(m, r, OZ_DIGITS_SOLVE))) &
-                                     ~static_cast<size_t>(255)) : 0;
+    const size_t oz_bytes = oz_on ? std::min(factors_oz_ws(m, r) + oz_spare, factors_oz_full(m, r)) & ~static_cast<size_t>(255) : 0;
     if (tc_g) {
         for (int i = 0; i < 3; ++i) sl[i] = cv.take<__nv_bfloat16>(rl * lds);
         for (int i = 0; i < 3; ++i) ql[i] = cv.take<__nv_bfloat16>(rl * ldq);

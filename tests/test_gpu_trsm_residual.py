@@ -125,3 +125,51 @@ def test_short_fp32_sketches_stay_on_the_fp64_units(gn, H, m):
     a, q = AX.cpu().numpy().astype(np.longdouble), core.Q2[:, :k].cpu().numpy().astype(np.longdouble)
     err = np.abs(F[:, :k].cpu().numpy() - a[:, 1:] @ q[1:])
     assert np.all(err <= (r + 4) * 2.0 ** -53 * (np.abs(a[:, 1:]) @ np.abs(q[1:])))   # r u |AX||Q_2|
+
+
+# base blocks of 128 and of 32 columns; FP32 sketches (eight digits) and FP64 ones (nine)
+@pytest.mark.parametrize("m,r", [(3000, 256), (9000, 700), (40000, 300)])
+@pytest.mark.parametrize("f64", [False, True])
+def test_every_accepted_workspace_gives_the_same_factors(gn, H, m, r, f64):
+    """From the smallest workspace that gn_factors takes up to gn_workspace_size: fewer rows at
+    a time, or the FP64 units, with the residual of a substitution each time."""
+    n, l = 60, 8
+    g = torch.Generator(device="cuda").manual_seed(r)
+    rn = lambda a, b: torch.randn(a, b, generator=g, device="cuda", dtype=torch.float64)
+    core = gn.Core.empty(r, l, "cuda")
+    core.R.copy_(torch.triu(rn(r, r), 1) / r ** 0.5 + torch.eye(r, dtype=torch.float64, device="cuda"))
+    core.Q.copy_(rn(r + l, r))
+    core.k = r
+    dt = torch.float64 if f64 else torch.float32
+    AX, YtA = rn(m, r).to(dt), rn(r + l, n).to(dt)
+    full = H.workspace_bytes(m, 2 * r, r, l, gn.F64 if f64 else gn.BF16)
+    buf = torch.empty(full, dtype=torch.uint8, device="cuda")
+    rows = torch.linspace(0, m - 1, 16, device="cuda").long()
+
+    def run(nbytes):
+        F = torch.empty(m, r, dtype=torch.float64, device="cuda")
+        G = torch.empty(r, n, dtype=torch.float64, device="cuda")
+        H.factors(AX, YtA, core, F, G, buf[:nbytes])
+        assert H.sync_status() == 0
+        return F
+    lo, need = 0, full   # run(lo) is refused, run(need) is not
+    while need - lo > 256:
+        mid = (lo + need) // 2
+        try:
+            run(mid)
+            need = mid
+        except gn.GNError as e:
+            assert e.status == 4
+            lo = mid
+    assert need < full
+    # eight digits: a window of 2^-56 below the largest entries of a row and a column, K <= 512
+    tol = (r + 4) * 2.0 ** -53 + (0 if f64 else 512 ** 0.5 * 2.0 ** -52)
+    for nbytes in (need, need + (full - need) // 5, (need + full) // 2, full):
+        assert backward(run(nbytes), core.R, AX, rows) <= tol
+
+
+def test_workspace_size_asks_for_what_the_factors_take(gn, H):
+    """At a shape whose largest call is the factors', the smallest size that solves all rows
+    together is the one asked for: it was 0.7 GB more at 32768 x 16384, r = 1000."""
+    m, n, r, l = 32768, 16384, 1000, 500
+    assert H.workspace_bytes(m, n, r, l, gn.BF16) <= 1.3e9
