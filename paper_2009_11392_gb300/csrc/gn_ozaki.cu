@@ -24,12 +24,16 @@
 // worst-case rounding error.  FP32 operands take 7 digits too: the digits cover
 // a window below the row's largest entry, not each entry's own 24 bits.
 // FP64 operands of the FP64 path take nine digits (63 bits below each row's
-// largest entry, orders 0..8): 45 slice products instead of 28.  Measured against
+// largest entry, orders 0..8): 45 slice products instead of 28, and one for the
+// entries' sizes.  Measured against
 // extended precision (relative Frobenius error of a Gaussian product, K = 500 /
 // 2048): 4.8e-17 / 6.7e-17, the FP64 units 3.0e-16 / 9.2e-16; with low-rank, 1 %
 // sparse and graded (1e8) matrices the slices stay at 3e-17..8e-17 and the units
-// at 8e-17..1.4e-15.  The error scales with max|a_i.| max|b_.j|, not with
-// sum |a_ik| |b_kj|.
+// at 8e-17..1.4e-15.  The digits' error scales with max|a_i.| max|b_.j|; entries whose
+// sum |a_ik| |b_kj| is small beside that are formed with FP64 FMA (OZ_SMALL), so that
+// each entry keeps the bound of an FP64 sum.  FP64 sketch 8000 x 4000, r = 200, us:
+// Gaussian operands 2240, X and Y selecting columns and rows 4050, 2 % dense operands
+// 33400 (nearly every entry); the FP64 units 40320 each.
 #include "gn_internal.cuh"
 
 #include <cooperative_groups.h>
@@ -70,10 +74,13 @@ size_t al256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 // orders and K parts stay within 64 MB (short, wide products in one launch); 160 MB
 // with more than seven digits: their wide products (Y^T A of an FP64 sketch) then have
 // enough 256-row tiles, which need 62 B per cycle and SM from L2 where 128-row ones
-// need 94 of the ~60 there are (20000 x 10000, r = 500: 28.4 -> 26.3 ms).
+// need 94 of the ~60 there are.  Measured at one shape only, 20000 x 10000, r = 500: 28.4
+// -> 26.3 ms with nine outputs; with twelve, panels a third wider (213 MB) cost 1.2 ms.
+// Whole tiles of 256 columns there: the last tile of a panel costs as much at 64 columns
+// (sketch at 32768 x 16384, r = 1000: 124 -> 109 ms).
 long long oz_npanel(long long M, long long N, long long parts, int orders) {
     long long np = ((orders > 7 ? 160LL : 64LL) << 20) / (4LL * orders * std::max<long long>(M, 1) * std::max<long long>(parts, 1));
-    np = std::max<long long>(np, OZ_NPANEL) / 16 * 16;
+    np = std::max<long long>(np, OZ_NPANEL) / (orders > 7 ? OZ_NPANEL : 16) * (orders > 7 ? OZ_NPANEL : 16);
     return std::min<long long>(N, np);
 }
 long long r8(long long x) { return (x + 7) / 8 * 8; }
@@ -778,11 +785,12 @@ double oz_us(long long M, long long N, long long K, int sms) {
     return one * std::max(1.0, M / m) * std::max(1.0, N / n) * std::max(1.0, static_cast<double>(K) / kc);
 }
 // Products of up to 16 M multiply-adds stay on the FP64 units (three launches and a tile's chain
-// take ~40 us whatever the size), and larger ones that the estimates put at half the time there: few rows and columns
-// over a long K, or few of them against many over a short one, where a tile of 128 rows and its
-// slices are mostly padding.  Both products of a sketch at m, n, r, l = 1000, 500, 20, 10: 115 us
-// in slices, 73 on the units; 4096, 2048, 100, 50: 0.44 ms and 5.25; 20000, 10000, 500, 250: 22.8
-// and 428.5; 100000, 40, 10, 5: 2.12 and 0.78; 40, 100000, 10, 5: 2.37 and 1.57.
+// take ~40 us whatever the size), and larger ones that the estimates put at half the time
+// there: few rows and columns over a long K, or few of them against many over a short one,
+// where a tile of 128 rows and its slices are mostly padding.  Both products of a sketch at
+// m, n, r, l = 1000, 500, 20, 10: 115 us in slices, 73 on the units; 4096, 2048, 100, 50: 0.45 ms
+// and 5.25; 20000, 10000, 500, 250: 23.0 and 428.5; 100000, 40, 10, 5: 2.12 and 0.78; 40, 100000,
+// 10, 5: 2.37 and 1.57.
 bool oz_f64_pays(long long M, long long N, long long K, int sms) {
     return M >= 1 && N >= 1 && K >= 1 && !small_gemm(M, N, K) && 0.5 * oz_us(M, N, K, sms) < f64_units_us(M, N, K, sms);
 }
