@@ -181,20 +181,24 @@ gn_status gn_set_fp64_accum(gn_handle h, int64_t part_k);
  * factorization runs in 256-column blocks and each block's reflectors update
  * the columns to its right as two products after U = V T; below that, the columns beyond
  * the next two panels of the look-ahead) and the formation of the thin Q; in
- * gn_factors / gn_approx, the products of the blocked triangular solve
+ * gn_factors / gn_approx with AX of 1024 rows or more, the products of the triangular solve
  * F R = AX (eq. 5.1; 8 digits per operand) and, after a truncation, AX Q_2; in gn_apply, the products
  * with AX and Y^T A.  1 (default): on the BF16 tensor cores by exact digit
  * slicing (gn_dgemm_tc; FP64-level accuracy, about 1e-13 of |A||B| per
- * element); 0: on the FP64 units.  The panels, the small diagonal-block solves
- * and the detector stay in FP64 either way.
+ * element); 0: on the FP64 units.  The panels, the substitutions inside the
+ * solve's blocks of 32 or 128 columns and the detector stay in FP64 either way.
  * For GN_F64 operands the switch covers gn_sketch (and the calls built on it),
- * the core product C, the factors, gn_apply and gn_hmt's two products: 1
- * (default) forms those of more than 2^24 multiply-adds from nine digits per operand (63 bits below the largest entry of each
- * row of the left and column of the right operand: the error per element is
- * about 2^-60 sqrt(K) max_k |a_ik| max_k |b_kj|, below the rounding error of an
- * FP64 sum), infinities and NaN as the FP64 units give them; a workspace too
- * small for the slices (gn_workspace_size includes them) selects the FP64 units
- * for that product. */
+ * the core product C, the factors, gn_hmt's two products and gn_apply (there also
+ * the core-sized products and solves of GN_F32 sketches): 1 (default) forms
+ * products of more than 2^24 multiply-adds, where that is faster, from nine digits
+ * per operand (63 bits below the largest entry of each row of the left and column
+ * of the right operand).  Every entry keeps the bound of an FP64 sum, about
+ * K 2^-53 sum_k |a_ik| |b_kj|: where that sum is small beside max_k |a_ik|
+ * max_k |b_kj| (sparse or graded operands, selections), the entry is formed with
+ * FP64 FMA instead, as are rows and columns with infinities or NaN, which so come
+ * out as on the FP64 units.  Operands for which that is most entries take about
+ * the FP64 units' time.  0, or a workspace too small for the slices
+ * (gn_workspace_size includes them), selects the FP64 units for the product. */
 gn_status gn_set_fp64_tc(gn_handle h, int32_t on);
 
 /* C = alpha op(A) op(B) + beta C, FP64 (A may be FP32), computed on the BF16

@@ -197,8 +197,8 @@ __global__ void reduce_sum_kernel(const double* __restrict__ part, long long n, 
 // split over a cluster whose partial sums are added in rank order through
 // distributed shared memory (one launch, a fixed order of additions).
 // 1000 x 20 x 500: 94 + 5 us as 64 x 64 tiles with split K and a reduction
-// launch, 28 us here (10 M multiply-adds: 21 us at the units' rate); 30 x 500 x
-// 1000: 95 + 6 and 43 us (31); both sketch products at 64 x 64, r = 8: 108 and 14.
+// launch, 25 us here (10 M multiply-adds: 21 us at the units' rate); 30 x 500 x
+// 1000: 95 + 6 and 41 us (31); both sketch products at 64 x 64, r = 8: 108 and 9.
 // --------------------------------------------------------------------------
 constexpr int SG_THREADS = 128;
 constexpr int SG_BM = 32;
@@ -363,7 +363,7 @@ struct SmallPlan {
 SmallPlan small_plan(long long M, long long N, long long K, int sms) {
     SmallPlan p;
     // columns per warp: the widest that wastes nothing over the next narrower and keeps two CTAs per SM
-    // with K split as far as it goes (48 x 32 x 8000: 128 CTAs of one column per warp, 32 of four)
+    // with K split as far as it goes (48 x 32 x 8000: 128 CTAs of one column per warp, 79 us; 32 CTAs of four, 172)
     p.nc = 1;
     const long long most = std::max<long long>(1, std::min<long long>(SG_MAX_SPLIT, K / SG_KC));
     for (int c : {2, 4}) {
@@ -380,7 +380,8 @@ SmallPlan small_plan(long long M, long long N, long long K, int sms) {
 }
 
 // Microseconds of a product on the FP64 units, two multiply-adds per cycle and SM at ~1.93 GHz:
-// by the small kernel (a CTA's warps take nc instructions per element of K) and by the tiled one.
+// by the small kernel (a CTA's warps take nc instructions of 64 cycles per element of K; where an SM
+// has one CTA the chain takes up to 104) and by the tiled one.
 double small_us(long long M, long long N, long long K, int sms) {
     const SmallPlan p = small_plan(M, N, K, sms);
     return 5.0 + std::max(1.0, static_cast<double>(p.tiles * p.splits) / sms) * std::min(K, p.kchunk) * p.nc * 64.0 / 1930.0;
@@ -392,7 +393,7 @@ double tiled_us(long long M, long long N, long long K, int sms) {
 }
 // Whether dgemm takes the small kernel: small products, larger ones whose 64 x 64 tiles leave SMs
 // idle (the adjoint's three 256 x 256 x 384 products: 0.08 ms less), and skinny ones, whose tiles
-// are mostly padding (12 x 8 x 400000: 1.7 ms against 3.5; 100 x 10 x 30000: 0.13 against 0.51).
+// are mostly padding (12 x 8 x 400000: 2.7 ms against 3.5; 100 x 10 x 30000: 0.21 against 0.51).
 bool takes_small(long long M, long long N, long long K, int sms) {
     if (K < 1 || (M + SG_BM - 1) / SG_BM > 65535 || K > 0x7FFFFFFF - 2 * SG_KC) return false;
     if (M * N * K <= SG_MAX_MACS) return true;

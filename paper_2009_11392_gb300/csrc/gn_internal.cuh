@@ -257,7 +257,7 @@ gn_status dgemm_fast(gn_handle h, long long M, long long N, long long K, double 
                      long long lda, int ta, const double* B, long long ldb, int tb, double beta, double* C,
                      long long ldc, double* ws, size_t ws_bytes);
 
-// Core diagnostics (one CTA): out3[0] = est ||R^{-1}||_2 (if want_estimate),
+// Core diagnostics (one CTA up to 32 columns, two clusters up to 4096 with X, one CTA otherwise): out3[0] = est ||R^{-1}||_2 (if want_estimate),
 // out3[1] = est ||R||_2 (if eps_relative), out3[2] = the absolute threshold
 // used (eps, or eps * est ||R||_2); *k_out = first i with |R_ii| <= threshold.
 // ws: 2 r doubles.  X (r min(r, 128) doubles, or null): scratch of the version on
