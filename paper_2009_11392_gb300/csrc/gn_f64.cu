@@ -2908,7 +2908,15 @@ gn_status sum3_f32_to_f64(gn_handle h, const float* a, const float* b, const flo
 gn_status quantize_bf16(gn_handle h, const void* src, int src_f64, long long rows, long long cols,
                         long long lds, __nv_bfloat16* hi, __nv_bfloat16* lo, long long ldd) {
     if (rows * cols == 0) return GN_OK;
-    if (rows > 0x7FFFFFFF || cols > 0x7FFFFFFF - 256) return GN_ERR_SHAPE;
+    constexpr long long PART = 1LL << 30;   // (the kernel counts rows and columns in 32 bits)
+    if (rows > PART || cols > PART) {
+        for (long long i0 = 0; i0 < rows; i0 += PART)
+            for (long long j0 = 0; j0 < cols; j0 += PART)
+                GN_TRY(quantize_bf16(h, static_cast<const char*>(src) + (i0 * lds + j0) * (src_f64 ? 8 : 4), src_f64,
+                                     std::min(PART, rows - i0), std::min(PART, cols - j0), lds, hi + i0 * ldd + j0,
+                                     lo ? lo + i0 * ldd + j0 : nullptr, ldd));
+        return GN_OK;
+    }
     const int r = static_cast<int>(rows), c = static_cast<int>(cols);
     const long long tasks = rows * ((cols + 255) / 256);
     const unsigned blocks = static_cast<unsigned>(std::min<long long>((tasks + 7) / 8, 64LL * h->sm_count));
